@@ -107,6 +107,7 @@ constexpr double kPolarTheta = 0.2;
 constexpr float kPolarY = 0.019933422f;  // 1 - cos(kPolarTheta): polar iff y < kPolarY
 constexpr int kChunk = 8;    // l-chunk of the checkpointed FP32 adjoint (even)
 constexpr int kChunkDf = 4;  // l-chunk of the checkpointed double-float adjoint (even)
+constexpr int kFxChunk = 16;  // l-chunk of the checkpointed fixed-point adjoint
 
 inline __host__ __device__ int64_t lm_off(int L, int m) {
   return (int64_t)m * (L + 1) - (int64_t)m * (m - 1) / 2;
@@ -170,25 +171,28 @@ struct Grid {
 
   // Legendre recurrence tables (device), index lm(m, l)
   DevMem A64, A32;        // A_lm of the rescaled recurrence mu_l = A_l x mu_{l-1} - mu_{l-2}
-  DevMem A2f;             // A_lm as a double-float pair (float2 hi, lo) for the FP32X2 kernels
   DevMem BRS32;           // {B, R, S}_lm (FP32) of the difference form used near the poles
   DevMem c64;             // lambda_lm = c_lm mu_lm
   DevMem ls;              // int [L+1][npair] first l (same parity as m) that is injected
   DevMem st64, st32;      // {mu_ls, mu_ls+1} [L+1][npair]
+  DevMem lsx, stx;        // the same for the fixed-point stages (|mu| > 2^-64, values FP64)
+  DevMem xfx;             // uint64 cos(theta) 2^63 of the north ring [npair] (fixed-point stages)
+  DevMem mumax;           // unsigned [L+1]: high word of the largest |mu_l| of each m (FP64 bits)
   DevMem ck32;            // FP32 {mu_l0, mu_l0+1} at every chunk start l0 = m + kChunk c
   DevMem ck_base;         // int64 [L+1]: offset of m's block [pair][chunk] in ck32
   DevMem ls_tmin;         // int [L+1][ceil(npair / kTileMinPT)]: smallest ls of each tile of pairs
-  // warp tasks of the checkpointed adjoints: int2 {m, first chunk} per 32 consecutive
-  // chunks of one m, m ascending (FP32 chunking; the double-float list is built with ck64)
+  // warp tasks of the checkpointed FP32 adjoint: int2 {m, first chunk} per 32 consecutive
+  // chunks of one m, m ascending
   DevMem wt32;
   int nwt32 = 0;
-  mutable DevMem wtdf;
+  // tables of the double-float kernels, built on their first use: A_lm and y as double-float
+  // pairs (float2), {mu_l0, mu_l0+1} (float4) every kChunkDf, its offsets, and the warp tasks
+  mutable DevMem A2f, y2f, ck64, ck64_base, wtdf;
   mutable int nwtdf = 0;
-  mutable DevMem ck64;    // double-float {mu_l0, mu_l0+1} (float4) every kChunkDf; built on first use
-  mutable DevMem ck64_base;  // int64 [L+1]: offset of m's block [pair][chunk] in ck64
-  mutable DevMem y2f;     // y as a double-float pair (float2), built with ck64
   mutable std::mutex ck64_mu;
   std::vector<double> fmm_h;  // sqrt((2m+1)/(2m)) (host, for rebuilding seeds)
+  DevMem ckx;             // FP64 {mu_l0, mu_l0+1} at every l0 = m + kFxChunk c (zero before the start)
+  DevMem ckx_base;        // int64 [L+1]: offset of m's block [pair][chunk] in ckx
 
   // autotuner decisions for launches on this grid (legendre.cu), by kernel / precision / maps
   struct Tuned {
@@ -219,29 +223,26 @@ inline Grid* as_grid(const void* h) {
 // ---- launchers (legendre.cu) ----
 // alm: [nmaps][nlm] complex coefficients multiplied by c_lm; F: [nmaps][nring][L+1]
 int legendre_synth(const Grid& g, int prec, int nmaps, const void* alm, void* F, cudaStream_t s);
-// ring spectra -> out[nmaps][nlm] complex FP64 (final coefficients).  FP64 reads F (with
-// per-CTA partial sums in part); the other precisions read the eo layout, which the forward
-// ring FFT wrote into part.
-int legendre_adjoint(const Grid& g, int prec, int nmaps, const void* F, void* part, size_t part_bytes,
-                     double* out, cudaStream_t s);
+// ring spectra -> out[nmaps][nlm] complex FP64 (final coefficients), from the eo layout, which
+// the forward ring FFT wrote into part.
+int legendre_adjoint(const Grid& g, int prec, int nmaps, void* part, size_t part_bytes, double* out,
+                     cudaStream_t s);
 size_t legendre_adjoint_part_bytes(const Grid& g, int prec, int nmaps);
 
 // ---- launchers (ringfft.cu) ----
 // Layout of the adjoint Legendre input ("eo") that the forward ring FFTs write for the
-// checkpointed adjoints (every precision but FP64): maps in chunks of eo_maps(prec) (the
-// adjoint's maps per launch); chunk c starts at scalar c * eo_maps * (L+1) * npair * 4 and,
+// adjoints: maps in chunks of eo_maps(prec) (the adjoint's maps per launch); chunk c starts at
+// scalar c * eo_maps * (L+1) * npair * 4 and,
 // for its NMc maps, holds eo[(m * npair + p) * 4 NMc + q]: q < 2 NMc the even-l parts
 // (north + south ring spectra, re / im per map), q >= 2 NMc the odd-l parts (north - south).
-// Scalars are float (FP32 modes) or double-float pairs (FP32X2).
+// Scalars are double (FP64), float (FP32 modes) or double-float pairs (FP32X2).
 inline int eo_maps(int prec) { return prec == CMBWS_FP32X2 ? 3 : 4; }
 // F (ring spectra) -> pixel maps map[nmaps][npix] (FP64 out)
 int ringfft_synth(const Grid& g, int prec, int nmaps, const void* F, double* map, cudaStream_t s);
-// map[nmaps][npix] (FP64 in) -> ring spectra: F (FP64) or the adjoint input eo (other
-// precisions); weighted: multiply by quadrature weights
-int ringfft_analysis(const Grid& g, int prec, int nmaps, const double* map, int weighted, void* F,
-                     void* eo, cudaStream_t s);
-// F -> pixels -> * pix[map] -> ring spectra, written to F in place (FP64) or to eo (other
-// precisions).  pix: [nmaps] device pointers (prec type) of npix.
+// map[nmaps][npix] (FP64 in) -> adjoint input eo; weighted: multiply by quadrature weights
+int ringfft_analysis(const Grid& g, int prec, int nmaps, const double* map, int weighted, void* eo,
+                     cudaStream_t s);
+// F -> pixels -> * pix[map] -> adjoint input eo.  pix: [nmaps] device pointers (prec type) of npix.
 int ringfft_fused(const Grid& g, int prec, int nmaps, void* F, const void* const* pix, void* eo,
                   cudaStream_t s);
 int ringfft_smem_ok(const Grid& g, int prec);
@@ -251,7 +252,7 @@ std::vector<int2> adjoint_warp_tasks(int L, int chunk);
 
 // ---- grid setup (setup.cu) ----
 int grid_build_tables(Grid& g);
-// build the double-float chunk checkpoints of the FP32X2 adjoint if not yet built
+// build the double-float tables if not yet built
 int grid_ensure_ck64(const Grid& g);
 
 // ---- pack / unpack (setup.cu) ----
@@ -273,6 +274,14 @@ inline bool valid_prec(int prec) {
 
 // ---- double-float Legendre stage (legendre_df.cu) ----
 int legendre_synth_df(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s);
+// double-float adjoint from chunk checkpoints: eo (double-float adjoint input of nm <= 3
+// maps) -> out (FP64 coefficients)
+int legendre_adj_df_ck(const Grid& g, int nm, const void* eo, double* out, cudaStream_t s);
+// ---- FP64 Legendre stage in fixed point (legendre_fx.cu) ----
+int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s);
+// eo: ring parts (double), ee: int [nmaps][L+1] workspace
+int legendre_adjoint_fx(const Grid& g, int nmaps, const void* eo, int* ee, double* out, cudaStream_t s);
+int fx_status_take(bool* timed_out);  // as tc_status_take, for these kernels
 // ---- tensor-core Legendre synthesis (legendre_tc.cu), prec TF32 / 3XTF32 / BF16 / BF16X3 ----
 int legendre_synth_tc(const Grid& g, int prec, int nmaps, const void* alm, void* F, cudaStream_t s);
 // adjoint synthesis on the tensor cores from the FP32 adjoint input (eo layout), prec BF16 / BF16X3
@@ -281,9 +290,6 @@ int legendre_adjoint_tc(const Grid& g, int prec, int nmaps, const float* eo, dou
 // reads and clears the device-side status of the tensor-core kernels of the current device
 // (synchronous): *timed_out is true if a bounded mbarrier wait ran out since the last read
 int tc_status_take(bool* timed_out);
-// double-float adjoint from chunk checkpoints: eo (double-float adjoint input of nm <= 3
-// maps) -> out (FP64 coefficients)
-int legendre_adj_df_ck(const Grid& g, int nm, const void* eo, double* out, cudaStream_t s);
 
 // Raise a kernel's dynamic shared-memory limit to at least `bytes` on the current device.
 // The limit only ever grows, so concurrent launches with different sizes (several host

@@ -1,0 +1,203 @@
+// Fixed-point arithmetic of the FP64 Legendre stage (legendre_fx.cu).
+//
+// GB300 issues 1.9 FP64 multiply-adds per clock and SM, so the recurrence runs in 64-bit
+// integers (a 32 x 32 -> 64 bit multiply issues at 56 per clock and SM) and the contraction on
+// the FP16 tensor cores over 8-bit digits, whose products and sums are exact in FP32.
+//
+// Values.  mu_l (common.h: the rescaled Legendre values) is held as V = sigma mu 2^S, |V| < 2^62,
+// with S = 62 - b chosen per m from the largest |mu_l| of the grid (|mu| < 2^b, recorded when the
+// grid is planned; b is 1 to 4 in practice, so the quantum is 2^-58 or finer).  The sign sigma
+// = + + - - by l - m modulo 4 turns mu_l = A x mu_{l-1} - mu_{l-2} into V2 - A x V1 (l - m even) and
+// V2 + A x V1 (odd); the coefficients (synthesis) or the results (adjoint) take sigma back.
+// For the products V = h 2^32 + l with both words signed; for the contraction the bytes of
+// V + 2^63 are its base-256 digits, byte 7 less 128, the others as they are.
+// Before a pair's values are of order one (they grow from 2^-64 where its walk starts; smaller
+// ones are below the last digit), V carries a binary exponent e (a multiple of 8):
+// mu = V 2^-(S + e), V shifted down by 8 bits as it grows; e is 0 from |mu| ~ 2^-7 on.
+//
+// Coefficients and ring parts are scaled by a power of two per (m, map) to |a| < 2^54 and split
+// into 7 signed digits (-128..127).  With digits u_i of V (7 of them, from byte 7 down, V rounded
+// to them) and d_j of a, the contraction sums u_i d_j for i + j <= 7 in FP32: u is passed as an
+// FP16 subnormal (the byte itself, u 2^-24), d as an FP16 integer; |sum| < 2^24 units over 64
+// terms of 7 products each, so every sum is exact.  The dropped products are below 2^-57 of the
+// largest one.  Integer sums do not depend on their order or on the tile.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <climits>
+
+namespace cmbws {
+
+typedef long long fx_t;
+typedef unsigned long long fxu_t;
+
+constexpr int kFxABits = 54;  // coefficients and ring parts: |a| < 2^54
+constexpr int kFxDig = 7;     // digits of both factors
+constexpr int kFxBlk = 8;     // sums kept: i + j = 0..7
+
+// 32 x 32 -> 64 bit products as PTX: written in C, the compiler folds the sign extensions of
+// the digits into 64-bit shifts and then multiplies 64 x 64 bits.
+__device__ __forceinline__ fx_t fx_mul(int a, int b) {
+  fx_t r;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ fxu_t fx_mulu(unsigned a, unsigned b) {
+  fxu_t r;
+  asm("mul.wide.u32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// S of a row from the high word of the largest |mu| of its m (0: nothing recorded)
+__device__ __forceinline__ int fx_scale(unsigned mu_hi) {
+  return 62 - max(0, (int)(mu_hi >> 20) - 1022);
+}
+
+// v 2^k rounded to nearest (v finite, |v 2^k| < 2^63)
+__device__ __forceinline__ fx_t fx_from_double(double v, int k) {
+  const fxu_t b = (fxu_t)__double_as_longlong(v);
+  const int be = (int)((b >> 52) & 0x7ff);
+  const fxu_t m = (b & 0xfffffffffffffull) | (be ? 1ull << 52 : 0ull);
+  const int s = max(be, 1) - 1075 + k;  // v = m 2^(max(be, 1) - 1075)
+  fxu_t r;
+  if (s >= 0) r = s < 64 ? m << s : 0;
+  else r = s > -64 ? (m + (1ull << (-s - 1))) >> -s : 0;
+  return (b >> 63) ? -(fx_t)r : (fx_t)r;
+}
+// Digits of two scaled coefficients as FP16 integers, the first in the lower half: w[j] holds the
+// digits d_j (j = 0 the leading one).  1024 + u has a byte u in its lowest mantissa bits; minus
+// 1152 leaves u - 128 exactly.
+__device__ __forceinline__ void fx_coef_digits(fx_t v0, fx_t v1, unsigned (&w)[kFxDig]) {
+  const fxu_t a = (fxu_t)v0 + 0x80808080808080ull, b = (fxu_t)v1 + 0x80808080808080ull;
+#pragma unroll
+  for (int j = 0; j < kFxDig; ++j) {
+    const int byte = kFxDig - 1 - j;
+    const unsigned x = (unsigned)(byte < 4 ? a : a >> 32), y = (unsigned)(byte < 4 ? b : b >> 32);
+    const unsigned sel = (unsigned)(byte & 3);
+    unsigned t = __byte_perm(x, y, sel | ((sel + 4) << 4));       // bytes u0, u1
+    t = __byte_perm(t, 0x64646464u, 0x4140);                      // 0x64 above each
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(w[j]) : "r"(t), "r"(0x64806480u));
+  }
+}
+
+// A_lm as {upper word, lower word, shift, rounding constant} of a recurrence step: with
+// A < 2^sh the words hold A 2^(63 - sh), the shift is 2 + sh
+__device__ __forceinline__ int4 fx_coef(double A) {
+  if (!(A > 0.0)) return make_int4(0, 0, 2, 0);
+  const fxu_t b = (fxu_t)__double_as_longlong(A);
+  const int E = (int)((b >> 52) & 0x7ff) - 1023;
+  const int sh = max(E + 1, 0);
+  const fxu_t m = ((b & 0xfffffffffffffull) | (1ull << 52)) << (11 + E - sh);  // E >= -10
+  return make_int4((int)(m >> 32), (int)m, 2 + sh, 1 << (29 - sh));
+}
+
+// A x V1 rounded; x = xh 2^32 + xl holds cos(theta) 2^63.  A x is formed as A x 2^(62 - sh)
+// (dropping the lowest partial product), the product with V1 keeps 96 bits of which the shift takes
+// the upper 64.  2^63 is added to the sum of the cross products and taken out again from its upper
+// word, which is then unsigned.
+__device__ __forceinline__ fx_t fx_ax(int4 A, unsigned xh, unsigned xl, fx_t V1) {
+  const unsigned Ah = (unsigned)A.x, Al = (unsigned)A.y;
+  const fxu_t X = fx_mulu(Ah, xh) + (fx_mulu(Ah, xl) >> 32) + (fx_mulu(Al, xh) >> 32);
+  const int Xl = (int)X, Xh = (int)((unsigned)(X >> 32) + ((unsigned)X >> 31));
+  const int Vl = (int)V1, Vh = (int)((unsigned)((fxu_t)V1 >> 32) + ((unsigned)V1 >> 31));
+  const fxu_t cr = (fxu_t)fx_mul(Xl, Vh) + (fxu_t)fx_mul(Xh, Vl) + ((1ull << 63) + (unsigned)A.w);
+  const fxu_t hh = (fxu_t)fx_mul(Xh, Vh) + (cr >> 32) - 0x80000000ull;
+  const unsigned lo = (unsigned)hh, hi = (unsigned)(hh >> 32);
+  const unsigned ph = __funnelshift_l(lo, hi, A.z), pl = __funnelshift_l((unsigned)cr, lo, A.z);
+  return (fx_t)(((fxu_t)ph << 32) | pl);
+}
+
+// Row state of one ring pair: the last two values (V1 at l - 1, V2 at l - 2) and their exponent.
+// A pair that has not started holds zeros.
+struct FxState {
+  fx_t V1 = 0, V2 = 0;
+  int e = 0;
+  // two steps, l - m even and l + 1; the new values are V2 and V1
+  __device__ __forceinline__ void step2(int4 A0, int4 A1, unsigned xh, unsigned xl) {
+    const fx_t a = V2 - fx_ax(A0, xh, xl, V1);
+    V2 = a;
+    V1 += fx_ax(A1, xh, xl, a);
+  }
+};
+
+// start values (mu_l, mu_l+1), l - m even, at scale S -> state whose V2, V1 are those two values;
+// neg: sigma of l is -
+__device__ __forceinline__ FxState fx_start(double v0, double v1, int S, bool neg) {
+  FxState st;
+  const unsigned h = max((unsigned)__double2hiint(v0) & 0x7fffffffu,
+                         (unsigned)__double2hiint(v1) & 0x7fffffffu);
+  if (h == 0) return st;
+  // |V| < 2^(S + e + E), E = exponent bound of the larger value: at most 2^59 unless e is 0
+  st.e = max(0, (59 - S - ((int)(h >> 20) - 1022))) & ~7;
+  st.V2 = fx_from_double(neg ? -v0 : v0, S + st.e);
+  st.V1 = fx_from_double(neg ? -v1 : v1, S + st.e);
+  return st;
+}
+
+// room for a step with coefficient A while an exponent is left: |V| below 2^(61 - sh)
+__device__ __forceinline__ void fx_renorm(FxState& st, int4 A) {
+  const int ah = (int)(st.V1 >> 32), bh = (int)(st.V2 >> 32);
+  const int h = max(ah ^ (ah >> 31), bh ^ (bh >> 31));
+  if (st.e > 0 && (h >> (31 - A.z)) != 0) {
+    st.V1 = (st.V1 + 128) >> 8;
+    st.V2 = (st.V2 + 128) >> 8;
+    st.e -= 8;
+  }
+}
+
+// the value V at exponent e brought to exponent 0
+__device__ __forceinline__ fx_t fx_emit(fx_t V, int e) {
+  if (e == 0) return V;
+  return e > 62 ? 0 : (V + (1ll << (e - 1))) >> e;
+}
+
+// step2 of a pair that may start at l (with the state s0) or still carry an exponent
+__device__ __forceinline__ void fx_step2_slow(FxState& st, int4 A0, int4 A1, unsigned xh, unsigned xl,
+                                              bool start, const FxState& s0) {
+  fx_renorm(st, A0);
+  st.V2 -= fx_ax(A0, xh, xl, st.V1);
+  fx_renorm(st, A1);
+  st.V1 += fx_ax(A1, xh, xl, st.V2);
+  if (start) st = s0;
+}
+
+// Seven digit words of two consecutive values (the first in the lower half): w[i] holds the two
+// bytes 7 - i as FP16 subnormals.  The values are rounded to bit 8.
+__device__ __forceinline__ void fx_digit_pair(fx_t E0, fx_t E1, unsigned (&w)[kFxDig]) {
+  const fxu_t a = (fxu_t)E0 + ((1ull << 63) + 128), b = (fxu_t)E1 + ((1ull << 63) + 128);
+  const unsigned l0 = (unsigned)a, l1 = (unsigned)b, h0 = (unsigned)(a >> 32), h1 = (unsigned)(b >> 32);
+  const unsigned p0 = __byte_perm(l0, l1, 0x5410), p1 = __byte_perm(l0, l1, 0x7632);
+  const unsigned p2 = __byte_perm(h0, h1, 0x5410), p3 = __byte_perm(h0, h1, 0x7632);
+  w[0] = __byte_perm(p3, 0, 0x4341);
+  w[1] = p3 & 0x00ff00ffu;
+  w[2] = __byte_perm(p2, 0, 0x4341);
+  w[3] = p2 & 0x00ff00ffu;
+  w[4] = __byte_perm(p1, 0, 0x4341);
+  w[5] = p1 & 0x00ff00ffu;
+  w[6] = __byte_perm(p0, 0, 0x4341);
+}
+
+// Sums of one output column: sum_s I_s 2^(8 (7 - s)) over the blocks s = i + j, kept as
+// H 2^32 + L (H the blocks 0..3).
+struct FxSum {
+  fx_t H = 0, L = 0;
+  // I_s of one drain; |I_s| < 2^24, and I_0, I_2 (fewer products, smaller leading digits) below
+  // 2^23, so that the upper blocks combine pairwise in 32 bits
+  __device__ __forceinline__ void add(int s, int v, int& prev) {
+    if (s == 0 || s == 2) prev = v;
+    else if (s == 1) H += fx_mul(prev * 256 + v, 65536);
+    else if (s == 3) H += (fx_t)(prev * 256 + v);
+    else if (s < 7) L += fx_mul(v, 1 << (8 * (7 - s)));
+    else L += (fx_t)v;
+  }
+  // less 128 times the sum of the coefficients (sum, 2^-30 of it in hi), for byte 7 stored plus
+  // 128: 128 sum_k a_k 2^8 in these units
+  __device__ __forceinline__ double value(fx_t shi, fx_t slo, int k) const {
+    const fx_t h = H - (shi << 13), l = L - (slo << 15);
+    return scalbn((double)h * 4294967296.0 + (double)l, k);
+  }
+};
+
+}  // namespace cmbws

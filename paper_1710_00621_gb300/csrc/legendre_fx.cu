@@ -1,0 +1,714 @@
+// FP64 Legendre stage (CMBWS_FP64): the recurrence in 64-bit fixed
+// point on the CUDA cores, the contraction on the tcgen05 tensor cores over 8-bit digits with
+// exact sums.  The arithmetic, its digits and their error are described in fixed.h.
+//
+// Both stages are products with Lambda[pair][l] = mu_l(theta_pair) (Sec. 2.1):
+//   synthesis   D[pair][col] = sum_l Lambda[pair][l] B[l][col], col = parity(l - m) 8 + part;
+//   adjoint     D[l][col] = sum_pairs Lambda[pair][l] B[pair][col], col = h 8 + part, h = 0 the
+//               even part (north + south) and h = 1 the odd one; row l reads its own parity.
+// The 7 digits of Lambda are the A operand (shared memory, one tile per digit), those of the
+// coefficients or ring parts the B operand (7 x 16 rows); digit i of A times the digits
+// 0..7 - i of B accumulate into columns 16 i.. of the accumulator, so that block s of 16 columns
+// holds the sum over i + j = s.  Every 64 terms the blocks are read from tensor memory and added
+// as integers.
+#include <climits>
+
+#include "common.h"
+#include "fixed.h"
+#include "tcgen05.h"
+
+namespace cmbws {
+
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kM = 128;              // MMA rows: ring pairs (synthesis) or values of l (adjoint)
+constexpr int kNT = 2 * kM;          // threads per CTA: two per row
+constexpr int kBStep = kFxDig * 512;  // one K step of B: 7 digits of 16 rows x 16 halves
+constexpr uint32_t kCols = kFxBlk * 16;  // accumulator columns
+
+__device__ unsigned int g_fx_status = 0;  // bit 0: a bounded mbarrier wait ran out
+
+// kind::f16, FP16 A and B, FP32 D, M = 128, N = 16 nb; A K-major or MN-major, B K-major
+__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t adesc, uint64_t bdesc, int nb, bool mn,
+                                        uint32_t acc) {
+  const uint32_t idesc = (1u << 4) | (mn ? 1u << 15 : 0u) | ((uint32_t)(2 * nb) << 17) | (8u << 24);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+      : "memory");
+}
+// One K step: digit i of A (tiles atile bytes apart) times the digits 0..7 - i of B into blocks
+// i..7; `first` clears the accumulator (digit 1 writes blocks 1..7, digit 0 block 0).
+__device__ __forceinline__ void mma_step(uint32_t d, uint32_t ab, int atile, uint32_t alb, uint32_t asb,
+                                         uint32_t bb, bool mn, bool first) {
+  const uint64_t a0 = smem_desc(ab, alb, asb), a1 = smem_desc(ab + atile, alb, asb);
+  const uint64_t b0 = smem_desc(bb, 128, 256);
+  mma_f16(d + 16, a1, b0, kFxDig, mn, first ? 0u : 1u);
+  if (first) {
+    mma_f16(d, a0, b0, 1, mn, 0u);
+    mma_f16(d + 16, a0, smem_desc(bb + 512, 128, 256), kFxDig - 1, mn, 1u);
+  } else {
+    mma_f16(d, a0, b0, kFxDig, mn, 1u);
+  }
+#pragma unroll
+  for (int i = 2; i < kFxDig; ++i)
+    mma_f16(d + 16 * i, smem_desc(ab + i * atile, alb, asb), b0, kFxBlk - i, mn, 1u);
+}
+
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_addr(slot)),
+               "n"(kCols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void tmem_free(uint32_t tb) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tb), "n"(kCols) : "memory");
+}
+
+// digit words of zero (byte 7 is stored plus 128)
+__device__ __forceinline__ unsigned zero_digit(int i) { return i == 0 ? 0x00800080u : 0u; }
+
+// Eight values of l of one pair as digits: per digit one 16-byte row of A (8 halves), tiles `tile`
+// bytes apart.  co: the recurrence coefficients; la: the first l; ls: where the pair starts (s0 the
+// values there); skip: the state already holds the first two values; wait(): the previous stage's
+// MMAs have read the tile.
+template <typename W>
+__device__ __forceinline__ void fx_walk8(FxState& s, const int4* co, unsigned xh, unsigned xl, int la,
+                                         int ls, const FxState& s0, bool skip, unsigned char* row,
+                                         int tile, W&& wait) {
+  // warp-uniform: a pair starts here, or still carries an exponent
+  if (__any_sync(kFull, s.e > 0 || (ls >= la && ls < la + 8))) {
+    wait();
+#pragma unroll 1
+    for (int j = 0; j < 8; j += 2) {
+      unsigned d[kFxDig];
+      if (!skip || j > 0) fx_step2_slow(s, co[j], co[j + 1], xh, xl, ls == la + j, s0);
+      fx_digit_pair(fx_emit(s.V2, s.e), fx_emit(s.V1, s.e), d);
+#pragma unroll
+      for (int i = 0; i < kFxDig; ++i) *reinterpret_cast<unsigned*>(row + i * tile + 2 * j) = d[i];
+    }
+    return;
+  }
+  uint4 w[kFxDig];
+  unsigned* ww = reinterpret_cast<unsigned*>(w);
+#pragma unroll
+  for (int j = 0; j < 8; j += 2) {
+    unsigned d[kFxDig];
+    if (j > 0 || !skip) s.step2(co[j], co[j + 1], xh, xl);
+    fx_digit_pair(s.V2, s.V1, d);
+#pragma unroll
+    for (int i = 0; i < kFxDig; ++i) ww[4 * i + j / 2] = d[i];
+  }
+  wait();
+#pragma unroll
+  for (int i = 0; i < kFxDig; ++i) *reinterpret_cast<uint4*>(row + i * tile) = w[i];
+}
+
+__device__ __forceinline__ int digit_sum(uint32_t d) {
+  return __float2int_rn(__uint_as_float(d) * 16777216.f);  // FP16 subnormals: units of 2^-24
+}
+
+__device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
+
+// ---- synthesis ----
+constexpr int kSynK = 16;                        // values of l per stage (one K step)
+constexpr int kSynPeriod = 8;                    // stages between two reads: 64 terms per parity
+constexpr int kSynTile = kM * kSynK * 2;         // one digit of A
+constexpr int kSynA = kFxDig * kSynTile;
+struct SynLayout {
+  static constexpr int kA = 0;                      // also the odd sums at the end: double[8][128]
+  static constexpr int kB = kSynA;                  // two stages of B
+  static constexpr int kCoef = kB + 2 * kBStep;     // int4[2][16]
+  static constexpr int kCorr = kCoef + 2 * kSynK * 16;  // fxu_t[16][2]
+  static constexpr int kBar = kCorr + 16 * 16;      // uint64_t[2]
+  static constexpr int kMisc = kBar + 16;           // tensor memory base, bad flag, first start, exponents
+  static constexpr int kBytes = kMisc + 32;
+};
+
+// Two threads per ring pair (row of A) walk l upwards: one from the first start of the CTA's pairs,
+// one from the checkpoint in the middle of the rest (half the chain, twice the warps to hide the
+// recurrence's latency).  Per stage each writes the digits of 8 values of l as one 16-byte row per
+// digit tile (consecutive threads are 16 bytes apart); every second stage it converts one
+// coefficient part to digits of B.  One thread issues the stage's MMAs after its barrier; they read
+// the tile while the threads compute the next values in registers.
+template <int NM>
+__global__ void __launch_bounds__(kNT, 3)
+k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double* __restrict__ Acoef,
+               const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
+               const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
+               const double2* __restrict__ ck, const int64_t* __restrict__ ck_base,
+               const int2* __restrict__ pring, double2* __restrict__ F, int64_t F_stride, int L, int npair,
+               int R) {
+  using LY = SynLayout;
+  constexpr int P = 2 * NM;
+  extern __shared__ __align__(1024) unsigned char sm[];
+  int4* s_coef = reinterpret_cast<int4*>(sm + LY::kCoef);
+  fxu_t* s_corr = reinterpret_cast<fxu_t*>(sm + LY::kCorr);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + LY::kBar);
+  uint32_t* s_tb = reinterpret_cast<uint32_t*>(sm + LY::kMisc);
+  int* s_bad = reinterpret_cast<int*>(sm + LY::kMisc + 4);
+  int* s_lo = reinterpret_cast<int*>(sm + LY::kMisc + 8);
+  unsigned* s_emax = reinterpret_cast<unsigned*>(sm + LY::kMisc + 16);
+
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int row = tid & (kM - 1), chain = tid >> 7;  // chain: warp-uniform
+  const int m = blockIdx.y;
+  const int64_t lmo = lm_off(L, m) - m;  // index of (m, l) is lmo + l
+  const int S = fx_scale(mumax[m]);
+
+  // scale of each map: the largest exponent among this m's coefficients
+  if (tid < 4) s_emax[tid] = 0;
+  if (tid == 0) {
+    *s_bad = 0;
+    mbar_init(&mbar[0], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NM; ++k) {
+    unsigned e = 0;
+#pragma unroll 4
+    for (int l = m + tid; l <= L; l += kNT) {
+      const double2 v = alm[k * alm_stride + lmo + l];
+      e = max(e, max((unsigned)__double2hiint(v.x) & 0x7fffffffu,
+                     (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+    }
+    e = __reduce_max_sync(kFull, e >> 20);
+    if ((tid & 31) == 0) atomicMax(&s_emax[k], e);
+  }
+  // zero B (columns of the other parity and of absent maps stay zero)
+  for (int i = tid; i < 2 * kBStep / 16; i += kNT)
+    reinterpret_cast<uint4*>(sm + LY::kB)[i] = make_uint4(0, 0, 0, 0);
+  if (warp == 0) tmem_alloc(s_tb);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tb = *s_tb;
+  const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+
+  // this thread's coefficient part of a stage (of the stages t with t mod 2 = chain): value k of l
+  // (0..7 of the first chain, 8..15 of the second), part q (re / im of each map)
+  const int bk = tid & 15, bq = (tid >> 4) & 7;
+  const bool bon = bq < P;
+  const int eb = bon ? (int)s_emax[bq >> 1] - 1022 : 0;  // |a| < 2^eb; 1025 if not finite
+  const double* bsrc = reinterpret_cast<const double*>(alm + (bq >> 1) * alm_stride + lmo) + (bq & 1);
+  unsigned char* bdst = sm + LY::kB + (bk & 1) * 256 + (bk >> 3) * 128 + (bq & 7) * 16 + (bk & 7) * 2;
+  unsigned char* arow = sm + LY::kA + chain * (kSynTile / 2) + row * 16;
+
+  int gs = 0;  // stages issued by this CTA
+  bool bad = false;
+  for (int r = 0; r < R; ++r) {
+    const int p = (blockIdx.x * R + r) * kM + row;
+    const bool valid = p < npair;
+    const int ls = valid ? ls_tab[(int64_t)m * npair + p] : INT_MAX;
+    const uint64_t x = valid ? xfx[p] : 0;
+    const unsigned xh = (unsigned)(x >> 32), xl = (unsigned)x;
+    FxState s0;  // the pair's start values
+    if (ls <= L) {
+      const double2 v = st[(int64_t)m * npair + p];
+      s0 = fx_start(v.x, v.y, S, ((ls - m) & 2) != 0);
+    }
+    if (tid == 0) *s_lo = INT_MAX;
+    if (tid < 32) s_corr[tid] = 0;
+    __syncthreads();
+    const int wlo = __reduce_min_sync(kFull, ls);
+    if ((tid & 31) == 0) atomicMin(s_lo, wlo);
+    // rows of pairs that have not started: zero digits
+#pragma unroll
+    for (int i = 0; i < kFxDig; ++i) {
+      const unsigned z = zero_digit(i);
+      *reinterpret_cast<uint4*>(arow + i * kSynTile) = make_uint4(z, z, z, z);
+    }
+    __syncthreads();
+    const int lo = min(*s_lo, L + 1);
+    // the second chain starts at a checkpoint l = lm near the middle of lo..L (past L: none)
+    const int cm = ((lo + L) / 2 - m + kFxChunk / 2) / kFxChunk;
+    int lm = m + kFxChunk * cm;
+    if (lm <= lo) lm += kFxChunk;
+    const int len = lo <= L ? max(min(lm, L + 1) - lo, L + 1 - lm) : 0;
+    const int nst = (len + kSynK / 2 - 1) / (kSynK / 2);
+    // l of value k (0..15) of stage t, or -1
+    auto l_of = [&](int t, int k) {
+      const int l = (k < 8 ? lo : lm - 8) + 8 * t + k;
+      return t < nst && l <= L && (k >= 8 || l < lm) ? l : -1;
+    };
+    auto load_a = [&](int t) {  // coefficient part of stage t
+      const int l = l_of(t, bk);
+      return (bon && eb < 1025 && l >= 0) ? bsrc[2 * l] : 0.0;
+    };
+    auto load_c = [&](int t) {  // recurrence coefficient of stage t (16 threads)
+      const int l = l_of(t, tid & 15);
+      return l >= 0 ? Acoef[lmo + l] : 0.0;
+    };
+    const bool con = tid >= 112 && tid < 128;
+    const bool neg = (((bk < 8 ? lo - m : 0) + bk) & 2) != 0;  // sigma of this thread's values of l
+    double anext = load_a(chain), cnext = con ? load_c(0) : 0.0;
+    if (con) s_coef[tid & 15] = fx_coef(cnext);
+    cnext = con ? load_c(1) : 0.0;
+    __syncthreads();
+
+    FxState s;
+    if (chain && valid && lm <= L) {
+      const double2 v = ck[ck_base[m] + (int64_t)p * ((L - m + kFxChunk) / kFxChunk) + (lm - m) / kFxChunk];
+      s = fx_start(v.x, v.y, S, false);
+    }
+    const int la0 = chain ? lm : lo;                   // first l of this thread's chain
+    const int lst = chain && ls <= lm ? INT_MAX : ls;  // where the pair starts in it
+    FxSum acc[P];  // sums of the parity `chain`
+    fx_t shi = 0, slo = 0;
+    for (int t = 0; t < nst; ++t, ++gs) {
+      if (con) {  // coefficients of the next stage
+        s_coef[((t + 1) & 1) * kSynK + (tid & 15)] = fx_coef(cnext);
+        cnext = load_c(t + 2);
+      }
+      if ((t & 1) == chain) {
+        const double av = anext;
+        anext = load_a(t + 2);
+        if (bon) {  // B of this stage: its buffer was read two stages ago
+          const fx_t v = fx_from_double(neg ? -av : av, kFxABits - eb);
+          unsigned dig[kFxDig];
+          fx_coef_digits(v, 0, dig);
+          shi += v >> 30;
+          slo += v & ((1 << 30) - 1);
+#pragma unroll
+          for (int j = 0; j < kFxDig; ++j)
+            *reinterpret_cast<unsigned short*>(bdst + (gs & 1) * kBStep + j * 512) = (unsigned short)dig[j];
+        }
+      }
+      auto wait = [&]() {  // the previous stage's MMAs have read the tile
+        if (gs >= 1 && !*s_bad && !mbar_wait(&mbar[0], (gs - 1) & 1)) bad = true;
+      };
+      if (wlo < la0 + 8 * t + 8)  // some pair of the warp has started
+        fx_walk8(s, s_coef + (t & 1) * kSynK + 8 * chain, xh, xl, la0 + 8 * t, lst, s0, chain && t == 0,
+                 arow, kSynTile, wait);
+      else
+        wait();
+      fence_smem_async();
+      tc_fence_before();
+      if (bad) atomicOr(s_bad, 1);
+      __syncthreads();
+      const bool first = t % kSynPeriod == 0;
+      if (tid == 0 && !*s_bad) {
+        tc_fence_after();
+        mma_step(tb, smem_addr(sm + LY::kA), kSynTile, kSynTile / 2, 128,
+                 smem_addr(sm + LY::kB + (gs & 1) * kBStep), false, first);
+        tc_commit(&mbar[0]);
+      }
+      if (t % kSynPeriod == kSynPeriod - 1 || t == nst - 1) {
+        if (!*s_bad && !mbar_wait(&mbar[0], gs & 1)) bad = true;
+        tc_fence_after();
+        int prev[P];
+#pragma unroll
+        for (int b = 0; b < kFxBlk; ++b) {
+          uint32_t d[8];
+          tmem_ld8(tb + lane_base + 16 * b + 8 * chain, d);
+          tmem_ld_wait();
+#pragma unroll
+          for (int q = 0; q < P; ++q) acc[q].add(b, digit_sum(d[q]), prev[q]);
+        }
+        tc_fence_before();  // read before the next stage's MMAs, which follow its barrier
+      }
+    }
+    if (bon) {
+      atomicAdd(&s_corr[2 * ((bk & 1) * 8 + bq)], (fxu_t)shi);
+      atomicAdd(&s_corr[2 * ((bk & 1) * 8 + bq) + 1], (fxu_t)slo);
+    }
+    if (bad) atomicOr(s_bad, 1);
+    __syncthreads();
+    const bool failed = *s_bad != 0;
+    double v[P];
+    double* s_odd = reinterpret_cast<double*>(sm + LY::kA);  // [part][row]; all MMAs are done
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+      const int ea = (int)s_emax[q >> 1] - 1022;
+      v[q] = acc[q].value((fx_t)s_corr[2 * (8 * chain + q)], (fx_t)s_corr[2 * (8 * chain + q) + 1], ea - S - 6);
+      // a map with a non-finite coefficient, and a timed-out wait, give NaN
+      if ((ea >= 1025 && ls <= L) || failed) v[q] = fx_nan();
+      if (chain) s_odd[q * kM + row] = v[q];
+    }
+    __syncthreads();
+    if (valid && !chain) {
+      const int2 rr = pring[p];
+#pragma unroll
+      for (int k = 0; k < NM; ++k) {
+        const double ox = s_odd[2 * k * kM + row], oy = s_odd[(2 * k + 1) * kM + row];
+        F[k * F_stride + (int64_t)rr.x * (L + 1) + m] = make_double2(v[2 * k] + ox, v[2 * k + 1] + oy);
+        if (rr.y >= 0)
+          F[k * F_stride + (int64_t)rr.y * (L + 1) + m] = make_double2(v[2 * k] - ox, v[2 * k + 1] - oy);
+      }
+    }
+    __syncthreads();  // s_corr and the A rows are reset for the next group
+  }
+  if (tid == 0 && *s_bad) atomicOr(&g_fx_status, 1u);
+  if (warp == 0) tmem_free(tb);
+}
+
+// Tiles: groups of 128 ring pairs per CTA, taken one after the other (the autotuner's list of the
+// synthesis; without it one group per CTA).
+template <int NM>
+int launch_synth_variant(int v, const Grid& g, const void* alm, int64_t as, void* F, int64_t fs,
+                         cudaStream_t s) {
+  const int R = v == 0 ? 2 : v == 3 ? 4 : 1;
+  const int L = g.lmax;
+  dim3 grd((g.npair + kM * R - 1) / (kM * R), L + 1);
+  auto kern = k_leg_synth_fx<NM>;
+  CMBWS_TRY(ensure_dyn_smem((const void*)kern, SynLayout::kBytes));
+  ProfScope ps(PROF_LEG_SYNTH, s, 1, leg_work(g, NM));
+  kern<<<grd, kNT, SynLayout::kBytes, s>>>((const double2*)alm, as, g.A64.as<double>(),
+                                          g.mumax.as<unsigned>(), g.lsx.as<int>(), g.stx.as<double2>(),
+                                          g.xfx.as<uint64_t>(), g.ckx.as<double2>(),
+                                          g.ckx_base.as<int64_t>(), g.pair_ring.as<int2>(), (double2*)F, fs, L,
+                                          g.npair, R);
+  CMBWS_LAUNCH_CHECK();
+  return CMBWS_OK;
+}
+
+template <int NM>
+int launch_synth(const Grid& g, const void* alm, int64_t as, void* F, int64_t fs, cudaStream_t s) {
+  int v = 1;
+  if (autotune_mode() != 0)
+    CMBWS_TRY(autotune_pick(
+        g, synth_tune_key(CMBWS_FP64, NM), 4, 1,
+        [&](int vv) { return launch_synth_variant<NM>(vv, g, alm, as, F, fs, s); }, s, &v));
+  return launch_synth_variant<NM>(v, g, alm, as, F, fs, s);
+}
+
+int synth_dispatch(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s) {
+  const int64_t as = nlm_of(g.lmax), fs = (int64_t)g.nring * (g.lmax + 1);
+  for (int k0 = 0; k0 < nmaps; k0 += 4) {
+    const int nm = nmaps - k0 < 4 ? nmaps - k0 : 4;
+    const void* a = (const double2*)alm + k0 * as;
+    void* f = (double2*)F + k0 * fs;
+    int st = CMBWS_OK;
+    switch (nm) {
+      case 1: st = launch_synth<1>(g, a, as, f, fs, s); break;
+      case 2: st = launch_synth<2>(g, a, as, f, fs, s); break;
+      case 3: st = launch_synth<3>(g, a, as, f, fs, s); break;
+      default: st = launch_synth<4>(g, a, as, f, fs, s); break;
+    }
+    if (st != CMBWS_OK) return st;
+  }
+  return CMBWS_OK;
+}
+
+// ---- adjoint ----
+constexpr int kAdjK = 32;                       // ring pairs per stage (two K steps)
+constexpr int kAdjTile = kM * kAdjK * 2;        // one digit of A
+constexpr int kAdjOct = kAdjK * 16;             // bytes between rows 8 i and 8 (i + 1) of A
+struct AdjLayout {
+  static constexpr int kA = 0;
+  static constexpr int kB = kFxDig * kAdjTile;       // two stages of B (two K steps each)
+  static constexpr int kCoef = kB + 4 * kBStep;      // int4[128]
+  static constexpr int kCorr = kCoef + kM * 16;      // fxu_t[16][2]
+  static constexpr int kBar = kCorr + 16 * 16;       // uint64_t[2]
+  static constexpr int kMisc = kBar + 16;            // tensor memory base, bad flag
+  static constexpr int kBytes = kMisc + 16;
+};
+
+__device__ __forceinline__ unsigned part_exp(double v) {
+  return ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
+}
+
+// ee[map][m] = exponent bound of the map's ring parts at m: |e| < 2^ee (1025: not all finite)
+template <int NM>
+__global__ void __launch_bounds__(256)
+k_eo_exp(const double* __restrict__ eo, int npair, int L, int* __restrict__ ee) {
+  __shared__ unsigned s_e[NM];
+  const int m = blockIdx.x, tid = threadIdx.x;
+  if (tid < NM) s_e[tid] = 0;
+  __syncthreads();
+  const double* src = eo + (int64_t)m * npair * 4 * NM;
+  unsigned e[NM];
+#pragma unroll
+  for (int k = 0; k < NM; ++k) e[k] = 0;
+  for (int i = tid; i < 2 * npair; i += 256) {  // (pair, parity): 2 NM values
+#pragma unroll
+    for (int k = 0; k < NM; ++k)
+      e[k] = max(e[k], max(part_exp(src[(int64_t)i * 2 * NM + 2 * k]), part_exp(src[(int64_t)i * 2 * NM + 2 * k + 1])));
+  }
+#pragma unroll
+  for (int k = 0; k < NM; ++k) {
+    const unsigned v = __reduce_max_sync(kFull, e[k]);
+    if ((tid & 31) == 0) atomicMax(&s_e[k], v);
+  }
+  __syncthreads();
+  if (tid < NM) ee[(int64_t)tid * (L + 1) + m] = (int)s_e[tid] - 1022;
+}
+
+// One CTA per (m, 128 values of l) loops over the ring pairs, 32 per stage: lane = pair, warp =
+// chunk of 16 values of l, which each thread walks from the chunk's FP64 checkpoint; rows of A are
+// values of l (MN-major: a thread writes 8 consecutive values of its pair as one 16-byte row).
+// Every output has one owner; stages without a started pair are skipped.
+template <int NM>
+__global__ void __launch_bounds__(kNT, 3)
+k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const double* __restrict__ Acoef,
+             const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
+             const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
+             const double2* __restrict__ ck, const int64_t* __restrict__ ck_base,
+             const int* __restrict__ tmin, const double* __restrict__ c64, double2* __restrict__ out,
+             int64_t nlm, int L, int npair) {
+  using LY = AdjLayout;
+  constexpr int P = 2 * NM;
+  static_assert(kFxChunk == 16 && kAdjK == 32 && kTileMinPT == 16, "stage shape");
+  const int m = blockIdx.y;
+  const int lb0 = m + kM * (int)blockIdx.x;  // first l of the tile
+  if (lb0 > L) return;                       // CTA-uniform, before any barrier
+  extern __shared__ __align__(1024) unsigned char sm[];
+  int4* s_coef = reinterpret_cast<int4*>(sm + LY::kCoef);
+  fxu_t* s_corr = reinterpret_cast<fxu_t*>(sm + LY::kCorr);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + LY::kBar);
+  uint32_t* s_tb = reinterpret_cast<uint32_t*>(sm + LY::kMisc);
+  int* s_bad = reinterpret_cast<int*>(sm + LY::kMisc + 4);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t lmo = lm_off(L, m) - m;
+  const int llast = min(L, lb0 + kM - 1);
+  const int ntm = (npair + kTileMinPT - 1) / kTileMinPT;
+  const int nst = (npair + kAdjK - 1) / kAdjK;
+  const int* tm = tmin + (int64_t)m * ntm;
+  // first stage from s on with a pair that starts by the tile's last l
+  auto next_stage = [&](int s) {
+    while (s < nst && tm[2 * s] > llast && (2 * s + 1 >= ntm || tm[2 * s + 1] > llast)) ++s;
+    return s;
+  };
+  int s = next_stage(0);
+  if (s >= nst) {  // no pair has a significant value in the tile: the sums are zero
+    const int l = lb0 + tid;
+    if (tid < kM && l <= L)
+#pragma unroll
+      for (int k = 0; k < NM; ++k) out[k * nlm + lmo + l] = make_double2(0.0, 0.0);
+    return;
+  }
+  const int S = fx_scale(mumax[m]);
+  if (tid == 0) {
+    *s_bad = 0;
+    mbar_init(&mbar[0], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (tid < 32) s_corr[tid] = 0;
+  if (tid < kM) {
+    const int l = lb0 + tid;
+    s_coef[tid] = fx_coef(l <= L ? Acoef[lmo + l] : 0.0);
+  }
+  for (int i = tid; i < 4 * kBStep / 16; i += kNT)  // B columns of absent maps stay zero
+    reinterpret_cast<uint4*>(sm + LY::kB)[i] = make_uint4(0, 0, 0, 0);
+  if (warp == 0) tmem_alloc(s_tb);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tb = *s_tb;
+  const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+
+  // chunk of this warp
+  const int l0 = lb0 + kFxChunk * warp;
+  const bool cval = l0 <= L;
+  const int nck = (L - m + kFxChunk) / kFxChunk;
+  const double2* ckc = ck + (cval ? ck_base[m] + (l0 - m) / kFxChunk : 0);  // + p * nck
+  const int* lsm = ls_tab + (int64_t)m * npair;
+  const double2* stm = st + (int64_t)m * npair;
+  unsigned char* arow = sm + LY::kA + 2 * warp * kAdjOct + lane * 16;
+
+  // this thread's ring parts of a stage: column nn of parity par, pairs 8 oct + 2 quarter + 0..1
+  const int quarter = tid & 3, nn = (tid >> 2) & 7, oct = (tid >> 5) & 3, par = tid >> 7;
+  const bool bon = nn < P;
+  const int eb = bon ? ee[(int64_t)(nn >> 1) * (L + 1) + m] : 0;
+  const double* bsrc = eo + (int64_t)m * npair * 2 * P + par * P + nn;
+  unsigned char* bdst = sm + LY::kB + (oct >> 1) * kBStep + par * 256 + (oct & 1) * 128 + nn * 16 + quarter * 4;
+
+  // inputs of a stage, loaded one stage ahead
+  struct In {
+    double e[2];
+    double2 c;
+    uint64_t x;
+    int ls;
+  };
+  auto load = [&](int t, In& in) {
+    const int p = t * kAdjK + lane;
+    const bool ok = t < nst && p < npair;
+    in.ls = ok ? lsm[p] : INT_MAX;
+    in.x = ok ? xfx[p] : 0;
+    in.c = make_double2(0.0, 0.0);
+    if (ok && cval) in.c = ckc[(int64_t)p * nck];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int q = t * kAdjK + 8 * oct + 2 * quarter + i;
+      in.e[i] = 0.0;
+      if (bon && eb < 1025 && t < nst && q < npair) in.e[i] = bsrc[(int64_t)q * 2 * P];
+    }
+  };
+  In in;
+  load(s, in);
+
+  const int grp = tid >> 7;  // real (0) or imaginary (1) parts of row tid mod 128
+  FxSum acc[NM];
+  fx_t shi = 0, slo = 0;
+  bool bad = false, zeroed = false;
+  for (int k = 0; s < nst; ++k) {
+    const int sn = next_stage(s + 1);
+    const int p = s * kAdjK + lane, ls = in.ls;
+    const unsigned xh = (unsigned)(in.x >> 32), xl = (unsigned)in.x;
+    const bool on = cval && __any_sync(kFull, ls <= min(L, l0 + kFxChunk - 1));
+    FxState w, s0;
+    if (on) {
+      w = fx_start(in.c.x, in.c.y, S, false);  // zeros if the pair starts later
+      const bool inj = ls > l0 && ls < l0 + kFxChunk && ls <= L;
+      if (__any_sync(kFull, inj)) {
+        double2 v = make_double2(0.0, 0.0);
+        if (inj) v = stm[p];
+        s0 = fx_start(v.x, v.y, S, ((ls - m) & 2) != 0);
+      }
+    }
+    const double ev[2] = {in.e[0], in.e[1]};
+    load(sn, in);
+    if (bon) {  // B of this stage: its buffer was read two stages ago
+      fx_t v[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        v[i] = fx_from_double(ev[i], kFxABits - eb);
+        shi += v[i] >> 30;
+        slo += v[i] & ((1 << 30) - 1);
+      }
+      unsigned dig[kFxDig];
+      fx_coef_digits(v[0], v[1], dig);
+#pragma unroll
+      for (int j = 0; j < kFxDig; ++j)
+        *reinterpret_cast<unsigned*>(bdst + (k & 1) * 2 * kBStep + j * 512) = dig[j];
+    }
+    auto wait = [&]() {  // the previous stage's MMAs have read the tile
+      if (k >= 1 && !*s_bad && !mbar_wait(&mbar[0], (k - 1) & 1)) bad = true;
+    };
+    if (on) {
+      const int lst = ls > l0 ? ls : INT_MAX;
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h)
+        fx_walk8(w, s_coef + kFxChunk * warp + 8 * h, xh, xl, l0 + 8 * h, lst, s0, h == 0,
+                 arow + h * kAdjOct, kAdjTile, wait);
+      zeroed = false;
+    } else {
+      wait();
+      if (!zeroed)  // no pair of the stage has started in this chunk: zero digits
+#pragma unroll
+        for (int i = 0; i < kFxDig; ++i) {
+          const unsigned z = zero_digit(i);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            *reinterpret_cast<uint4*>(arow + i * kAdjTile + h * kAdjOct) = make_uint4(z, z, z, z);
+        }
+      zeroed = true;
+    }
+    fence_smem_async();
+    tc_fence_before();
+    if (bad) atomicOr(s_bad, 1);
+    __syncthreads();
+    const bool first = (k & 1) == 0;  // sums are read after every second stage (64 pairs)
+    if (tid == 0 && !*s_bad) {
+      tc_fence_after();
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks)
+        mma_step(tb, smem_addr(sm + LY::kA) + ks * 256, kAdjTile, 128, kAdjOct,
+                 smem_addr(sm + LY::kB + ((k & 1) * 2 + ks) * kBStep), true, first && ks == 0);
+      tc_commit(&mbar[0]);
+    }
+    if ((k & 1) == 1 || sn >= nst) {
+      if (!*s_bad && !mbar_wait(&mbar[0], k & 1)) bad = true;
+      tc_fence_after();
+      int prev[NM];
+      const int odd = tid & 1;  // parity of l - m of this thread's row
+#pragma unroll
+      for (int b = 0; b < kFxBlk; ++b) {
+        uint32_t d[16];
+        tmem_ld16(tb + lane_base + 16 * b, d);
+        tmem_ld_wait();
+#pragma unroll
+        for (int q = 0; q < NM; ++q)
+          acc[q].add(b, digit_sum(odd ? (grp ? d[9 + 2 * q] : d[8 + 2 * q]) : (grp ? d[1 + 2 * q] : d[2 * q])),
+                     prev[q]);
+      }
+      tc_fence_before();  // read before the next stage's MMAs, which follow its barrier
+    }
+    s = sn;
+  }
+  if (bon) {
+    atomicAdd(&s_corr[2 * (par * 8 + nn)], (fxu_t)shi);
+    atomicAdd(&s_corr[2 * (par * 8 + nn) + 1], (fxu_t)slo);
+  }
+  if (bad) atomicOr(s_bad, 1);
+  __syncthreads();
+  const bool failed = *s_bad != 0;
+  if (tid == 0 && failed) atomicOr(&g_fx_status, 1u);
+  if (warp == 0) tmem_free(tb);
+  const int l = lb0 + (tid & (kM - 1));  // row of D
+  if (l > L) return;
+  const fxu_t* corr = s_corr + 16 * (tid & 1) + 2 * grp;
+  const double cc = (tid & 2) ? -c64[lmo + l] : c64[lmo + l];  // sigma of l
+  double* o = reinterpret_cast<double*>(out + lmo + l) + grp;
+#pragma unroll
+  for (int q = 0; q < NM; ++q) {
+    const int ea = ee[(int64_t)q * (L + 1) + m];
+    const double v = acc[q].value((fx_t)corr[4 * q], (fx_t)corr[4 * q + 1], ea - S - 6);
+    // a map with a non-finite ring part, and a timed-out wait, give NaN
+    o[2 * q * nlm] = (failed || ea >= 1025) ? fx_nan() : cc * v;
+  }
+}
+
+template <int NM>
+int launch_adj(const Grid& g, const void* eo, int* ee, double* out, cudaStream_t s) {
+  const int L = g.lmax;
+  ProfScope ps(PROF_LEG_ADJ, s, 1, leg_work(g, NM));
+  k_eo_exp<NM><<<L + 1, 256, 0, s>>>((const double*)eo, g.npair, L, ee);
+  CMBWS_LAUNCH_CHECK();
+  dim3 grd((L + kM) / kM, L + 1);
+  auto kern = k_leg_adj_fx<NM>;
+  CMBWS_TRY(ensure_dyn_smem((const void*)kern, AdjLayout::kBytes));
+  kern<<<grd, kNT, AdjLayout::kBytes, s>>>((const double*)eo, ee, g.A64.as<double>(), g.mumax.as<unsigned>(),
+                                          g.lsx.as<int>(), g.stx.as<double2>(), g.xfx.as<uint64_t>(),
+                                          g.ckx.as<double2>(), g.ckx_base.as<int64_t>(),
+                                          g.ls_tmin.as<int>(), g.c64.as<double>(), (double2*)out,
+                                          nlm_of(L), L, g.npair);
+  CMBWS_LAUNCH_CHECK();
+  return CMBWS_OK;
+}
+
+int adj_dispatch(const Grid& g, int nmaps, const void* eo, int* ee, double* out, cudaStream_t s) {
+  const int64_t nlm = nlm_of(g.lmax), cs = (int64_t)(g.lmax + 1) * g.npair * 4;
+  for (int k0 = 0; k0 < nmaps; k0 += 4) {
+    const int nm = nmaps - k0 < 4 ? nmaps - k0 : 4;
+    const void* e = (const double*)eo + k0 * cs;
+    int* x = ee + (int64_t)k0 * (g.lmax + 1);
+    double* o = out + 2 * k0 * nlm;
+    int st = CMBWS_OK;
+    switch (nm) {
+      case 1: st = launch_adj<1>(g, e, x, o, s); break;
+      case 2: st = launch_adj<2>(g, e, x, o, s); break;
+      case 3: st = launch_adj<3>(g, e, x, o, s); break;
+      default: st = launch_adj<4>(g, e, x, o, s); break;
+    }
+    if (st != CMBWS_OK) return st;
+  }
+  return CMBWS_OK;
+}
+
+}  // namespace
+
+int legendre_adjoint_fx(const Grid& g, int nmaps, const void* eo, int* ee, double* out, cudaStream_t s) {
+  return adj_dispatch(g, nmaps, eo, ee, out, s);
+}
+
+int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s) {
+  return synth_dispatch(g, nmaps, alm, F, s);
+}
+
+int fx_status_take(bool* timed_out) {
+  unsigned int v = 0;
+  CMBWS_CUDA(cudaMemcpyFromSymbol(&v, g_fx_status, sizeof(v)));
+  *timed_out = (v & 1u) != 0;
+  if (v) {
+    const unsigned int zero = 0;
+    CMBWS_CUDA(cudaMemcpyToSymbol(g_fx_status, &zero, sizeof(zero)));
+  }
+  return CMBWS_OK;
+}
+
+}  // namespace cmbws

@@ -27,6 +27,7 @@
 #include <climits>
 
 #include "common.h"
+#include "tcgen05.h"
 
 namespace cmbws {
 
@@ -42,17 +43,6 @@ constexpr int kTcKB = 32;   // values of l per stage (4 MMAs of K = 8)
 // to drop; tf32_rna() clears them (needed where the rounded value is reused).
 __device__ __forceinline__ uint32_t tf32_bits(float x) { return __float_as_uint(x) + 0x1000u; }
 __device__ __forceinline__ uint32_t tf32_rna(float x) { return tf32_bits(x) & 0xFFFFE000u; }
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// K-major, no-swizzle shared-memory matrix descriptor: core matrices of 8 rows x 16 bytes,
-// LBO = byte step between core matrices along K, SBO = along N; descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
-}
 
 // Instruction descriptor: D FP32, A and B TF32, both K-major, N = 16, M = 128.
 constexpr uint32_t kIdesc = (1u << 4) | (2u << 7) | (2u << 10) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
@@ -92,28 +82,6 @@ __device__ unsigned int g_tc_status = 0;
 // Test support (cmbws_testing_stall_waits): when > 0, every CTA first waits at most this many
 // SM clocks on an mbarrier phase that nothing completes, so the wait runs out.
 __device__ long long g_tc_stall_cycles = 0;
-
-constexpr long long kWaitCycles = 1ll << 32;  // about two seconds at 2 GHz
-
-// Wait for the completion of phase `parity` of an mbarrier; false after `limit` SM clocks (or
-// 2^26 polls).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
-                                          long long limit = kWaitCycles) {
-  const uint32_t a = smem_addr(bar);
-  const long long t0 = clock64();
-  for (int it = 0; it < (1 << 26); ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}\n"
-        : "=r"(done)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (clock64() - t0 > limit) break;
-  }
-  return false;
-}
 
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32]) {
   asm volatile(
@@ -1343,6 +1311,9 @@ int tc_status_take(bool* timed_out) {
     const unsigned int zero = 0;
     CMBWS_CUDA(cudaMemcpyToSymbol(g_tc_status, &zero, sizeof(zero)));
   }
+  bool fx = false;
+  CMBWS_TRY(fx_status_take(&fx));
+  *timed_out |= fx;
   return CMBWS_OK;
 }
 

@@ -444,7 +444,7 @@ int Model::group_chain(Group& G, int prec, int which, cudaStream_t s) {
   }
   CMBWS_TRY(legendre_synth(g, prec, G.nmaps, G.alm.p, G.F.p, s));
   CMBWS_TRY(ringfft_fused(g, prec, G.nmaps, G.F.p, pix, part.p, s));
-  CMBWS_TRY(legendre_adjoint(g, prec, G.nmaps, G.F.p, part.p, part.bytes, G.out.as<double>(), s));
+  CMBWS_TRY(legendre_adjoint(g, prec, G.nmaps, part.p, part.bytes, G.out.as<double>(), s));
   return CMBWS_OK;
 }
 
@@ -488,7 +488,7 @@ int Model::mix_chain(Group& G, int prec, cudaStream_t s) {
   for (int j = 0; j < G.nmaps; ++j) pix[j] = !is_f32(prec) ? pixQ64[G.bands[j]].p : pixQ32[G.bands[j]].p;
   CMBWS_TRY(legendre_synth(g, prec, G.nmaps, G.alm.p, G.F.p, s));
   CMBWS_TRY(ringfft_fused(g, prec, G.nmaps, G.F.p, pix, part.p, s));
-  CMBWS_TRY(legendre_adjoint(g, prec, G.nmaps, G.F.p, part.p, part.bytes, G.out.as<double>(), s));
+  CMBWS_TRY(legendre_adjoint(g, prec, G.nmaps, part.p, part.bytes, G.out.as<double>(), s));
   return CMBWS_OK;
 }
 
@@ -656,7 +656,7 @@ int Model::apply_precond_merged(const double* r, double* z, int prec, cudaStream
       pix[j] = !is_f32(prec) ? P.pixM64[G.bands[j]].p : P.pixM32[G.bands[j]].p;
     CMBWS_TRY(legendre_synth(g, prec, G.nmaps, G.alm.p, G.F.p, s));
     CMBWS_TRY(ringfft_fused(g, prec, G.nmaps, G.F.p, pix, part.p, s));
-    CMBWS_TRY(legendre_adjoint(g, prec, G.nmaps, G.F.p, part.p, part.bytes, G.out.as<double>(), s));
+    CMBWS_TRY(legendre_adjoint(g, prec, G.nmaps, part.p, part.bytes, G.out.as<double>(), s));
   }
   {
     const dim3 grd = tri_grid(Lcomp, 128);
@@ -709,8 +709,8 @@ int Model::rhs(const double* const* d, const double* const* w1, const double* w2
           pixtmp.as<double>() + j * n, n);
       CMBWS_LAUNCH_CHECK();
     }
-    CMBWS_TRY(ringfft_analysis(g, ap, G.nmaps, pixtmp.as<double>(), 0, G.F.p, part.p, s));
-    CMBWS_TRY(legendre_adjoint(g, ap, G.nmaps, G.F.p, part.p, part.bytes, G.out.as<double>(), s));
+    CMBWS_TRY(ringfft_analysis(g, ap, G.nmaps, pixtmp.as<double>(), 0, part.p, s));
+    CMBWS_TRY(legendre_adjoint(g, ap, G.nmaps, part.p, part.bytes, G.out.as<double>(), s));
   }
   // transposed variable mixing of B u_nu, then the epilogue without a prior term (x = NULL)
   if (nmix) CMBWS_TRY(mixvar_adjoint(ap, s));

@@ -1,8 +1,7 @@
 // Adjoint synthesis / analysis without any device allocation.
 //
-// cmbws_sht_analysis keeps its workspace (ring spectra, the per-CTA partial
-// sums of the adjoint Legendre kernel, the reduced coefficients) in buffers
-// the grid allocates on first use.  Some callers cannot allocate device
+// cmbws_sht_analysis keeps its workspace (the adjoint Legendre stage's input and
+// the coefficients) in buffers the grid allocates on first use.  Some callers cannot allocate device
 // memory at that point: host runtimes that hand the library a fixed memory
 // budget and forbid cudaMalloc after start-up, or real-time loops that must
 // not block on the allocator (cudaMalloc can synchronise the device).
@@ -89,26 +88,33 @@ extern "C" int cmbws_sht_analysis_noalloc(cmbws_grid gh, cmbws_prec prec, const 
     set_error("cmbws_sht_analysis_noalloc: ring length %d too large for this precision", g->max_n);
     return CMBWS_ERR_ARG;
   }
+  // the documented limit: ring spectra, adjoint scratch (FP64: partial sums of blocks of 256 ring
+  // pairs) and coefficients together; what is used below stays under it
   const size_t es = prec_size(prec);
   const int64_t nlm = nlm_of(g->lmax);
+  const int cm = eo_maps(prec), nc = nmaps < cm ? nmaps : cm;
   const size_t fb = round256((size_t)nmaps * g->nring * (g->lmax + 1) * 2 * es);
-  const size_t pb = round256(legendre_adjoint_part_bytes(*g, prec, nmaps));
+  const size_t sb = prec == CMBWS_FP64
+                        ? round256((size_t)((g->npair + 255) / 256) * 2 * nc * nlm * 8)
+                        : round256(legendre_adjoint_part_bytes(*g, prec, nmaps));
   const size_t ob = round256((size_t)nmaps * nlm * 16);
-  if (fb + pb + ob > kScratchBytes) {
+  const size_t pb = round256(legendre_adjoint_part_bytes(*g, prec, nc));
+  if (fb + sb + ob > kScratchBytes || pb + ob > kScratchBytes) {
     set_error("cmbws_sht_analysis_noalloc: needs %zu bytes of scratch for nmaps=%d, lmax=%d, "
               "nring=%d; the static scratch holds %zu bytes (use cmbws_sht_analysis)",
-              fb + pb + ob, nmaps, g->lmax, g->nring, kScratchBytes);
+              fb + sb + ob, nmaps, g->lmax, g->nring, kScratchBytes);
     return CMBWS_ERR_ARG;
   }
   void* base = nullptr;
   CMBWS_TRY(scratch_address(&base));
-  unsigned char* p = static_cast<unsigned char*>(base);
-  void* F = p;
-  void* part = p + fb;
-  double* out = reinterpret_cast<double*>(p + fb + pb);
+  unsigned char* part = static_cast<unsigned char*>(base);
+  double* out = reinterpret_cast<double*>(part + pb);
   cudaStream_t s = (cudaStream_t)stream;
-  CMBWS_TRY(ringfft_analysis(*g, prec, nmaps, map, weighted, F, part, s));
-  CMBWS_TRY(legendre_adjoint(*g, prec, nmaps, F, part, pb, out, s));
+  for (int k = 0; k < nmaps; k += cm) {
+    const int nm = nmaps - k < cm ? nmaps - k : cm;
+    CMBWS_TRY(ringfft_analysis(*g, prec, nm, map + k * g->npix, weighted, part, s));
+    CMBWS_TRY(legendre_adjoint(*g, prec, nm, part, pb, out + 2 * k * nlm, s));
+  }
   CMBWS_TRY(unpack_alm(*g, nmaps, out, alm, s));
   return CMBWS_OK;
 }

@@ -50,6 +50,11 @@ __device__ __forceinline__ T2 cmul(T2 a, T2 b) {
   r.y = a.x * b.y + a.y * b.x;
   return r;
 }
+// a product rounded by itself (never contracted with a following addition)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ df mul_rn(df a, df b) { return a * b; }
+
 template <typename T2>
 __device__ __forceinline__ T2 cconj(T2 a) {
   a.y = -a.y;
@@ -545,19 +550,14 @@ k_ringfft(typename V2<T>::t* __restrict__ F, int64_t F_stride, double* __restric
     // G = (c - i s) X
     T gx = c * xnx + s * xny, gy = c * xny - s * xnx;
     T2 on, os;
-    on.x = cm * gx;
-    on.y = -cm * gy;
+    on.x = mul_rn(cm, gx);
+    on.y = mul_rn(-cm, gy);
     if (m == 0) on.y = 0;
     if (has_s) {
       gx = c * xsx + s * xsy;
       gy = c * xsy - s * xsx;
-      os.x = cm * gx;
-      os.y = m == 0 ? T(0) : -cm * gy;
-    }
-    if (!eo) {
-      FN[m] = on;
-      if (has_s) FS[m] = os;
-      continue;
+      os.x = mul_rn(cm, gx);
+      os.y = m == 0 ? T(0) : mul_rn(-cm, gy);
     }
     // the adjoint input: even-l part north + south, odd-l part north - south (a ring pair
     // without a south ring counts its north ring in both)
@@ -588,11 +588,11 @@ size_t smem_bytes(const Grid& g) {
 // others 128; 16-byte values with 8192-entry buffers (one CTA per SM) 512.
 template <typename T, int MODE>
 int launch(const Grid& g, int nmaps, void* F, double* map_out, const double* map_in, int weighted,
-           const void* const* pix, void* eo, int eo_nm, cudaStream_t s);
+           const void* const* pix, void* eo, cudaStream_t s);
 
 template <typename T, int MODE, int NT>
 int launch_nt(const Grid& g, int nmaps, void* F, double* map_out, const double* map_in,
-              int weighted, const void* const* pix, void* eo, int eo_nm, cudaStream_t s) {
+              int weighted, const void* const* pix, void* eo, cudaStream_t s) {
   using T2 = typename V2<T>::t;
   const size_t sm = smem_bytes<T>(g);
   if (sm > 227 * 1024) {
@@ -607,6 +607,7 @@ int launch_nt(const Grid& g, int nmaps, void* F, double* map_out, const double* 
   constexpr bool f32 = std::is_same<T, float>::value, f64 = std::is_same<T, double>::value;
   const TP* rw = nullptr;
   if (MODE == MODE_ANALYSIS && weighted) rw = f32 ? (const TP*)g.ring_w32.p : (const TP*)g.ring_w64.p;
+  const int prec = f32 ? CMBWS_FP32 : f64 ? CMBWS_FP64 : CMBWS_FP32X2;
   const T2* tab = f32 ? (const T2*)g.fft32.p : f64 ? (const T2*)g.fft64.p : (const T2*)g.fftdf.p;
   for (int k0 = 0; k0 < nmaps; k0 += kMaxPix) {
     const int nm = nmaps - k0 < kMaxPix ? nmaps - k0 : kMaxPix;
@@ -624,7 +625,7 @@ int launch_nt(const Grid& g, int nmaps, void* F, double* map_out, const double* 
                               map_in ? map_in + k0 * g.npix : nullptr, g.npix, rw, pp,
                               g.plans_d.as<FftPlan>(), g.pair_plan.as<int>(),
                               g.pair_ring.as<int2>(), g.pair_phase.as<int>(), g.ring_off.as<int64_t>(),
-                              tab, g.tw_off, g.nmax2, g.lmax, (T*)eo, eo_nm, k0, nmaps, g.npair);
+                              tab, g.tw_off, g.nmax2, g.lmax, (T*)eo, eo_maps(prec), k0, nmaps, g.npair);
     CMBWS_LAUNCH_CHECK();
   }
   return CMBWS_OK;
@@ -632,15 +633,15 @@ int launch_nt(const Grid& g, int nmaps, void* F, double* map_out, const double* 
 
 template <typename T, int MODE>
 int launch(const Grid& g, int nmaps, void* F, double* map_out, const double* map_in, int weighted,
-           const void* const* pix, void* eo, int eo_nm, cudaStream_t s) {
+           const void* const* pix, void* eo, cudaStream_t s) {
   // 16-byte values (double-float, FP64) with 8192-entry buffers: about 140 KB per CTA, one CTA
   // per SM, so that CTA gets 512 threads (16 warps instead of 8)
   if constexpr (!std::is_same<T, float>::value)
     if (g.nmax2 >= 8192)
-      return launch_nt<T, MODE, 512>(g, nmaps, F, map_out, map_in, weighted, pix, eo, eo_nm, s);
+      return launch_nt<T, MODE, 512>(g, nmaps, F, map_out, map_in, weighted, pix, eo, s);
   if (g.nmax2 >= 4096)
-    return launch_nt<T, MODE, 256>(g, nmaps, F, map_out, map_in, weighted, pix, eo, eo_nm, s);
-  return launch_nt<T, MODE, 128>(g, nmaps, F, map_out, map_in, weighted, pix, eo, eo_nm, s);
+    return launch_nt<T, MODE, 256>(g, nmaps, F, map_out, map_in, weighted, pix, eo, s);
+  return launch_nt<T, MODE, 128>(g, nmaps, F, map_out, map_in, weighted, pix, eo, s);
 }
 
 }  // namespace
@@ -655,30 +656,27 @@ int ringfft_smem_ok(const Grid& g, int prec) {
 int ringfft_synth(const Grid& g, int prec, int nmaps, const void* F, double* map, cudaStream_t s) {
   void* f = const_cast<void*>(F);
   if (prec == CMBWS_FP32X2)
-    return launch<df, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, 0, s);
+    return launch<df, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, s);
   if (!is_f32(prec))
-    return launch<double, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, 0, s);
-  return launch<float, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, 0, s);
+    return launch<double, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, s);
+  return launch<float, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, s);
 }
 
-int ringfft_analysis(const Grid& g, int prec, int nmaps, const double* map, int weighted, void* F,
-                     void* eo, cudaStream_t s) {
+int ringfft_analysis(const Grid& g, int prec, int nmaps, const double* map, int weighted, void* eo,
+                     cudaStream_t s) {
   if (prec == CMBWS_FP32X2)
-    return launch<df, MODE_ANALYSIS>(g, nmaps, F, nullptr, map, weighted, nullptr, eo,
-                                     eo_maps(prec), s);
+    return launch<df, MODE_ANALYSIS>(g, nmaps, nullptr, nullptr, map, weighted, nullptr, eo, s);
   if (!is_f32(prec))
-    return launch<double, MODE_ANALYSIS>(g, nmaps, F, nullptr, map, weighted, nullptr, nullptr, 0, s);
-  return launch<float, MODE_ANALYSIS>(g, nmaps, F, nullptr, map, weighted, nullptr, eo,
-                                      eo_maps(prec), s);
+    return launch<double, MODE_ANALYSIS>(g, nmaps, nullptr, nullptr, map, weighted, nullptr, eo, s);
+  return launch<float, MODE_ANALYSIS>(g, nmaps, nullptr, nullptr, map, weighted, nullptr, eo, s);
 }
 
 int ringfft_fused(const Grid& g, int prec, int nmaps, void* F, const void* const* pix, void* eo,
                   cudaStream_t s) {
   if (prec == CMBWS_FP32X2)
-    return launch<df, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, eo, eo_maps(prec), s);
-  if (!is_f32(prec))
-    return launch<double, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, nullptr, 0, s);
-  return launch<float, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, eo, eo_maps(prec), s);
+    return launch<df, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, eo, s);
+  if (!is_f32(prec)) return launch<double, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, eo, s);
+  return launch<float, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, eo, s);
 }
 
 }  // namespace cmbws

@@ -37,6 +37,7 @@ namespace cmbws {
 namespace {
 
 constexpr double kStartThreshold = 1e-30;
+constexpr double kStartThresholdFx = 0x1p-64;  // fixed-point stages: below their last digit
 constexpr double kShiftUp = 0x1p600;     // 2^600
 constexpr double kShiftDown = 0x1p-600;  // 2^-600
 constexpr double kGrow = 0x1p500;
@@ -141,8 +142,11 @@ __global__ void k_seeds(const double* __restrict__ sinth, const double* __restri
 __global__ void k_start(const double* __restrict__ y, const double* __restrict__ A, int L, int npair,
                         const double* __restrict__ sv, const int* __restrict__ sk,
                         int* __restrict__ ls, double2* __restrict__ st64, float2* __restrict__ st32,
+                        int* __restrict__ lsx, double2* __restrict__ stx,
                         const int64_t* __restrict__ ck_base, float2* __restrict__ ck,
-                        const int64_t* __restrict__ ck64_base, float4* __restrict__ ck64) {
+                        const int64_t* __restrict__ ckx_base, double2* __restrict__ ckx,
+                        const int64_t* __restrict__ ck64_base, float4* __restrict__ ck64,
+                        unsigned* __restrict__ mumax) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (p >= npair) return;
@@ -153,24 +157,38 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
   double v1 = sqrt(2.0 * m + 3.0) * (1.0 - yy) * v0;
   const double* Am = A + lm_off(L, m) - m;  // Am[l] = A_lm
   int l = m;
-  int found = L + 1;
+  int found = L + 1, foundx = L + 1;
+  double x0 = 0.0, x1 = 0.0;
   double o0 = 0.0, o1 = 0.0;
+  unsigned mx = 0;  // high word of the largest |mu_l| from the start on
   const int nck = (L - m + kChunk) / kChunk;
+  const int nckx = (L - m + kFxChunk) / kFxChunk;
   const int nckd = (L - m + kChunkDf) / kChunkDf;
   float2* ckp = ck ? ck + ck_base[m] + (int64_t)p * nck : nullptr;
+  double2* ckq = ckx ? ckx + ckx_base[m] + (int64_t)p * nckx : nullptr;
   float4* ckd = ck64 ? ck64 + ck64_base[m] + (int64_t)p * nckd : nullptr;
   while (l <= L) {
     if (found > L && k == 0 && (fabs(v0) > kStartThreshold || fabs(v1) > kStartThreshold)) {
       found = l;
       o0 = v0;
       o1 = (l + 1 <= L) ? v1 : 0.0;
-      if (!ckp && !ckd) break;
+    }
+    if (foundx > L && k == 0 && (fabs(v0) > kStartThresholdFx || fabs(v1) > kStartThresholdFx)) {
+      foundx = l;
+      x0 = v0;
+      x1 = (l + 1 <= L) ? v1 : 0.0;
+    }
+    if (found <= l) {
+      mx = max(mx, (unsigned)__double2hiint(v0) & 0x7fffffffu);
+      if (l + 1 <= L) mx = max(mx, (unsigned)__double2hiint(v1) & 0x7fffffffu);
     }
     // chunk checkpoints: the recurrence pair at the chunk's first l once the pair has
     // started there, zero before (a pair starting inside the chunk is injected at ls)
     const double w0 = found <= l ? v0 : 0.0;
     const double w1 = (found <= l && l + 1 <= L) ? v1 : 0.0;
     if (ckp && (l - m) % kChunk == 0) ckp[(l - m) / kChunk] = make_float2((float)w0, (float)w1);
+    if (ckq && (l - m) % kFxChunk == 0)
+      ckq[(l - m) / kFxChunk] = foundx <= l ? make_double2(w0, w1) : make_double2(0.0, 0.0);
     if (ckd && (l - m) % kChunkDf == 0) {
       const float h0 = (float)w0, h1 = (float)w1;
       ckd[(l - m) / kChunkDf] = make_float4(h0, (float)(w0 - (double)h0), h1, (float)(w1 - (double)h1));
@@ -187,9 +205,13 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
     }
     l += 2;
   }
+  if (!ls) return;  // checkpoints only
   ls[idx] = found;
+  lsx[idx] = foundx;
+  stx[idx] = make_double2(x0, x1);
   st64[idx] = make_double2(o0, o1);
   st32[idx] = make_float2((float)o0, (float)o1);
+  if (mx) atomicMax(&mumax[m], mx);
 }
 
 template <typename T2, typename T>
@@ -261,6 +283,7 @@ int grid_build_tables(Grid& g) {
   g.npair = (g.nring + 1) / 2;
   std::vector<double> yh(g.npair), sh(g.npair);
   std::vector<float> yf(g.npair);
+  std::vector<uint64_t> xf(g.npair);
   std::vector<int> pr(2 * g.npair), phase(g.npair);
   for (int p = 0; p < g.npair; ++p) {
     const int south = g.nring - 1 - p;
@@ -270,6 +293,9 @@ int grid_build_tables(Grid& g) {
     yh[p] = 2.0 * s2 * s2;
     sh[p] = std::sin(g.theta[p]);
     yf[p] = (float)yh[p];
+    // cos(theta) 2^63 = 2^63 - y 2^63 (0 < y; at most 1 on the north rings and the equator)
+    const uint64_t yq = (uint64_t)std::ldexp(yh[p], 63);
+    xf[p] = yq < (1ull << 63) ? (1ull << 63) - yq : 0;
     const double half = M_PI / g.nphi[p];
     if (g.phi0[p] == 0.0) phase[p] = 0;
     else if (std::fabs(g.phi0[p] - half) < 1e-15) phase[p] = 1;
@@ -280,6 +306,7 @@ int grid_build_tables(Grid& g) {
   }
   CMBWS_TRY(g.y64.upload(yh.data(), yh.size() * 8));
   CMBWS_TRY(g.y32.upload(yf.data(), yf.size() * 4));
+  CMBWS_TRY(g.xfx.upload(xf.data(), xf.size() * 8));
   CMBWS_TRY(g.pair_ring.upload(pr.data(), pr.size() * 4));
   CMBWS_TRY(g.pair_phase.upload(phase.data(), phase.size() * 4));
   CMBWS_TRY(g.ring_off.upload(g.offset.data(), (g.nring + 1) * 8));
@@ -326,23 +353,14 @@ int grid_build_tables(Grid& g) {
     }
     CMBWS_TRY(g.BRS32.upload(brs.data(), nlm * 12));
   }
-  {
-    std::vector<float> A2(2 * nlm);
-    for (int64_t i = 0; i < nlm; ++i) {
-      const float h = (float)A[i];
-      A2[2 * i] = h;
-      A2[2 * i + 1] = (float)(A[i] - (double)h);
-    }
-    CMBWS_TRY(g.A2f.upload(A2.data(), nlm * 8));
-  }
   CMBWS_TRY(g.c64.upload(c.data(), nlm * 8));
 
   // ---- start values ----
   {
     std::vector<double> fmm(L + 1, 0.0);
     for (int m = 1; m <= L; ++m) fmm[m] = std::sqrt((2.0 * m + 1.0) / (2.0 * m));
-    g.fmm_h = fmm;
     DevMem d_fmm, d_sin, d_sv, d_sk;
+    g.fmm_h = fmm;
     CMBWS_TRY(d_fmm.upload(fmm.data(), fmm.size() * 8));
     CMBWS_TRY(d_sin.upload(sh.data(), sh.size() * 8));
     const int64_t nst = (int64_t)(L + 1) * g.npair;
@@ -350,6 +368,8 @@ int grid_build_tables(Grid& g) {
     CMBWS_TRY(d_sk.alloc(nst * 4));
     CMBWS_TRY(g.ls.alloc(nst * 4));
     CMBWS_TRY(g.st64.alloc(nst * 16));
+    CMBWS_TRY(g.lsx.alloc(nst * 4));
+    CMBWS_TRY(g.stx.alloc(nst * 16));
     CMBWS_TRY(g.st32.alloc(nst * 8));
     k_seeds<<<(g.npair + 127) / 128, 128>>>(d_sin.as<double>(), d_fmm.as<double>(), L, g.npair,
                                             d_sv.as<double>(), d_sk.as<int>());
@@ -369,9 +389,20 @@ int grid_build_tables(Grid& g) {
       g.nwt32 = (int)wt.size();
     }
     CMBWS_TRY(g.ck32.alloc((size_t)tot * 8));
+    int64_t totx = 0;
+    for (int m = 0; m <= L; ++m) {
+      cb[m] = totx;
+      totx += (int64_t)g.npair * ((L - m + kFxChunk) / kFxChunk);
+    }
+    CMBWS_TRY(g.ckx_base.upload(cb.data(), (L + 1) * 8));
+    CMBWS_TRY(g.ckx.alloc((size_t)totx * 16));
+    CMBWS_TRY(g.mumax.alloc((size_t)(L + 1) * 4));
+    CMBWS_CUDA(cudaMemset(g.mumax.p, 0, (size_t)(L + 1) * 4));
     k_start<<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
                           d_sk.as<int>(), g.ls.as<int>(), g.st64.as<double2>(), g.st32.as<float2>(),
-                          g.ck_base.as<int64_t>(), g.ck32.as<float2>(), nullptr, nullptr);
+                          g.lsx.as<int>(), g.stx.as<double2>(),
+                          g.ck_base.as<int64_t>(), g.ck32.as<float2>(), g.ckx_base.as<int64_t>(),
+                          g.ckx.as<double2>(), nullptr, nullptr, g.mumax.as<unsigned>());
     CMBWS_LAUNCH_CHECK();
     const int ntile = (g.npair + kTileMinPT - 1) / kTileMinPT;
     CMBWS_TRY(g.ls_tmin.alloc((size_t)(L + 1) * ntile * 4));
@@ -460,8 +491,8 @@ int grid_build_tables(Grid& g) {
   return CMBWS_OK;
 }
 
-__global__ void k_to_df(const double* __restrict__ v, float2* __restrict__ o, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_to_df(const double* __restrict__ v, float2* __restrict__ o, int64_t n) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float h = (float)v[i];
   o[i] = make_float2(h, (float)(v[i] - (double)h));
@@ -481,6 +512,7 @@ int grid_ensure_ck64(const Grid& gc) {
   if (gc.ck64.p) return CMBWS_OK;
   Grid& g = const_cast<Grid&>(gc);  // tables only; the geometry is not touched
   const int L = g.lmax;
+  const int64_t nlm = nlm_of(L);
   std::vector<int64_t> cb(L + 1, 0);
   int64_t tot = 0;
   for (int m = 0; m <= L; ++m) {
@@ -489,7 +521,7 @@ int grid_ensure_ck64(const Grid& gc) {
   }
   DevMem cbd;
   CMBWS_TRY(cbd.upload(cb.data(), (L + 1) * 8));
-  DevMem d_fmm, d_sin, d_sv, d_sk, ls_t, st64_t, st32_t;
+  DevMem d_fmm, d_sin, d_sv, d_sk;
   std::vector<double> sh(g.npair);
   for (int p = 0; p < g.npair; ++p) sh[p] = std::sin(g.theta[p]);
   CMBWS_TRY(d_fmm.upload(g.fmm_h.data(), g.fmm_h.size() * 8));
@@ -497,21 +529,21 @@ int grid_ensure_ck64(const Grid& gc) {
   const int64_t nst = (int64_t)(L + 1) * g.npair;
   CMBWS_TRY(d_sv.alloc(nst * 8));
   CMBWS_TRY(d_sk.alloc(nst * 4));
-  CMBWS_TRY(ls_t.alloc(nst * 4));
-  CMBWS_TRY(st64_t.alloc(nst * 16));
-  CMBWS_TRY(st32_t.alloc(nst * 8));
-  DevMem ck, y2;
+  DevMem ck, y2, A2;
   CMBWS_TRY(ck.alloc((size_t)tot * 16));
   CMBWS_TRY(y2.alloc((size_t)g.npair * 8));
+  CMBWS_TRY(A2.alloc((size_t)nlm * 8));
   k_to_df<<<(g.npair + 127) / 128, 128>>>(g.y64.as<double>(), y2.as<float2>(), g.npair);
+  CMBWS_LAUNCH_CHECK();
+  k_to_df<<<(unsigned)((nlm + 127) / 128), 128>>>(g.A64.as<double>(), A2.as<float2>(), nlm);
   CMBWS_LAUNCH_CHECK();
   k_seeds<<<(g.npair + 127) / 128, 128>>>(d_sin.as<double>(), d_fmm.as<double>(), L, g.npair,
                                           d_sv.as<double>(), d_sk.as<int>());
   CMBWS_LAUNCH_CHECK();
   dim3 grd((g.npair + 127) / 128, L + 1);
   k_start<<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
-                        d_sk.as<int>(), ls_t.as<int>(), st64_t.as<double2>(), st32_t.as<float2>(),
-                        g.ck_base.as<int64_t>(), nullptr, cbd.as<int64_t>(), ck.as<float4>());
+                        d_sk.as<int>(), nullptr, nullptr, nullptr, nullptr, nullptr, g.ck_base.as<int64_t>(),
+                        nullptr, nullptr, nullptr, cbd.as<int64_t>(), ck.as<float4>(), nullptr);
   CMBWS_LAUNCH_CHECK();
   CMBWS_CUDA(cudaDeviceSynchronize());
   {
@@ -522,6 +554,7 @@ int grid_ensure_ck64(const Grid& gc) {
     g.nwtdf = (int)wt.size();
   }
   g.y2f = std::move(y2);
+  g.A2f = std::move(A2);
   g.ck64_base = std::move(cbd);
   g.ck64 = std::move(ck);
   return CMBWS_OK;

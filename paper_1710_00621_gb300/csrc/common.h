@@ -144,7 +144,7 @@ struct FftPlan {
   int n;          // ring length
   int n2;         // power-of-two transform size (n itself, or the Bluestein size)
   int bluestein;  // 1 if n is not a power of two
-  int pad;
+  int fexp;       // Bluestein: the filter's scale in fftfx (stored times 2^(61 - fexp))
   int64_t chirp;  // offset (complex entries) of b_t = exp(i pi t^2 / n), t < n
   int64_t filt;   // offset of the Bluestein filter spectrum (n2 entries, includes 1/n2,
                   // bit-reversed order)
@@ -205,9 +205,10 @@ struct Grid {
   // ring FFT tables (device)
   std::vector<FftPlan> plans;
   DevMem plans_d;
-  DevMem fft64, fft32;    // complex tables: chirps, filters, phases, twiddles
+  DevMem fft32;           // complex tables: chirps, filters, phases, twiddles (float2)
   DevMem fftdf;           // the same as double-float pairs (float4 per entry)
-  int64_t tw_off = 0;     // offset of exp(-2 pi i k / nmax2), k < nmax2 / 2
+  DevMem fftfx;           // the same in fixed point: digits of the parts times 2^61 (int4, ringfft_fx.cu)
+  int64_t tw_off = 0;     // offset of exp(-2 pi i k / nmax2), k < nmax2
   int nmax2 = 1;          // largest power-of-two transform size
   int max_n = 1;
 
@@ -245,6 +246,11 @@ int ringfft_analysis(const Grid& g, int prec, int nmaps, const double* map, int 
 // F -> pixels -> * pix[map] -> adjoint input eo.  pix: [nmaps] device pointers (prec type) of npix.
 int ringfft_fused(const Grid& g, int prec, int nmaps, void* F, const void* const* pix, void* eo,
                   cudaStream_t s);
+// the FP64 forms (ringfft_fx.cu); their spectra carry no sqrt(2) factors (applied by legendre_fx.cu)
+int ringfft_fx_synth(const Grid& g, int nmaps, const void* F, double* map, cudaStream_t s);
+int ringfft_fx_analysis(const Grid& g, int nmaps, const double* map, int weighted, void* eo, cudaStream_t s);
+int ringfft_fx_fused(const Grid& g, int nmaps, const void* F, const void* const* pix, void* eo,
+                     cudaStream_t s);
 int ringfft_smem_ok(const Grid& g, int prec);
 
 // warp-task list {m, first chunk} for chunks of `chunk` values of l (adjoint scheduling)

@@ -325,6 +325,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
       const int ea = (int)s_emax[q >> 1] - 1022;
       v[q] = acc[q].value((fx_t)s_corr[2 * (8 * chain + q)], (fx_t)s_corr[2 * (8 * chain + q) + 1], ea - S - 6);
       // a map with a non-finite coefficient, and a timed-out wait, give NaN
+      if (m > 0) v[q] *= 0.70710678118654752440;  // the ring FFT's 1 / sqrt(2)
       if ((ea >= 1025 && ls <= L) || failed) v[q] = fx_nan();
       if (chain) s_odd[q * kM + row] = v[q];
     }
@@ -642,7 +643,8 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
   const int l = lb0 + (tid & (kM - 1));  // row of D
   if (l > L) return;
   const fxu_t* corr = s_corr + 16 * (tid & 1) + 2 * grp;
-  const double cc = (tid & 2) ? -c64[lmo + l] : c64[lmo + l];  // sigma of l
+  // sigma of l, and the ring FFT's sqrt(2)
+  const double cc = ((tid & 2) ? -c64[lmo + l] : c64[lmo + l]) * (m > 0 ? 1.41421356237309504880 : 1.0);
   double* o = reinterpret_cast<double*>(out + lmo + l) + grp;
 #pragma unroll
   for (int q = 0; q < NM; ++q) {

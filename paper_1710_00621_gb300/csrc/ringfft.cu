@@ -22,8 +22,8 @@
 // The fused mode goes synthesis -> pixel multiply -> analysis without the
 // pixel map leaving shared memory.
 //
-// Arithmetic: FP32, FP64, or double-float (df, CMBWS_FP32X2: FP64-accurate on the
-// FP32 pipe, whose rate is 61 times the FP64 one on GB300).  The double-float
+// Arithmetic: FP32, or double-float (df, CMBWS_FP32X2: FP64-accurate on the FP32 pipe, whose
+// rate is 61 times the FP64 one on GB300); FP64 transforms run in fixed point (ringfft_fx.cu).  The double-float
 // transform reads and writes double-float ring spectra (the layout of the
 // double-float Legendre stage), so FP64 conversions happen only at the pixels.
 #include <type_traits>
@@ -36,7 +36,6 @@ namespace cmbws {
 namespace {
 
 template <typename T> struct V2;
-template <> struct V2<double> { using t = double2; };
 template <> struct V2<float> { using t = float2; };
 template <> struct V2<df> { using t = df2; };
 // storage type of pixel factors and ring weights
@@ -52,7 +51,6 @@ __device__ __forceinline__ T2 cmul(T2 a, T2 b) {
 }
 // a product rounded by itself (never contracted with a following addition)
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ df mul_rn(df a, df b) { return a * b; }
 
 template <typename T2>
@@ -122,9 +120,8 @@ __device__ __forceinline__ T2 unit_root(int c, int e) {
 
 // Twiddles of a group: at one stage they are w0 exp(-2 pi i c / 2^(t+1)), c < 2^t, with w0 the
 // twiddle of the group's first butterfly.  In FP32 one table read per stage then serves the
-// group (the other factors are compile-time roots of unity, one complex multiply each); FP64
-// multiplies run at a 64th of that rate and a double-float complex multiply costs ~50 FP32
-// operations, so those read every twiddle from the table.
+// group (the other factors are compile-time roots of unity, one complex multiply each); a
+// double-float complex multiply costs ~50 FP32 operations, so there every twiddle is read.
 template <typename T2>
 __device__ __forceinline__ T2 group_twiddle(const T2* __restrict__ tw, int pos0, int step, int stride,
                                             const T2& w0, int c, int e) {
@@ -295,7 +292,7 @@ struct PixPtrs {
 
 // NT threads per CTA; the register cap keeps three CTAs of 256 threads (six of 128) resident
 // per SM in FP32 and double-float, which is what the transform buffer of the largest rings
-// allows (double-float and FP64 grids with 8192-entry buffers: one CTA of 512).
+// allows (double-float grids with 8192-entry buffers: one CTA of 512).
 //
 // Each ring pair's DFTs, in terms of the plan (n pixels; Bluestein plans convolve over n2):
 // * power of two: the inverse DFT is a DIT transform whose input (the folded spectrum) is
@@ -309,13 +306,8 @@ struct PixPtrs {
 // In the fused mode the pixel multiply and the chirp of the next transform happen in the last
 // pass of the inverse; in the synthesis mode that pass writes the pixel maps, and in the
 // analysis mode the first pass of the forward DFT reads them.
-// FP64 gets twice the register budget (two CTAs of 256 threads): under the FP32 cap its
-// transform spilled.
-template <typename T>
-constexpr int fft_min_blocks(int nt) { return (std::is_same<T, double>::value ? 512 : 768) / nt; }
-
 template <typename T, int MODE, int NT>
-__global__ void __launch_bounds__(NT, fft_min_blocks<T>(NT))
+__global__ void __launch_bounds__(NT, 768 / NT)
 k_ringfft(typename V2<T>::t* __restrict__ F, int64_t F_stride, double* __restrict__ map_out,
           const double* __restrict__ map_in, int64_t npix,
           const typename PixT<T>::t* __restrict__ ring_w, PixPtrs<typename PixT<T>::t> pix,
@@ -604,11 +596,11 @@ int launch_nt(const Grid& g, int nmaps, void* F, double* map_out, const double* 
   CMBWS_TRY(ensure_dyn_smem((const void*)kern, sm));
   using TP = typename PixT<T>::t;
   const int64_t fs = (int64_t)g.nring * (g.lmax + 1);
-  constexpr bool f32 = std::is_same<T, float>::value, f64 = std::is_same<T, double>::value;
+  constexpr bool f32 = std::is_same<T, float>::value;
   const TP* rw = nullptr;
   if (MODE == MODE_ANALYSIS && weighted) rw = f32 ? (const TP*)g.ring_w32.p : (const TP*)g.ring_w64.p;
-  const int prec = f32 ? CMBWS_FP32 : f64 ? CMBWS_FP64 : CMBWS_FP32X2;
-  const T2* tab = f32 ? (const T2*)g.fft32.p : f64 ? (const T2*)g.fft64.p : (const T2*)g.fftdf.p;
+  const int prec = f32 ? CMBWS_FP32 : CMBWS_FP32X2;
+  const T2* tab = f32 ? (const T2*)g.fft32.p : (const T2*)g.fftdf.p;
   for (int k0 = 0; k0 < nmaps; k0 += kMaxPix) {
     const int nm = nmaps - k0 < kMaxPix ? nmaps - k0 : kMaxPix;
     PixPtrs<TP> pp{};
@@ -619,7 +611,7 @@ int launch_nt(const Grid& g, int nmaps, void* F, double* map_out, const double* 
     // FP64 maps (synthesis output, analysis input) once
     const double fb = (double)g.nring * (g.lmax + 1) * sizeof(T2);
     const double pb = (double)g.npix * (MODE == MODE_FUSED ? sizeof(TP) : sizeof(double));
-    ProfScope ps(PROF_FFT, s, f32 ? 0 : f64 ? 1 : 2,
+    ProfScope ps(PROF_FFT, s, f32 ? 0 : 2,
                  byte_work(nm * ((MODE == MODE_FUSED ? 2.0 : 1.0) * fb + pb)));
     kern<<<grd, NT, sm, s>>>((T2*)F + k0 * fs, fs, map_out ? map_out + k0 * g.npix : nullptr,
                               map_in ? map_in + k0 * g.npix : nullptr, g.npix, rw, pp,
@@ -634,7 +626,7 @@ int launch_nt(const Grid& g, int nmaps, void* F, double* map_out, const double* 
 template <typename T, int MODE>
 int launch(const Grid& g, int nmaps, void* F, double* map_out, const double* map_in, int weighted,
            const void* const* pix, void* eo, cudaStream_t s) {
-  // 16-byte values (double-float, FP64) with 8192-entry buffers: about 140 KB per CTA, one CTA
+  // 16-byte values (double-float) with 8192-entry buffers: about 140 KB per CTA, one CTA
   // per SM, so that CTA gets 512 threads (16 warps instead of 8)
   if constexpr (!std::is_same<T, float>::value)
     if (g.nmax2 >= 8192)
@@ -647,7 +639,7 @@ int launch(const Grid& g, int nmaps, void* F, double* map_out, const double* map
 }  // namespace
 
 int ringfft_smem_ok(const Grid& g, int prec) {
-  const size_t sm = !is_f32(prec) ? smem_bytes<double>(g) : smem_bytes<float>(g);
+  const size_t sm = !is_f32(prec) ? smem_bytes<df>(g) : smem_bytes<float>(g);
   return sm <= 227 * 1024;
 }
 
@@ -657,8 +649,7 @@ int ringfft_synth(const Grid& g, int prec, int nmaps, const void* F, double* map
   void* f = const_cast<void*>(F);
   if (prec == CMBWS_FP32X2)
     return launch<df, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, s);
-  if (!is_f32(prec))
-    return launch<double, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, s);
+  if (!is_f32(prec)) return ringfft_fx_synth(g, nmaps, F, map, s);
   return launch<float, MODE_SYNTH>(g, nmaps, f, map, nullptr, 0, nullptr, nullptr, s);
 }
 
@@ -666,8 +657,7 @@ int ringfft_analysis(const Grid& g, int prec, int nmaps, const double* map, int 
                      cudaStream_t s) {
   if (prec == CMBWS_FP32X2)
     return launch<df, MODE_ANALYSIS>(g, nmaps, nullptr, nullptr, map, weighted, nullptr, eo, s);
-  if (!is_f32(prec))
-    return launch<double, MODE_ANALYSIS>(g, nmaps, nullptr, nullptr, map, weighted, nullptr, eo, s);
+  if (!is_f32(prec)) return ringfft_fx_analysis(g, nmaps, map, weighted, eo, s);
   return launch<float, MODE_ANALYSIS>(g, nmaps, nullptr, nullptr, map, weighted, nullptr, eo, s);
 }
 
@@ -675,7 +665,7 @@ int ringfft_fused(const Grid& g, int prec, int nmaps, void* F, const void* const
                   cudaStream_t s) {
   if (prec == CMBWS_FP32X2)
     return launch<df, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, eo, s);
-  if (!is_f32(prec)) return launch<double, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, eo, s);
+  if (!is_f32(prec)) return ringfft_fx_fused(g, nmaps, F, pix, eo, s);
   return launch<float, MODE_FUSED>(g, nmaps, F, nullptr, nullptr, 0, pix, eo, s);
 }
 

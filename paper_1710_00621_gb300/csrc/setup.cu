@@ -24,6 +24,7 @@
 // start of every chunk of kChunk = 8 values of l ([m][pair][chunk], FP32; about
 // npair (L+1)^2 / 16 x 8 bytes: 9.7 GB at Nside 1024, L = 3071), so that the adjoint can
 // restart the recurrence of any pair at any chunk without a serial walk along l.
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <complex>
@@ -139,6 +140,9 @@ __global__ void k_seeds(const double* __restrict__ sinth, const double* __restri
   }
 }
 
+// PLAN: starts, largest values and the checkpoints of the FP32 and fixed-point adjoints; otherwise
+// the double-float checkpoints only
+template <bool PLAN>
 __global__ void k_start(const double* __restrict__ y, const double* __restrict__ A, int L, int npair,
                         const double* __restrict__ sv, const int* __restrict__ sk,
                         int* __restrict__ ls, double2* __restrict__ st64, float2* __restrict__ st32,
@@ -164,21 +168,21 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
   const int nck = (L - m + kChunk) / kChunk;
   const int nckx = (L - m + kFxChunk) / kFxChunk;
   const int nckd = (L - m + kChunkDf) / kChunkDf;
-  float2* ckp = ck ? ck + ck_base[m] + (int64_t)p * nck : nullptr;
-  double2* ckq = ckx ? ckx + ckx_base[m] + (int64_t)p * nckx : nullptr;
-  float4* ckd = ck64 ? ck64 + ck64_base[m] + (int64_t)p * nckd : nullptr;
+  float2* ckp = PLAN ? ck + ck_base[m] + (int64_t)p * nck : nullptr;
+  double2* ckq = PLAN ? ckx + ckx_base[m] + (int64_t)p * nckx : nullptr;
+  float4* ckd = PLAN ? nullptr : ck64 + ck64_base[m] + (int64_t)p * nckd;
   while (l <= L) {
     if (found > L && k == 0 && (fabs(v0) > kStartThreshold || fabs(v1) > kStartThreshold)) {
       found = l;
       o0 = v0;
       o1 = (l + 1 <= L) ? v1 : 0.0;
     }
-    if (foundx > L && k == 0 && (fabs(v0) > kStartThresholdFx || fabs(v1) > kStartThresholdFx)) {
+    if (PLAN && foundx > L && k == 0 && (fabs(v0) > kStartThresholdFx || fabs(v1) > kStartThresholdFx)) {
       foundx = l;
       x0 = v0;
       x1 = (l + 1 <= L) ? v1 : 0.0;
     }
-    if (found <= l) {
+    if (PLAN && found <= l) {
       mx = max(mx, (unsigned)__double2hiint(v0) & 0x7fffffffu);
       if (l + 1 <= L) mx = max(mx, (unsigned)__double2hiint(v1) & 0x7fffffffu);
     }
@@ -186,10 +190,10 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
     // started there, zero before (a pair starting inside the chunk is injected at ls)
     const double w0 = found <= l ? v0 : 0.0;
     const double w1 = (found <= l && l + 1 <= L) ? v1 : 0.0;
-    if (ckp && (l - m) % kChunk == 0) ckp[(l - m) / kChunk] = make_float2((float)w0, (float)w1);
-    if (ckq && (l - m) % kFxChunk == 0)
+    if (PLAN && (l - m) % kChunk == 0) ckp[(l - m) / kChunk] = make_float2((float)w0, (float)w1);
+    if (PLAN && (l - m) % kFxChunk == 0)
       ckq[(l - m) / kFxChunk] = foundx <= l ? make_double2(w0, w1) : make_double2(0.0, 0.0);
-    if (ckd && (l - m) % kChunkDf == 0) {
+    if (!PLAN && (l - m) % kChunkDf == 0) {
       const float h0 = (float)w0, h1 = (float)w1;
       ckd[(l - m) / kChunkDf] = make_float4(h0, (float)(w0 - (double)h0), h1, (float)(w1 - (double)h1));
     }
@@ -205,7 +209,7 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
     }
     l += 2;
   }
-  if (!ls) return;  // checkpoints only
+  if (!PLAN) return;
   ls[idx] = found;
   lsx[idx] = foundx;
   stx[idx] = make_double2(x0, x1);
@@ -252,6 +256,26 @@ __global__ void k_tile_min(const int* __restrict__ ls, int npair, int ntile, int
   const int p1 = min(npair, (t + 1) * kTileMinPT);
   for (int p = t * kTileMinPT; p < p1; ++p) v = min(v, ls[(int64_t)m * npair + p]);
   tmin[(int64_t)m * ntile + t] = v;
+}
+
+// Digits of v 2^k: upper, and lower of 31 bits balanced.
+__device__ __forceinline__ int2 fx_factor(double v, int k) {
+  const long long w = __double2ll_rn(scalbn(v, k));
+  const int h = (int)((w + (1ll << 30)) >> 31);
+  return make_int2(h, (int)(w - ((long long)h << 31)));
+}
+
+// FFT table entries as FP32, double-float and fixed point (times 2^sc)
+__global__ void k_fft_tables(const double2* __restrict__ t, const signed char* __restrict__ sc, int64_t n,
+                             float2* __restrict__ f32, float4* __restrict__ dfl, int4* __restrict__ fx) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double2 v = t[i];
+  const float2 h = make_float2((float)v.x, (float)v.y);
+  f32[i] = h;
+  dfl[i] = make_float4(h.x, (float)(v.x - (double)h.x), h.y, (float)(v.y - (double)h.y));
+  const int2 a = fx_factor(v.x, sc[i]), b = fx_factor(v.y, sc[i]);
+  fx[i] = make_int4(a.x, a.y, b.x, b.y);
 }
 
 }  // namespace
@@ -398,7 +422,7 @@ int grid_build_tables(Grid& g) {
     CMBWS_TRY(g.ckx.alloc((size_t)totx * 16));
     CMBWS_TRY(g.mumax.alloc((size_t)(L + 1) * 4));
     CMBWS_CUDA(cudaMemset(g.mumax.p, 0, (size_t)(L + 1) * 4));
-    k_start<<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
+    k_start<true><<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
                           d_sk.as<int>(), g.ls.as<int>(), g.st64.as<double2>(), g.st32.as<float2>(),
                           g.lsx.as<int>(), g.stx.as<double2>(),
                           g.ck_base.as<int64_t>(), g.ck32.as<float2>(), g.ckx_base.as<int64_t>(),
@@ -420,6 +444,7 @@ int grid_build_tables(Grid& g) {
     g.max_n = 1;
     g.nmax2 = 2;
     std::vector<std::complex<double>> tab;
+    std::vector<signed char> sc;  // binary scale of the fixed-point form of each entry
     auto plan_for = [&](int n) -> int {
       for (size_t i = 0; i < g.plans.size(); ++i)
         if (g.plans[i].n == n) return (int)i;
@@ -445,6 +470,11 @@ int grid_build_tables(Grid& g) {
         P.filt = (int64_t)tab.size();
         int lg2 = 0;
         while ((1 << lg2) < P.n2) ++lg2;
+        double big = 0.0;
+        for (int q = 0; q < P.n2; ++q) big = std::max(big, std::abs(v[q]) / (double)P.n2);
+        std::frexp(big, &P.fexp);  // |filter| < 2^fexp
+        sc.resize(tab.size(), 61);
+        sc.resize(tab.size() + P.n2, (signed char)(61 - P.fexp));
         for (int q = 0; q < P.n2; ++q) {
           int j = 0;
           for (int b = 0; b < lg2; ++b) j |= ((q >> b) & 1) << (lg2 - 1 - b);
@@ -465,26 +495,23 @@ int grid_build_tables(Grid& g) {
     };
     for (int p = 0; p < g.npair; ++p) pplan[p] = plan_for(g.nphi[p]);
     g.tw_off = (int64_t)tab.size();
-    for (int k = 0; k < g.nmax2 / 2; ++k) {
+    for (int k = 0; k < g.nmax2; ++k) {
       const double ang = -2.0 * M_PI * k / g.nmax2;
       tab.emplace_back(std::cos(ang), std::sin(ang));
     }
-    std::vector<float> tf(2 * tab.size());
-    for (size_t i = 0; i < tab.size(); ++i) {
-      tf[2 * i] = (float)tab[i].real();
-      tf[2 * i + 1] = (float)tab[i].imag();
-    }
-    std::vector<float> td(4 * tab.size());  // (re hi, re lo, im hi, im lo)
-    for (size_t i = 0; i < tab.size(); ++i) {
-      const double re = tab[i].real(), im = tab[i].imag();
-      td[4 * i] = (float)re;
-      td[4 * i + 1] = (float)(re - (double)(float)re);
-      td[4 * i + 2] = (float)im;
-      td[4 * i + 3] = (float)(im - (double)(float)im);
-    }
-    CMBWS_TRY(g.fft64.upload(tab.data(), tab.size() * 16));
-    CMBWS_TRY(g.fft32.upload(tf.data(), tf.size() * 4));
-    CMBWS_TRY(g.fftdf.upload(td.data(), td.size() * 4));
+    sc.resize(tab.size(), 61);
+    // the tables of every arithmetic from the FP64 values, on the device
+    DevMem t64, dsc;
+    CMBWS_TRY(t64.upload(tab.data(), tab.size() * 16));
+    CMBWS_TRY(dsc.upload(sc.data(), sc.size()));
+    CMBWS_TRY(g.fft32.alloc(tab.size() * 8));
+    CMBWS_TRY(g.fftdf.alloc(tab.size() * 16));
+    CMBWS_TRY(g.fftfx.alloc(tab.size() * 16));
+    k_fft_tables<<<(unsigned)((tab.size() + 255) / 256), 256>>>(
+        t64.as<double2>(), dsc.as<signed char>(), (int64_t)tab.size(), g.fft32.as<float2>(),
+        g.fftdf.as<float4>(), g.fftfx.as<int4>());
+    CMBWS_LAUNCH_CHECK();
+    CMBWS_CUDA(cudaDeviceSynchronize());
     CMBWS_TRY(g.plans_d.upload(g.plans.data(), g.plans.size() * sizeof(FftPlan)));
     CMBWS_TRY(g.pair_plan.upload(pplan.data(), pplan.size() * 4));
   }
@@ -541,7 +568,7 @@ int grid_ensure_ck64(const Grid& gc) {
                                           d_sv.as<double>(), d_sk.as<int>());
   CMBWS_LAUNCH_CHECK();
   dim3 grd((g.npair + 127) / 128, L + 1);
-  k_start<<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
+  k_start<false><<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
                         d_sk.as<int>(), nullptr, nullptr, nullptr, nullptr, nullptr, g.ck_base.as<int64_t>(),
                         nullptr, nullptr, nullptr, cbd.as<int64_t>(), ck.as<float4>(), nullptr);
   CMBWS_LAUNCH_CHECK();

@@ -67,3 +67,33 @@ def test_not_finite_stays_in_its_map(bad):
     r, o = to_host(ra), to_host(oa)
     assert not np.isfinite(o[2]).any()
     assert np.array_equal(o[:2], r[:2])
+
+
+# rings of 4..4 nside pixels: one to four thousand points, powers of two and Bluestein plans
+@pytest.mark.parametrize("nside,lmax,maps", [(1, 3, 1), (2, 12, 2), (24, 71, 1), (96, 100, 1)])
+def test_ring_lengths(nside, lmax, maps):
+    g = cw.cmbws_plan_grid(cw.CMBWS_GRID_HEALPIX, nside, lmax)
+    o = og.healpix(nside)
+    rng = np.random.default_rng(nside)
+    ell = np.concatenate([np.arange(lmax + 1)] + [np.arange(m, lmax + 1) for m in range(1, lmax + 1)
+                                                  for _ in range(2)])
+    # a steep spectrum: the ring spectra's first entries dominate the others
+    alm = rng.standard_normal((maps, (lmax + 1) ** 2)) * (1.0 + ell) ** -3.0
+    out = to_dev(np.zeros((maps, g.npix)))
+    cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(alm), out, maps)
+    f = rng.standard_normal((maps, g.npix))
+    back = to_dev(np.zeros((maps, (lmax + 1) ** 2)))
+    cw.cmbws_sht_analysis(g, cw.CMBWS_FP64, to_dev(f), back, maps, 1)
+    m, a = to_host(out), to_host(back)
+    for k in range(maps):
+        assert rel_err(m[k], osht.synthesis(o, lmax, alm[k])) < _tol(lmax)
+        assert rel_err(a[k], osht.adjoint(o, lmax, f[k], weighted=True)) < _tol(lmax)
+
+
+def test_zero_input():
+    g = cw.cmbws_plan_grid(cw.CMBWS_GRID_HEALPIX, 8, 23)
+    out = to_dev(np.ones(g.npix))
+    cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(np.zeros(24 ** 2)), out, 1)
+    back = to_dev(np.ones(24 ** 2))
+    cw.cmbws_sht_analysis(g, cw.CMBWS_FP64, to_dev(np.zeros(g.npix)), back, 1, 1)
+    assert not to_host(out).any() and not to_host(back).any()

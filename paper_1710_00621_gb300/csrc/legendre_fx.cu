@@ -3,12 +3,15 @@
 // exact sums.  The arithmetic, its digits and their error are described in fixed.h.
 //
 // Both stages are products with Lambda[pair][l] = mu_l(theta_pair) (Sec. 2.1):
-//   synthesis   D[pair][col] = sum_l Lambda[pair][l] B[l][col], col = parity(l - m) 8 + part;
-//   adjoint     D[l][col] = sum_pairs Lambda[pair][l] B[pair][col], col = h 8 + part, h = 0 the
-//               even part (north + south) and h = 1 the odd one; row l reads its own parity.
-// The 7 digits of Lambda are the A operand (shared memory, one tile per digit), those of the
-// coefficients or ring parts the B operand (7 x 16 rows); digit i of A times the digits
-// 0..7 - i of B accumulate into columns 16 i.. of the accumulator, so that block s of 16 columns
+//   synthesis   D[pair][col] = sum_l Lambda[pair][l] B[l][col], col = parity(l - m) W + part;
+//   adjoint     D[l][col] = sum_pairs Lambda[pair][l] B[pair][col], col = h W + part, h = 0 the
+//               even part (north + south) and h = 1 the odd one; row l reads its own parity.  The
+//               real parts of all maps come first: a warp takes either them or the imaginary ones
+//               (half the columns to read, no spills: one map at L = 1000 917 -> 836 us with the FFT).
+// W is 8 (up to 4 maps) or 16 (up to 8 maps): the recurrence, which is most of the work, serves all
+// of them.  The 7 digits of Lambda are the A operand (shared memory, one tile per digit), those of
+// the coefficients or ring parts the B operand (7 x 2 W rows); digit i of A times the digits
+// 0..7 - i of B accumulate into columns 2 W i.. of the accumulator, so that block s of 2 W columns
 // holds the sum over i + j = s.  Every 64 terms the blocks are read from tensor memory and added
 // as integers.
 #include <climits>
@@ -24,15 +27,27 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kM = 128;              // MMA rows: ring pairs (synthesis) or values of l (adjoint)
 constexpr int kNT = 2 * kM;          // threads per CTA: two per row
-constexpr int kBStep = kFxDig * 512;  // one K step of B: 7 digits of 16 rows x 16 halves
-constexpr uint32_t kCols = kFxBlk * 16;  // accumulator columns
+
+// Column layout for up to NM maps.  Up to 4 maps have an instance each; 5 and 6 maps share one, 7 and 8
+// another.  Eight columns per parity up to 4 maps keep three CTAs on an SM, which the recurrence's
+// latency needs; 16 columns for 5 to 8 maps give up one of them for half the recurrences.  Against
+// launches of 4 maps: analysis of 5 maps at L = 131 88 -> 60 us, an apply of A on 5 GL grids at
+// L = 511 969 -> 810 us, one on grids of 9 maps at L = 297 1114 -> 902 us.
+template <int NM>
+struct Cols {
+  static constexpr int W = NM <= 4 ? 8 : 16;           // columns per parity
+  static constexpr int kDig = 2 * W * 32;              // bytes of one digit of B: 2 W rows x 16 halves
+  static constexpr int kBStep = kFxDig * kDig;         // one K step of B
+  static constexpr uint32_t kTmem = kFxBlk * 2 * W;    // accumulator columns
+  static constexpr int kCtas = NM <= 4 ? 3 : 2;        // CTAs per SM (256 columns: two)
+};
 
 __device__ unsigned int g_fx_status = 0;  // bit 0: a bounded mbarrier wait ran out
 
-// kind::f16, FP16 A and B, FP32 D, M = 128, N = 16 nb; A K-major or MN-major, B K-major
-__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t adesc, uint64_t bdesc, int nb, bool mn,
+// kind::f16, FP16 A and B, FP32 D, M = 128, N = ncol; A K-major or MN-major, B K-major
+__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t adesc, uint64_t bdesc, int ncol, bool mn,
                                         uint32_t acc) {
-  const uint32_t idesc = (1u << 4) | (mn ? 1u << 15 : 0u) | ((uint32_t)(2 * nb) << 17) | (8u << 24);
+  const uint32_t idesc = (1u << 4) | (mn ? 1u << 15 : 0u) | ((uint32_t)(ncol >> 3) << 17) | (8u << 24);
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
@@ -41,30 +56,40 @@ __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t adesc, uint64_t bde
 }
 // One K step: digit i of A (tiles atile bytes apart) times the digits 0..7 - i of B into blocks
 // i..7; `first` clears the accumulator (digit 1 writes blocks 1..7, digit 0 block 0).
+template <typename C>
 __device__ __forceinline__ void mma_step(uint32_t d, uint32_t ab, int atile, uint32_t alb, uint32_t asb,
                                          uint32_t bb, bool mn, bool first) {
+  constexpr int N = 2 * C::W;
   const uint64_t a0 = smem_desc(ab, alb, asb), a1 = smem_desc(ab + atile, alb, asb);
   const uint64_t b0 = smem_desc(bb, 128, 256);
-  mma_f16(d + 16, a1, b0, kFxDig, mn, first ? 0u : 1u);
+  mma_f16(d + N, a1, b0, N * kFxDig, mn, first ? 0u : 1u);
   if (first) {
-    mma_f16(d, a0, b0, 1, mn, 0u);
-    mma_f16(d + 16, a0, smem_desc(bb + 512, 128, 256), kFxDig - 1, mn, 1u);
+    mma_f16(d, a0, b0, N, mn, 0u);
+    mma_f16(d + N, a0, smem_desc(bb + C::kDig, 128, 256), N * (kFxDig - 1), mn, 1u);
   } else {
-    mma_f16(d, a0, b0, kFxDig, mn, 1u);
+    mma_f16(d, a0, b0, N * kFxDig, mn, 1u);
   }
 #pragma unroll
   for (int i = 2; i < kFxDig; ++i)
-    mma_f16(d + 16 * i, smem_desc(ab + i * atile, alb, asb), b0, kFxBlk - i, mn, 1u);
+    mma_f16(d + N * i, smem_desc(ab + i * atile, alb, asb), b0, N * (kFxBlk - i), mn, 1u);
 }
 
+template <uint32_t COLS>
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_addr(slot)),
-               "n"(kCols)
+               "n"(COLS)
                : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
 }
+template <uint32_t COLS>
 __device__ __forceinline__ void tmem_free(uint32_t tb) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tb), "n"(kCols) : "memory");
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tb), "n"(COLS) : "memory");
+}
+template <int W>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&d)[W]) {
+  if constexpr (W == 4) tmem_ld4(taddr, d);
+  else if constexpr (W == 8) tmem_ld8(taddr, d);
+  else tmem_ld16(taddr, d);
 }
 
 // digit words of zero (byte 7 is stored plus 128)
@@ -117,14 +142,16 @@ constexpr int kSynK = 16;                        // values of l per stage (one K
 constexpr int kSynPeriod = 8;                    // stages between two reads: 64 terms per parity
 constexpr int kSynTile = kM * kSynK * 2;         // one digit of A
 constexpr int kSynA = kFxDig * kSynTile;
+template <typename C>
 struct SynLayout {
-  static constexpr int kA = 0;                      // also the odd sums at the end: double[8][128]
+  static constexpr int kA = 0;                      // also the odd sums at the end: double[2 NM][128]
   static constexpr int kB = kSynA;                  // two stages of B
-  static constexpr int kCoef = kB + 2 * kBStep;     // int4[2][16]
-  static constexpr int kCorr = kCoef + 2 * kSynK * 16;  // fxu_t[16][2]
-  static constexpr int kBar = kCorr + 16 * 16;      // uint64_t[2]
-  static constexpr int kMisc = kBar + 16;           // tensor memory base, bad flag, first start, exponents
-  static constexpr int kBytes = kMisc + 32;
+  static constexpr int kCoef = kB + 2 * C::kBStep;  // int4[2][16]
+  static constexpr int kCorr = kCoef + 2 * kSynK * 16;  // fxu_t[2 W][2]
+  static constexpr int kBar = kCorr + 2 * C::W * 16;    // uint64_t[2]
+  static constexpr int kMisc = kBar + 16;           // tensor memory base, bad flag, first start
+  static constexpr int kExp = kMisc + 16;           // exponents [8]
+  static constexpr int kBytes = kExp + 32;
 };
 
 // Two threads per ring pair (row of A) walk l upwards: one from the first start of the CTA's pairs,
@@ -134,15 +161,17 @@ struct SynLayout {
 // coefficient part to digits of B.  One thread issues the stage's MMAs after its barrier; they read
 // the tile while the threads compute the next values in registers.
 template <int NM>
-__global__ void __launch_bounds__(kNT, 3)
+__global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double* __restrict__ Acoef,
                const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
                const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
                const double2* __restrict__ ck, const int64_t* __restrict__ ck_base,
                const int2* __restrict__ pring, double2* __restrict__ F, int64_t F_stride, int L, int npair,
-               int R) {
-  using LY = SynLayout;
-  constexpr int P = 2 * NM;
+               int R, int nmaps) {
+  using C = Cols<NM>;
+  using LY = SynLayout<C>;
+  constexpr int P = 2 * NM, W = C::W;
+  const int nm = NM <= 4 ? NM : nmaps;
   extern __shared__ __align__(1024) unsigned char sm[];
   int4* s_coef = reinterpret_cast<int4*>(sm + LY::kCoef);
   fxu_t* s_corr = reinterpret_cast<fxu_t*>(sm + LY::kCorr);
@@ -150,7 +179,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   uint32_t* s_tb = reinterpret_cast<uint32_t*>(sm + LY::kMisc);
   int* s_bad = reinterpret_cast<int*>(sm + LY::kMisc + 4);
   int* s_lo = reinterpret_cast<int*>(sm + LY::kMisc + 8);
-  unsigned* s_emax = reinterpret_cast<unsigned*>(sm + LY::kMisc + 16);
+  unsigned* s_emax = reinterpret_cast<unsigned*>(sm + LY::kExp);
 
   const int tid = threadIdx.x, warp = tid >> 5;
   const int row = tid & (kM - 1), chain = tid >> 7;  // chain: warp-uniform
@@ -159,7 +188,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   const int S = fx_scale(mumax[m]);
 
   // scale of each map: the largest exponent among this m's coefficients
-  if (tid < 4) s_emax[tid] = 0;
+  if (tid < 8) s_emax[tid] = 0;
   if (tid == 0) {
     *s_bad = 0;
     mbar_init(&mbar[0], 1);
@@ -168,6 +197,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < NM; ++k) {
+    if (k >= nm) break;
     unsigned e = 0;
 #pragma unroll 4
     for (int l = m + tid; l <= L; l += kNT) {
@@ -179,22 +209,24 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     if ((tid & 31) == 0) atomicMax(&s_emax[k], e);
   }
   // zero B (columns of the other parity and of absent maps stay zero)
-  for (int i = tid; i < 2 * kBStep / 16; i += kNT)
+  for (int i = tid; i < 2 * C::kBStep / 16; i += kNT)
     reinterpret_cast<uint4*>(sm + LY::kB)[i] = make_uint4(0, 0, 0, 0);
-  if (warp == 0) tmem_alloc(s_tb);
+  if (warp == 0) tmem_alloc<C::kTmem>(s_tb);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tb = *s_tb;
   const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
 
-  // this thread's coefficient part of a stage (of the stages t with t mod 2 = chain): value k of l
-  // (0..7 of the first chain, 8..15 of the second), part q (re / im of each map)
-  const int bk = tid & 15, bq = (tid >> 4) & 7;
-  const bool bon = bq < P;
+  // this thread's coefficient part of a stage (W = 8: of the stages t with t mod 2 = chain): value k
+  // of l (0..7 of the first chain, 8..15 of the second), part q (re / im of each map)
+  constexpr int kBEvery = W == 8 ? 2 : 1;
+  const int bk = tid & 15, bq = (tid >> 4) & (W - 1);
+  const bool bon = bq < 2 * nm;
   const int eb = bon ? (int)s_emax[bq >> 1] - 1022 : 0;  // |a| < 2^eb; 1025 if not finite
   const double* bsrc = reinterpret_cast<const double*>(alm + (bq >> 1) * alm_stride + lmo) + (bq & 1);
-  unsigned char* bdst = sm + LY::kB + (bk & 1) * 256 + (bk >> 3) * 128 + (bq & 7) * 16 + (bk & 7) * 2;
+  unsigned char* bdst = sm + LY::kB + (bk & 1) * W * 32 + (bk >> 3) * 128 + (bq >> 3) * 256 + (bq & 7) * 16 +
+                        (bk & 7) * 2;
   unsigned char* arow = sm + LY::kA + chain * (kSynTile / 2) + row * 16;
 
   int gs = 0;  // stages issued by this CTA
@@ -211,7 +243,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
       s0 = fx_start(v.x, v.y, S, ((ls - m) & 2) != 0);
     }
     if (tid == 0) *s_lo = INT_MAX;
-    if (tid < 32) s_corr[tid] = 0;
+    if (tid < 4 * W) s_corr[tid] = 0;
     __syncthreads();
     const int wlo = __reduce_min_sync(kFull, ls);
     if ((tid & 31) == 0) atomicMin(s_lo, wlo);
@@ -244,7 +276,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     };
     const bool con = tid >= 112 && tid < 128;
     const bool neg = (((bk < 8 ? lo - m : 0) + bk) & 2) != 0;  // sigma of this thread's values of l
-    double anext = load_a(chain), cnext = con ? load_c(0) : 0.0;
+    double anext = load_a(kBEvery == 2 ? chain : 0), cnext = con ? load_c(0) : 0.0;
     if (con) s_coef[tid & 15] = fx_coef(cnext);
     cnext = con ? load_c(1) : 0.0;
     __syncthreads();
@@ -263,9 +295,9 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
         s_coef[((t + 1) & 1) * kSynK + (tid & 15)] = fx_coef(cnext);
         cnext = load_c(t + 2);
       }
-      if ((t & 1) == chain) {
+      if (kBEvery == 1 || (t & 1) == chain) {
         const double av = anext;
-        anext = load_a(t + 2);
+        anext = load_a(t + kBEvery);
         if (bon) {  // B of this stage: its buffer was read two stages ago
           const fx_t v = fx_from_double(neg ? -av : av, kFxABits - eb);
           unsigned dig[kFxDig];
@@ -274,7 +306,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
           slo += v & ((1 << 30) - 1);
 #pragma unroll
           for (int j = 0; j < kFxDig; ++j)
-            *reinterpret_cast<unsigned short*>(bdst + (gs & 1) * kBStep + j * 512) = (unsigned short)dig[j];
+            *reinterpret_cast<unsigned short*>(bdst + (gs & 1) * C::kBStep + j * C::kDig) = (unsigned short)dig[j];
         }
       }
       auto wait = [&]() {  // the previous stage's MMAs have read the tile
@@ -292,8 +324,8 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
       const bool first = t % kSynPeriod == 0;
       if (tid == 0 && !*s_bad) {
         tc_fence_after();
-        mma_step(tb, smem_addr(sm + LY::kA), kSynTile, kSynTile / 2, 128,
-                 smem_addr(sm + LY::kB + (gs & 1) * kBStep), false, first);
+        mma_step<C>(tb, smem_addr(sm + LY::kA), kSynTile, kSynTile / 2, 128,
+                 smem_addr(sm + LY::kB + (gs & 1) * C::kBStep), false, first);
         tc_commit(&mbar[0]);
       }
       if (t % kSynPeriod == kSynPeriod - 1 || t == nst - 1) {
@@ -302,8 +334,8 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
         int prev[P];
 #pragma unroll
         for (int b = 0; b < kFxBlk; ++b) {
-          uint32_t d[8];
-          tmem_ld8(tb + lane_base + 16 * b + 8 * chain, d);
+          uint32_t d[W];
+          tmem_ld<W>(tb + lane_base + 2 * W * b + W * chain, d);
           tmem_ld_wait();
 #pragma unroll
           for (int q = 0; q < P; ++q) acc[q].add(b, digit_sum(d[q]), prev[q]);
@@ -312,8 +344,8 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
       }
     }
     if (bon) {
-      atomicAdd(&s_corr[2 * ((bk & 1) * 8 + bq)], (fxu_t)shi);
-      atomicAdd(&s_corr[2 * ((bk & 1) * 8 + bq) + 1], (fxu_t)slo);
+      atomicAdd(&s_corr[2 * ((bk & 1) * W + bq)], (fxu_t)shi);
+      atomicAdd(&s_corr[2 * ((bk & 1) * W + bq) + 1], (fxu_t)slo);
     }
     if (bad) atomicOr(s_bad, 1);
     __syncthreads();
@@ -323,7 +355,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
 #pragma unroll
     for (int q = 0; q < P; ++q) {
       const int ea = (int)s_emax[q >> 1] - 1022;
-      v[q] = acc[q].value((fx_t)s_corr[2 * (8 * chain + q)], (fx_t)s_corr[2 * (8 * chain + q) + 1], ea - S - 6);
+      v[q] = acc[q].value((fx_t)s_corr[2 * (W * chain + q)], (fx_t)s_corr[2 * (W * chain + q) + 1], ea - S - 6);
       // a map with a non-finite coefficient, and a timed-out wait, give NaN
       if (m > 0) v[q] *= 0.70710678118654752440;  // the ring FFT's 1 / sqrt(2)
       if ((ea >= 1025 && ls <= L) || failed) v[q] = fx_nan();
@@ -334,6 +366,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
       const int2 rr = pring[p];
 #pragma unroll
       for (int k = 0; k < NM; ++k) {
+        if (k >= nm) break;
         const double ox = s_odd[2 * k * kM + row], oy = s_odd[(2 * k + 1) * kM + row];
         F[k * F_stride + (int64_t)rr.x * (L + 1) + m] = make_double2(v[2 * k] + ox, v[2 * k + 1] + oy);
         if (rr.y >= 0)
@@ -343,67 +376,50 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     __syncthreads();  // s_corr and the A rows are reset for the next group
   }
   if (tid == 0 && *s_bad) atomicOr(&g_fx_status, 1u);
-  if (warp == 0) tmem_free(tb);
+  if (warp == 0) tmem_free<C::kTmem>(tb);
 }
 
 // Tiles: groups of 128 ring pairs per CTA, taken one after the other (the autotuner's list of the
 // synthesis; without it one group per CTA).
 template <int NM>
-int launch_synth_variant(int v, const Grid& g, const void* alm, int64_t as, void* F, int64_t fs,
+int launch_synth_variant(int v, int nm, const Grid& g, const void* alm, int64_t as, void* F, int64_t fs,
                          cudaStream_t s) {
+  using LY = SynLayout<Cols<NM>>;
   const int R = v == 0 ? 2 : v == 3 ? 4 : 1;
   const int L = g.lmax;
   dim3 grd((g.npair + kM * R - 1) / (kM * R), L + 1);
   auto kern = k_leg_synth_fx<NM>;
-  CMBWS_TRY(ensure_dyn_smem((const void*)kern, SynLayout::kBytes));
-  ProfScope ps(PROF_LEG_SYNTH, s, 1, leg_work(g, NM));
-  kern<<<grd, kNT, SynLayout::kBytes, s>>>((const double2*)alm, as, g.A64.as<double>(),
-                                          g.mumax.as<unsigned>(), g.lsx.as<int>(), g.stx.as<double2>(),
-                                          g.xfx.as<uint64_t>(), g.ckx.as<double2>(),
-                                          g.ckx_base.as<int64_t>(), g.pair_ring.as<int2>(), (double2*)F, fs, L,
-                                          g.npair, R);
+  CMBWS_TRY(ensure_dyn_smem((const void*)kern, LY::kBytes));
+  ProfScope ps(PROF_LEG_SYNTH, s, 1, leg_work(g, nm));
+  kern<<<grd, kNT, LY::kBytes, s>>>((const double2*)alm, as, g.A64.as<double>(), g.mumax.as<unsigned>(),
+                                    g.lsx.as<int>(), g.stx.as<double2>(), g.xfx.as<uint64_t>(),
+                                    g.ckx.as<double2>(), g.ckx_base.as<int64_t>(),
+                                    g.pair_ring.as<int2>(), (double2*)F, fs, L, g.npair, R, nm);
   CMBWS_LAUNCH_CHECK();
   return CMBWS_OK;
 }
 
 template <int NM>
-int launch_synth(const Grid& g, const void* alm, int64_t as, void* F, int64_t fs, cudaStream_t s) {
+int launch_synth(int nm, const Grid& g, const void* alm, int64_t as, void* F, int64_t fs, cudaStream_t s) {
   int v = 1;
   if (autotune_mode() != 0)
     CMBWS_TRY(autotune_pick(
-        g, synth_tune_key(CMBWS_FP64, NM), 4, 1,
-        [&](int vv) { return launch_synth_variant<NM>(vv, g, alm, as, F, fs, s); }, s, &v));
-  return launch_synth_variant<NM>(v, g, alm, as, F, fs, s);
-}
-
-int synth_dispatch(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s) {
-  const int64_t as = nlm_of(g.lmax), fs = (int64_t)g.nring * (g.lmax + 1);
-  for (int k0 = 0; k0 < nmaps; k0 += 4) {
-    const int nm = nmaps - k0 < 4 ? nmaps - k0 : 4;
-    const void* a = (const double2*)alm + k0 * as;
-    void* f = (double2*)F + k0 * fs;
-    int st = CMBWS_OK;
-    switch (nm) {
-      case 1: st = launch_synth<1>(g, a, as, f, fs, s); break;
-      case 2: st = launch_synth<2>(g, a, as, f, fs, s); break;
-      case 3: st = launch_synth<3>(g, a, as, f, fs, s); break;
-      default: st = launch_synth<4>(g, a, as, f, fs, s); break;
-    }
-    if (st != CMBWS_OK) return st;
-  }
-  return CMBWS_OK;
+        g, synth_tune_key(CMBWS_FP64, nm < 4 ? nm : 4), 4, 1,
+        [&](int vv) { return launch_synth_variant<NM>(vv, nm, g, alm, as, F, fs, s); }, s, &v));
+  return launch_synth_variant<NM>(v, nm, g, alm, as, F, fs, s);
 }
 
 // ---- adjoint ----
 constexpr int kAdjK = 32;                       // ring pairs per stage (two K steps)
 constexpr int kAdjTile = kM * kAdjK * 2;        // one digit of A
 constexpr int kAdjOct = kAdjK * 16;             // bytes between rows 8 i and 8 (i + 1) of A
+template <typename C>
 struct AdjLayout {
   static constexpr int kA = 0;
   static constexpr int kB = kFxDig * kAdjTile;       // two stages of B (two K steps each)
-  static constexpr int kCoef = kB + 4 * kBStep;      // int4[128]
-  static constexpr int kCorr = kCoef + kM * 16;      // fxu_t[16][2]
-  static constexpr int kBar = kCorr + 16 * 16;       // uint64_t[2]
+  static constexpr int kCoef = kB + 4 * C::kBStep;   // int4[128]
+  static constexpr int kCorr = kCoef + kM * 16;      // fxu_t[2 W][2]
+  static constexpr int kBar = kCorr + 2 * C::W * 16; // uint64_t[2]
   static constexpr int kMisc = kBar + 16;            // tensor memory base, bad flag
   static constexpr int kBytes = kMisc + 16;
 };
@@ -415,19 +431,21 @@ __device__ __forceinline__ unsigned part_exp(double v) {
 // ee[map][m] = exponent bound of the map's ring parts at m: |e| < 2^ee (1025: not all finite)
 template <int NM>
 __global__ void __launch_bounds__(256)
-k_eo_exp(const double* __restrict__ eo, int npair, int L, int* __restrict__ ee) {
+k_eo_exp(const double* __restrict__ eo, int npair, int L, int* __restrict__ ee, int nmaps) {
+  const int nm = NM <= 4 ? NM : nmaps;
   __shared__ unsigned s_e[NM];
   const int m = blockIdx.x, tid = threadIdx.x;
   if (tid < NM) s_e[tid] = 0;
   __syncthreads();
-  const double* src = eo + (int64_t)m * npair * 4 * NM;
+  const double* src = eo + (int64_t)m * npair * 4 * nm;
   unsigned e[NM];
 #pragma unroll
   for (int k = 0; k < NM; ++k) e[k] = 0;
-  for (int i = tid; i < 2 * npair; i += 256) {  // (pair, parity): 2 NM values
+  for (int i = tid; i < 2 * npair; i += 256) {  // (pair, parity): 2 nm values
+    const double2* v = reinterpret_cast<const double2*>(src) + (int64_t)i * nm;
 #pragma unroll
     for (int k = 0; k < NM; ++k)
-      e[k] = max(e[k], max(part_exp(src[(int64_t)i * 2 * NM + 2 * k]), part_exp(src[(int64_t)i * 2 * NM + 2 * k + 1])));
+      if (k < nm) e[k] = max(e[k], max(part_exp(v[k].x), part_exp(v[k].y)));
   }
 #pragma unroll
   for (int k = 0; k < NM; ++k) {
@@ -435,7 +453,7 @@ k_eo_exp(const double* __restrict__ eo, int npair, int L, int* __restrict__ ee) 
     if ((tid & 31) == 0) atomicMax(&s_e[k], v);
   }
   __syncthreads();
-  if (tid < NM) ee[(int64_t)tid * (L + 1) + m] = (int)s_e[tid] - 1022;
+  if (tid < nm) ee[(int64_t)tid * (L + 1) + m] = (int)s_e[tid] - 1022;
 }
 
 // One CTA per (m, 128 values of l) loops over the ring pairs, 32 per stage: lane = pair, warp =
@@ -443,15 +461,17 @@ k_eo_exp(const double* __restrict__ eo, int npair, int L, int* __restrict__ ee) 
 // values of l (MN-major: a thread writes 8 consecutive values of its pair as one 16-byte row).
 // Every output has one owner; stages without a started pair are skipped.
 template <int NM>
-__global__ void __launch_bounds__(kNT, 3)
+__global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const double* __restrict__ Acoef,
              const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
              const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
              const double2* __restrict__ ck, const int64_t* __restrict__ ck_base,
              const int* __restrict__ tmin, const double* __restrict__ c64, double2* __restrict__ out,
-             int64_t nlm, int L, int npair) {
-  using LY = AdjLayout;
-  constexpr int P = 2 * NM;
+             int64_t nlm, int L, int npair, int nmaps) {
+  using C = Cols<NM>;
+  using LY = AdjLayout<C>;
+  constexpr int W = C::W;
+  const int nm = NM <= 4 ? NM : nmaps, P = 2 * nm;
   static_assert(kFxChunk == 16 && kAdjK == 32 && kTileMinPT == 16, "stage shape");
   const int m = blockIdx.y;
   const int lb0 = m + kM * (int)blockIdx.x;  // first l of the tile
@@ -478,8 +498,7 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
   if (s >= nst) {  // no pair has a significant value in the tile: the sums are zero
     const int l = lb0 + tid;
     if (tid < kM && l <= L)
-#pragma unroll
-      for (int k = 0; k < NM; ++k) out[k * nlm + lmo + l] = make_double2(0.0, 0.0);
+      for (int k = 0; k < nm; ++k) out[k * nlm + lmo + l] = make_double2(0.0, 0.0);
     return;
   }
   const int S = fx_scale(mumax[m]);
@@ -488,14 +507,14 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
     mbar_init(&mbar[0], 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  if (tid < 32) s_corr[tid] = 0;
+  if (tid < 4 * W) s_corr[tid] = 0;
   if (tid < kM) {
     const int l = lb0 + tid;
     s_coef[tid] = fx_coef(l <= L ? Acoef[lmo + l] : 0.0);
   }
-  for (int i = tid; i < 4 * kBStep / 16; i += kNT)  // B columns of absent maps stay zero
+  for (int i = tid; i < 4 * C::kBStep / 16; i += kNT)  // B columns of absent maps stay zero
     reinterpret_cast<uint4*>(sm + LY::kB)[i] = make_uint4(0, 0, 0, 0);
-  if (warp == 0) tmem_alloc(s_tb);
+  if (warp == 0) tmem_alloc<C::kTmem>(s_tb);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -511,16 +530,19 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
   const double2* stm = st + (int64_t)m * npair;
   unsigned char* arow = sm + LY::kA + 2 * warp * kAdjOct + lane * 16;
 
-  // this thread's ring parts of a stage: column nn of parity par, pairs 8 oct + 2 quarter + 0..1
-  const int quarter = tid & 3, nn = (tid >> 2) & 7, oct = (tid >> 5) & 3, par = tid >> 7;
+  // this thread's ring parts of a stage: column nn of parity par, kPP pairs from 8 oct + kPP sub on
+  constexpr int kPP = W / 4, kSub = 8 / kPP;
+  const int sub = tid & (kSub - 1), nn = (tid / kSub) & (W - 1), oct = (tid >> 5) & 3, par = tid >> 7;
+  const int col = (nn & 1) * (W / 2) + (nn >> 1);
   const bool bon = nn < P;
   const int eb = bon ? ee[(int64_t)(nn >> 1) * (L + 1) + m] : 0;
   const double* bsrc = eo + (int64_t)m * npair * 2 * P + par * P + nn;
-  unsigned char* bdst = sm + LY::kB + (oct >> 1) * kBStep + par * 256 + (oct & 1) * 128 + nn * 16 + quarter * 4;
+  unsigned char* bdst = sm + LY::kB + (oct >> 1) * C::kBStep + par * W * 32 + (oct & 1) * 128 +
+                        (col >> 3) * 256 + (col & 7) * 16 + sub * kPP * 2;
 
   // inputs of a stage, loaded one stage ahead
   struct In {
-    double e[2];
+    double e[kPP];
     double2 c;
     uint64_t x;
     int ls;
@@ -533,8 +555,8 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
     in.c = make_double2(0.0, 0.0);
     if (ok && cval) in.c = ckc[(int64_t)p * nck];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int q = t * kAdjK + 8 * oct + 2 * quarter + i;
+    for (int i = 0; i < kPP; ++i) {
+      const int q = t * kAdjK + 8 * oct + kPP * sub + i;
       in.e[i] = 0.0;
       if (bon && eb < 1025 && t < nst && q < npair) in.e[i] = bsrc[(int64_t)q * 2 * P];
     }
@@ -561,21 +583,22 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
         s0 = fx_start(v.x, v.y, S, ((ls - m) & 2) != 0);
       }
     }
-    const double ev[2] = {in.e[0], in.e[1]};
+    double ev[kPP];
+#pragma unroll
+    for (int i = 0; i < kPP; ++i) ev[i] = in.e[i];
     load(sn, in);
     if (bon) {  // B of this stage: its buffer was read two stages ago
-      fx_t v[2];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        v[i] = fx_from_double(ev[i], kFxABits - eb);
-        shi += v[i] >> 30;
-        slo += v[i] & ((1 << 30) - 1);
+      for (int i = 0; i < kPP; i += 2) {
+        const fx_t v = fx_from_double(ev[i], kFxABits - eb), u = fx_from_double(ev[i + 1], kFxABits - eb);
+        shi += (v >> 30) + (u >> 30);
+        slo += (v & ((1 << 30) - 1)) + (u & ((1 << 30) - 1));
+        unsigned dig[kFxDig];
+        fx_coef_digits(v, u, dig);
+#pragma unroll
+        for (int j = 0; j < kFxDig; ++j)
+          *reinterpret_cast<unsigned*>(bdst + (k & 1) * 2 * C::kBStep + j * C::kDig + 2 * i) = dig[j];
       }
-      unsigned dig[kFxDig];
-      fx_coef_digits(v[0], v[1], dig);
-#pragma unroll
-      for (int j = 0; j < kFxDig; ++j)
-        *reinterpret_cast<unsigned*>(bdst + (k & 1) * 2 * kBStep + j * 512) = dig[j];
     }
     auto wait = [&]() {  // the previous stage's MMAs have read the tile
       if (k >= 1 && !*s_bad && !mbar_wait(&mbar[0], (k - 1) & 1)) bad = true;
@@ -608,8 +631,8 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
       tc_fence_after();
 #pragma unroll
       for (int ks = 0; ks < 2; ++ks)
-        mma_step(tb, smem_addr(sm + LY::kA) + ks * 256, kAdjTile, 128, kAdjOct,
-                 smem_addr(sm + LY::kB + ((k & 1) * 2 + ks) * kBStep), true, first && ks == 0);
+        mma_step<C>(tb, smem_addr(sm + LY::kA) + ks * 256, kAdjTile, 128, kAdjOct,
+                 smem_addr(sm + LY::kB + ((k & 1) * 2 + ks) * C::kBStep), true, first && ks == 0);
       tc_commit(&mbar[0]);
     }
     if ((k & 1) == 1 || sn >= nst) {
@@ -619,35 +642,36 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
       const int odd = tid & 1;  // parity of l - m of this thread's row
 #pragma unroll
       for (int b = 0; b < kFxBlk; ++b) {
-        uint32_t d[16];
-        tmem_ld16(tb + lane_base + 16 * b, d);
+        uint32_t d[W / 2], f[W / 2];
+        const uint32_t c = tb + lane_base + 2 * W * b + grp * (W / 2);
+        tmem_ld<W / 2>(c, d);
+        tmem_ld<W / 2>(c + W, f);
         tmem_ld_wait();
 #pragma unroll
-        for (int q = 0; q < NM; ++q)
-          acc[q].add(b, digit_sum(odd ? (grp ? d[9 + 2 * q] : d[8 + 2 * q]) : (grp ? d[1 + 2 * q] : d[2 * q])),
-                     prev[q]);
+        for (int q = 0; q < NM; ++q) acc[q].add(b, digit_sum(odd ? f[q] : d[q]), prev[q]);
       }
       tc_fence_before();  // read before the next stage's MMAs, which follow its barrier
     }
     s = sn;
   }
   if (bon) {
-    atomicAdd(&s_corr[2 * (par * 8 + nn)], (fxu_t)shi);
-    atomicAdd(&s_corr[2 * (par * 8 + nn) + 1], (fxu_t)slo);
+    atomicAdd(&s_corr[2 * (par * W + nn)], (fxu_t)shi);
+    atomicAdd(&s_corr[2 * (par * W + nn) + 1], (fxu_t)slo);
   }
   if (bad) atomicOr(s_bad, 1);
   __syncthreads();
   const bool failed = *s_bad != 0;
   if (tid == 0 && failed) atomicOr(&g_fx_status, 1u);
-  if (warp == 0) tmem_free(tb);
+  if (warp == 0) tmem_free<C::kTmem>(tb);
   const int l = lb0 + (tid & (kM - 1));  // row of D
   if (l > L) return;
-  const fxu_t* corr = s_corr + 16 * (tid & 1) + 2 * grp;
+  const fxu_t* corr = s_corr + 2 * W * (tid & 1) + 2 * grp;
   // sigma of l, and the ring FFT's sqrt(2)
   const double cc = ((tid & 2) ? -c64[lmo + l] : c64[lmo + l]) * (m > 0 ? 1.41421356237309504880 : 1.0);
   double* o = reinterpret_cast<double*>(out + lmo + l) + grp;
 #pragma unroll
   for (int q = 0; q < NM; ++q) {
+    if (q >= nm) break;
     const int ea = ee[(int64_t)q * (L + 1) + m];
     const double v = acc[q].value((fx_t)corr[4 * q], (fx_t)corr[4 * q + 1], ea - S - 6);
     // a map with a non-finite ring part, and a timed-out wait, give NaN
@@ -656,50 +680,62 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
 }
 
 template <int NM>
-int launch_adj(const Grid& g, const void* eo, int* ee, double* out, cudaStream_t s) {
+int launch_adj(int nm, const Grid& g, const double* eo, int* ee, double* out, cudaStream_t s) {
+  using LY = AdjLayout<Cols<NM>>;
   const int L = g.lmax;
-  ProfScope ps(PROF_LEG_ADJ, s, 1, leg_work(g, NM));
-  k_eo_exp<NM><<<L + 1, 256, 0, s>>>((const double*)eo, g.npair, L, ee);
+  ProfScope ps(PROF_LEG_ADJ, s, 1, leg_work(g, nm));
+  k_eo_exp<NM><<<L + 1, 256, 0, s>>>(eo, g.npair, L, ee, nm);
   CMBWS_LAUNCH_CHECK();
   dim3 grd((L + kM) / kM, L + 1);
   auto kern = k_leg_adj_fx<NM>;
-  CMBWS_TRY(ensure_dyn_smem((const void*)kern, AdjLayout::kBytes));
-  kern<<<grd, kNT, AdjLayout::kBytes, s>>>((const double*)eo, ee, g.A64.as<double>(), g.mumax.as<unsigned>(),
-                                          g.lsx.as<int>(), g.stx.as<double2>(), g.xfx.as<uint64_t>(),
-                                          g.ckx.as<double2>(), g.ckx_base.as<int64_t>(),
-                                          g.ls_tmin.as<int>(), g.c64.as<double>(), (double2*)out,
-                                          nlm_of(L), L, g.npair);
+  CMBWS_TRY(ensure_dyn_smem((const void*)kern, LY::kBytes));
+  kern<<<grd, kNT, LY::kBytes, s>>>(eo, ee, g.A64.as<double>(), g.mumax.as<unsigned>(), g.lsx.as<int>(),
+                                    g.stx.as<double2>(), g.xfx.as<uint64_t>(), g.ckx.as<double2>(),
+                                    g.ckx_base.as<int64_t>(), g.ls_tmin.as<int>(), g.c64.as<double>(),
+                                    (double2*)out, nlm_of(L), L, g.npair, nm);
   CMBWS_LAUNCH_CHECK();
-  return CMBWS_OK;
-}
-
-int adj_dispatch(const Grid& g, int nmaps, const void* eo, int* ee, double* out, cudaStream_t s) {
-  const int64_t nlm = nlm_of(g.lmax), cs = (int64_t)(g.lmax + 1) * g.npair * 4;
-  for (int k0 = 0; k0 < nmaps; k0 += 4) {
-    const int nm = nmaps - k0 < 4 ? nmaps - k0 : 4;
-    const void* e = (const double*)eo + k0 * cs;
-    int* x = ee + (int64_t)k0 * (g.lmax + 1);
-    double* o = out + 2 * k0 * nlm;
-    int st = CMBWS_OK;
-    switch (nm) {
-      case 1: st = launch_adj<1>(g, e, x, o, s); break;
-      case 2: st = launch_adj<2>(g, e, x, o, s); break;
-      case 3: st = launch_adj<3>(g, e, x, o, s); break;
-      default: st = launch_adj<4>(g, e, x, o, s); break;
-    }
-    if (st != CMBWS_OK) return st;
-  }
   return CMBWS_OK;
 }
 
 }  // namespace
 
-int legendre_adjoint_fx(const Grid& g, int nmaps, const void* eo, int* ee, double* out, cudaStream_t s) {
-  return adj_dispatch(g, nmaps, eo, ee, out, s);
+int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s) {
+  const int64_t as = nlm_of(g.lmax), fs = (int64_t)g.nring * (g.lmax + 1);
+  for (int k0 = 0; k0 < nmaps; k0 += kFxMaps) {
+    const int nm = nmaps - k0 < kFxMaps ? nmaps - k0 : kFxMaps;
+    const void* a = (const double2*)alm + k0 * as;
+    void* f = (double2*)F + k0 * fs;
+    switch (nm) {
+      case 1: CMBWS_TRY(launch_synth<1>(nm, g, a, as, f, fs, s)); break;
+      case 2: CMBWS_TRY(launch_synth<2>(nm, g, a, as, f, fs, s)); break;
+      case 3: CMBWS_TRY(launch_synth<3>(nm, g, a, as, f, fs, s)); break;
+      case 4: CMBWS_TRY(launch_synth<4>(nm, g, a, as, f, fs, s)); break;
+      case 5:
+      case 6: CMBWS_TRY(launch_synth<6>(nm, g, a, as, f, fs, s)); break;
+      default: CMBWS_TRY(launch_synth<8>(nm, g, a, as, f, fs, s)); break;
+    }
+  }
+  return CMBWS_OK;
 }
 
-int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s) {
-  return synth_dispatch(g, nmaps, alm, F, s);
+int legendre_adjoint_fx(const Grid& g, int nmaps, const void* eo, int* ee, double* out, cudaStream_t s) {
+  const int64_t nlm = nlm_of(g.lmax), cs = (int64_t)(g.lmax + 1) * g.npair * 4;
+  for (int k0 = 0; k0 < nmaps; k0 += kFxMaps) {
+    const int nm = nmaps - k0 < kFxMaps ? nmaps - k0 : kFxMaps;
+    const double* e = (const double*)eo + k0 * cs;
+    int* x = ee + (int64_t)k0 * (g.lmax + 1);
+    double* o = out + 2 * k0 * nlm;
+    switch (nm) {
+      case 1: CMBWS_TRY(launch_adj<1>(nm, g, e, x, o, s)); break;
+      case 2: CMBWS_TRY(launch_adj<2>(nm, g, e, x, o, s)); break;
+      case 3: CMBWS_TRY(launch_adj<3>(nm, g, e, x, o, s)); break;
+      case 4: CMBWS_TRY(launch_adj<4>(nm, g, e, x, o, s)); break;
+      case 5:
+      case 6: CMBWS_TRY(launch_adj<6>(nm, g, e, x, o, s)); break;
+      default: CMBWS_TRY(launch_adj<8>(nm, g, e, x, o, s)); break;
+    }
+  }
+  return CMBWS_OK;
 }
 
 int fx_status_take(bool* timed_out) {

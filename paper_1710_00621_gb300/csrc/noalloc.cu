@@ -89,13 +89,13 @@ extern "C" int cmbws_sht_analysis_noalloc(cmbws_grid gh, cmbws_prec prec, const 
     return CMBWS_ERR_ARG;
   }
   // the documented limit: ring spectra, adjoint scratch (FP64: partial sums of blocks of 256 ring
-  // pairs) and coefficients together; what is used below stays under it
+  // pairs for up to 4 maps) and coefficients together; what is used below stays under it
   const size_t es = prec_size(prec);
   const int64_t nlm = nlm_of(g->lmax);
   const int cm = eo_maps(prec), nc = nmaps < cm ? nmaps : cm;
   const size_t fb = round256((size_t)nmaps * g->nring * (g->lmax + 1) * 2 * es);
   const size_t sb = prec == CMBWS_FP64
-                        ? round256((size_t)((g->npair + 255) / 256) * 2 * nc * nlm * 8)
+                        ? round256((size_t)((g->npair + 255) / 256) * 2 * (nc < 4 ? nc : 4) * nlm * 8)
                         : round256(legendre_adjoint_part_bytes(*g, prec, nmaps));
   const size_t ob = round256((size_t)nmaps * nlm * 16);
   const size_t pb = round256(legendre_adjoint_part_bytes(*g, prec, nc));

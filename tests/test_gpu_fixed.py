@@ -97,3 +97,23 @@ def test_zero_input():
     back = to_dev(np.ones(24 ** 2))
     cw.cmbws_sht_analysis(g, cw.CMBWS_FP64, to_dev(np.zeros(g.npix)), back, 1, 1)
     assert not to_host(out).any() and not to_host(back).any()
+
+
+@pytest.mark.parametrize("maps", [5, 6, 7, 8, 9])
+@pytest.mark.parametrize("n,lmax", [(66, 31), (130, 127), (259, 129)])
+def test_maps_of_a_batch_are_those_of_single_calls(n, lmax, maps):
+    """Integer sums do not depend on how the maps are grouped: equal bit for bit."""
+    g = cw.cmbws_plan_grid(cw.CMBWS_GRID_GL, n, lmax)
+    rng = np.random.default_rng(n + 1000 * lmax + maps)
+    alm = rng.standard_normal((maps, (lmax + 1) ** 2)) * 10.0 ** rng.uniform(-3, 3, (maps, 1))
+    f = rng.standard_normal((maps, g.npix))
+    out, back = to_dev(np.zeros((maps, g.npix))), to_dev(np.zeros_like(alm))
+    cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(alm), out, maps)
+    cw.cmbws_sht_analysis(g, cw.CMBWS_FP64, to_dev(f), back, maps, 0)
+    m, a = to_host(out), to_host(back)
+    for k in range(maps):
+        one, bone = to_dev(np.zeros((1, g.npix))), to_dev(np.zeros((1, (lmax + 1) ** 2)))
+        cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(alm[k:k + 1]), one, 1)
+        cw.cmbws_sht_analysis(g, cw.CMBWS_FP64, to_dev(f[k:k + 1]), bone, 1, 0)
+        assert np.array_equal(m[k], to_host(one)[0])
+        assert np.array_equal(a[k], to_host(bone)[0])

@@ -1,7 +1,7 @@
 // Preconditioned conjugate gradients for A x = b (Sec. 2.3) with M_PI (Sec. 3.3).
 //
-// Vectors are FP64 on the device.  Dot products are deterministic: a fixed
-// grid writes per-block partial sums, one block adds them in a fixed order.
+// Vectors are FP64 on the device.  Dot products are deterministic: every block of a grid of up to
+// 1024 writes its partial sum, and the block that ends last adds them in a fixed order.
 // The host reads one or two scalars per iteration (alpha and beta are
 // computed on the host in FP64).
 //
@@ -11,6 +11,7 @@
 // residual falls by inner_tol, then x += d and r = b - A x with an
 // FP64-accurate chain (native FP64 or double-float, opts.cert_prec); the loop
 // ends when that residual certifies tol.
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <cmath>
@@ -38,26 +39,53 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return t;
 }
 
-// partial[b] = sum_{i in block-stride range} a[i] * b[i]
-__global__ void k_dot_partial(const double* __restrict__ a, const double* __restrict__ b, int64_t n,
-                              double* __restrict__ partial) {
+// Sum over the grid of the blocks' sums s (in thread 0) to *out: the block that ends last adds the
+// partial sums, thread t those of blocks t, t + 256, .. in that order, and leaves the counter at
+// zero for the next sum on the stream.  A vector of fewer than 1024 x 256 elements takes as many
+// blocks as it fills (the others' partial sums would be zeros).  Launch latency bounds these kernels
+// for short vectors: a 17-iteration solve for 8192 unknowns spent 876 us in them with a second launch
+// for the sum and always 1024 blocks, 566 us like this.  The order of the additions is the same.
+__device__ __forceinline__ void grid_sum(double s, double* sh, double* partial, unsigned* count,
+                                         double* out) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    __stcg(&partial[blockIdx.x], s);
+    __threadfence();
+    last = atomicAdd(count, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double t = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) t += __ldcg(&partial[i]);
+  t = block_sum(t, sh);
+  if (threadIdx.x == 0) {
+    *out = t;
+    *count = 0;
+  }
+}
+
+// *out = a . b
+__global__ void k_dot(const double* __restrict__ a, const double* __restrict__ b, int64_t n,
+                      double* __restrict__ partial, unsigned* __restrict__ count,
+                      double* __restrict__ out) {
   __shared__ double sh[32];
   double s = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     s += a[i] * b[i];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+  grid_sum(block_sum(s, sh), sh, partial, count, out);
 }
 
-// x += alpha p; r -= alpha q; partial sums of r.r, with alpha = rz / pq read from the device
+// x += alpha p; r -= alpha q; *out = r.r, with alpha = rz / pq read from the device
 // (the PCG scalars stay on the device between the host's one read per iteration); alpha = 0
 // when p.q is not a positive finite number or r.z is not finite, and the host then reports the
 // breakdown with x, r unchanged.
 __global__ void k_update_xr_dev(double* __restrict__ x, double* __restrict__ r,
                                 const double* __restrict__ p, const double* __restrict__ q,
                                 const double* __restrict__ rz, const double* __restrict__ pq,
-                                int64_t n, double* __restrict__ partial) {
+                                int64_t n, double* __restrict__ partial, unsigned* __restrict__ count,
+                                double* __restrict__ out) {
   __shared__ double sh[32];
   const double a = *rz, b = *pq;
   const double alpha = (b > 0.0 && isfinite(b) && isfinite(a)) ? a / b : 0.0;
@@ -69,8 +97,7 @@ __global__ void k_update_xr_dev(double* __restrict__ x, double* __restrict__ r,
     r[i] = ri;
     s += ri * ri;
   }
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+  grid_sum(block_sum(s, sh), sh, partial, count, out);
 }
 
 // p = z + (rz_new / rz_old) p, the ratio read from the device
@@ -83,9 +110,10 @@ __global__ void k_xpby_dev(const double* __restrict__ z, double* __restrict__ p,
     p[i] = z[i] + beta * p[i];
 }
 
-// r = b - y; partial sums of r.r
+// r = b - y; *out = r.r
 __global__ void k_resid(const double* __restrict__ b, const double* __restrict__ y,
-                        double* __restrict__ r, int64_t n, double* __restrict__ partial) {
+                        double* __restrict__ r, int64_t n, double* __restrict__ partial,
+                        unsigned* __restrict__ count, double* __restrict__ out) {
   __shared__ double sh[32];
   double s = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -94,8 +122,7 @@ __global__ void k_resid(const double* __restrict__ b, const double* __restrict__
     r[i] = ri;
     s += ri * ri;
   }
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+  grid_sum(block_sum(s, sh), sh, partial, count, out);
 }
 
 // y += x
@@ -105,9 +132,10 @@ __global__ void k_axpy1(const double* __restrict__ x, double* __restrict__ y, in
     y[i] += x[i];
 }
 
-// partial sums of |x + d - t|^2 (distance of the current iterate to a reference solution)
-__global__ void k_err_partial(const double* __restrict__ x, const double* __restrict__ d,
-                              const double* __restrict__ t, int64_t n, double* __restrict__ partial) {
+// *out = |x + d - t|^2 (distance of the current iterate to a reference solution)
+__global__ void k_err(const double* __restrict__ x, const double* __restrict__ d,
+                      const double* __restrict__ t, int64_t n, double* __restrict__ partial,
+                      unsigned* __restrict__ count, double* __restrict__ out) {
   __shared__ double sh[32];
   double s = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -115,16 +143,7 @@ __global__ void k_err_partial(const double* __restrict__ x, const double* __rest
     const double e = x[i] + d[i] - t[i];
     s += e * e;
   }
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
-}
-
-__global__ void k_finish(const double* __restrict__ partial, int nb, double* __restrict__ out) {
-  __shared__ double sh[32];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) s += partial[i];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) *out = s;
+  grid_sum(block_sum(s, sh), sh, partial, count, out);
 }
 
 struct Clock {
@@ -142,9 +161,9 @@ struct Comm {
 };
 
 // Device scalar slots after the reduction partials (red + kRedBlocks): 0 the last finished
-// sum, 1 p.q, 2 r.r, 3 + (it & 1) r.z of iteration it.
+// sum, 1 p.q, 2 r.r, 3 + (it & 1) r.z of iteration it, 7 the counter of grid_sum.
 constexpr int kScal = 8;
-constexpr int kSlotPQ = 1, kSlotRR = 2, kSlotRZ = 3;
+constexpr int kSlotPQ = 1, kSlotRR = 2, kSlotRZ = 3, kSlotCount = 7;
 
 struct Solver {
   Model& M;
@@ -155,12 +174,12 @@ struct Solver {
   const Comm* comm = nullptr;
 
   double* slot(int i) { return red + kRedBlocks + i; }
+  unsigned* count() { return reinterpret_cast<unsigned*>(slot(kSlotCount)); }
+  int blocks() const { return (int)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (n + kRedThreads - 1) / kRedThreads)); }
   // sum of a . b into a device slot (no host synchronisation)
   int dot_dev(const double* a, const double* b, double* out) {
     ProfScope ps_(PROF_CG, s);
-    k_dot_partial<<<kRedBlocks, kRedThreads, 0, s>>>(a, b, n, red);
-    CMBWS_LAUNCH_CHECK();
-    k_finish<<<1, kRedThreads, 0, s>>>(red, kRedBlocks, out);
+    k_dot<<<blocks(), kRedThreads, 0, s>>>(a, b, n, red, count(), out);
     CMBWS_LAUNCH_CHECK();
     return CMBWS_OK;
   }
@@ -182,23 +201,15 @@ struct Solver {
     return CMBWS_OK;
   }
 
+  // the last finished sum (slot 0), read back
   int finish(double* out) {
-    {
-      ProfScope ps_(PROF_CG, s);
-      k_finish<<<1, kRedThreads, 0, s>>>(red, kRedBlocks, red + kRedBlocks);
-      CMBWS_LAUNCH_CHECK();
-    }
-    CMBWS_CUDA(cudaMemcpyAsync(hscal, red + kRedBlocks, 8, cudaMemcpyDeviceToHost, s));
+    CMBWS_CUDA(cudaMemcpyAsync(hscal, slot(0), 8, cudaMemcpyDeviceToHost, s));
     CMBWS_CUDA(cudaStreamSynchronize(s));
     *out = *hscal;
     return CMBWS_OK;
   }
   int dot(const double* a, const double* b, double* out) {
-    {
-      ProfScope ps_(PROF_CG, s);
-      k_dot_partial<<<kRedBlocks, kRedThreads, 0, s>>>(a, b, n, red);
-      CMBWS_LAUNCH_CHECK();
-    }
+    CMBWS_TRY(dot_dev(a, b, slot(0)));
     return finish(out);
   }
   int cert = CMBWS_FP64;  // arithmetic of the true-residual applies
@@ -208,7 +219,7 @@ struct Solver {
     CMBWS_TRY(reduce(tmp));
     {
       ProfScope ps_(PROF_CG, s);
-      k_resid<<<kRedBlocks, kRedThreads, 0, s>>>(b, tmp, r, n, red);
+      k_resid<<<blocks(), kRedThreads, 0, s>>>(b, tmp, r, n, red, count(), slot(0));
       CMBWS_LAUNCH_CHECK();
     }
     return finish(rr);
@@ -321,7 +332,8 @@ static int record_iteration(Solver& S, const PcgRecord& rec, const double* d, do
   if (!M.track_err) return CMBWS_OK;
   {
     ProfScope ps_(PROF_CG, S.s);
-    k_err_partial<<<kRedBlocks, kRedThreads, 0, S.s>>>(rec.x, d, M.cg_xtrue.as<double>(), S.n, S.red);
+    k_err<<<S.blocks(), kRedThreads, 0, S.s>>>(rec.x, d, M.cg_xtrue.as<double>(), S.n, S.red, S.count(),
+                                               S.slot(0));
     CMBWS_LAUNCH_CHECK();
   }
   double ee;
@@ -388,10 +400,8 @@ static int pcg_core(Solver& S, int prec, int use_M, double* d, double* r, double
     CMBWS_TRY(S.dot_dev(p, q, S.slot(kSlotPQ)));
     {
       ProfScope ps_(PROF_CG, S.s);
-      k_update_xr_dev<<<kRedBlocks, kRedThreads, 0, S.s>>>(d, r, p, q, rz_cur, S.slot(kSlotPQ), n,
-                                                           S.red);
-      CMBWS_LAUNCH_CHECK();
-      k_finish<<<1, kRedThreads, 0, S.s>>>(S.red, kRedBlocks, S.slot(kSlotRR));
+      k_update_xr_dev<<<S.blocks(), kRedThreads, 0, S.s>>>(d, r, p, q, rz_cur, S.slot(kSlotPQ), n, S.red,
+                                                           S.count(), S.slot(kSlotRR));
       CMBWS_LAUNCH_CHECK();
     }
     CMBWS_TRY(S.read_slots());
@@ -425,7 +435,7 @@ static int pcg_core(Solver& S, int prec, int use_M, double* d, double* r, double
     CMBWS_TRY(S.dot_dev(r, z, rz_nxt));
     {
       ProfScope ps_(PROF_CG, S.s);
-      k_xpby_dev<<<kRedBlocks, kRedThreads, 0, S.s>>>(z, p, rz_nxt, rz_cur, n);
+      k_xpby_dev<<<S.blocks(), kRedThreads, 0, S.s>>>(z, p, rz_nxt, rz_cur, n);
       CMBWS_LAUNCH_CHECK();
     }
   }
@@ -452,6 +462,8 @@ static int cg_solve_impl(Model& M, const double* b, double* x, const cmbws_cg_op
   CMBWS_TRY(M.cg_red.ensure((kRedBlocks + kScal) * 8));
   if (!M.cg_host) CMBWS_CUDA(cudaMallocHost(&M.cg_host, kScal * 8));
   Solver S{M, s, n, M.cg_red.as<double>(), M.cg_host};
+  // the scalars and grid_sum's counter start at zero
+  CMBWS_CUDA(cudaMemsetAsync(S.slot(0), 0, kScal * 8, s));
   S.cert = o.cert_prec == CMBWS_FP32X2 ? CMBWS_FP32X2 : CMBWS_FP64;
   S.comm = comm;
   const long long sht0 = M.n_sht;
@@ -549,7 +561,7 @@ static int cg_solve_impl(Model& M, const double* b, double* x, const cmbws_cg_op
     }
     {
       ProfScope ps_(PROF_CG, s);
-      k_axpy1<<<kRedBlocks, kRedThreads, 0, s>>>(d, x, n);
+      k_axpy1<<<S.blocks(), kRedThreads, 0, s>>>(d, x, n);
       CMBWS_LAUNCH_CHECK();
     }
     CMBWS_TRY(S.true_residual(b, x, r, tmp, &rr));

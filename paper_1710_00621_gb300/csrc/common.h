@@ -181,6 +181,7 @@ struct Grid {
   DevMem ck32;            // FP32 {mu_l0, mu_l0+1} at every chunk start l0 = m + kChunk c
   DevMem ck_base;         // int64 [L+1]: offset of m's block [pair][chunk] in ck32
   DevMem ls_tmin;         // int [L+1][ceil(npair / kTileMinPT)]: smallest ls of each tile of pairs
+  DevMem lsx_tmin;        // the same of lsx
   // warp tasks of the checkpointed FP32 adjoint: int2 {m, first chunk} per 32 consecutive
   // chunks of one m, m ascending
   DevMem wt32;

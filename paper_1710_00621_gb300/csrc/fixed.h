@@ -9,8 +9,9 @@
 // grid is planned; b is 1 to 4 in practice, so the quantum is 2^-58 or finer).  The sign sigma
 // = + + - - by l - m modulo 4 turns mu_l = A x mu_{l-1} - mu_{l-2} into V2 - A x V1 (l - m even) and
 // V2 + A x V1 (odd); the coefficients (synthesis) or the results (adjoint) take sigma back.
-// For the products V = h 2^32 + l with both words signed; for the contraction the bytes of
-// V + 2^63 are its base-256 digits, byte 7 less 128, the others as they are.
+// For the products V = h 2^32 + l with both words signed: the state holds V + 2^31, whose upper word
+// is h and whose lower one is l + 2^31.  For the contraction the bytes of V + 2^63 are its base-256
+// digits, byte 7 less 128, the others as they are.
 // Before a pair's values are of order one (they grow from 2^-64 where its walk starts; smaller
 // ones are below the last digit), V carries a binary exponent e (a multiple of 8):
 // mu = V 2^-(S + e), V shifted down by 8 bits as it grows; e is 0 from |mu| ~ 2^-7 on.
@@ -34,6 +35,7 @@ typedef long long fx_t;
 typedef unsigned long long fxu_t;
 
 constexpr int kFxABits = 54;  // coefficients and ring parts: |a| < 2^54
+constexpr fx_t kFxBias = 1ll << 31;
 constexpr int kFxDig = 7;     // digits of both factors
 constexpr int kFxBlk = 8;     // sums kept: i + j = 0..7
 
@@ -82,37 +84,41 @@ __device__ __forceinline__ void fx_coef_digits(fx_t v0, fx_t v1, unsigned (&w)[k
   }
 }
 
-// A_lm as {upper word, lower word, shift, rounding constant} of a recurrence step: with
-// A < 2^sh the words hold A 2^(63 - sh), the shift is 2 + sh
+// A_lm as {upper word, signed lower word, shift, rounding constant} of a recurrence step: with
+// A < 2^sh the words hold A 2^(62 - sh), the shift is 3 + sh
 __device__ __forceinline__ int4 fx_coef(double A) {
-  if (!(A > 0.0)) return make_int4(0, 0, 2, 0);
+  if (!(A > 0.0)) return make_int4(0, 0, 3, 0);
   const fxu_t b = (fxu_t)__double_as_longlong(A);
   const int E = (int)((b >> 52) & 0x7ff) - 1023;
   const int sh = max(E + 1, 0);
-  const fxu_t m = ((b & 0xfffffffffffffull) | (1ull << 52)) << (11 + E - sh);  // E >= -10
-  return make_int4((int)(m >> 32), (int)m, 2 + sh, 1 << (29 - sh));
+  const fxu_t m = ((b & 0xfffffffffffffull) | (1ull << 52)) << (10 + E - sh);  // E >= -10
+  return make_int4((int)((m + (1ull << 31)) >> 32), (int)m, 3 + sh, 1 << (28 - sh));
 }
 
-// A x V1 rounded; x = xh 2^32 + xl holds cos(theta) 2^63.  A x is formed as A x 2^(62 - sh)
-// (dropping the lowest partial product), the product with V1 keeps 96 bits of which the shift takes
-// the upper 64.  2^63 is added to the sum of the cross products and taken out again from its upper
-// word, which is then unsigned.
+// A x V1 rounded; V1 is biased, x = xh 2^32 + xl holds cos(theta) 2^63.  A x is formed as
+// A x 2^(61 - sh) plus 2^31, so that its words split as V's do (the lower word of A is signed: the sum
+// of the three lower terms then fits 32 bits).  The parts dropped from it are one unit on average,
+// which is put back: a constant error of A x is a drift of the phase.  The product with V1 keeps 96
+// bits of which the shift takes the upper 64 (dropped: below 2 units).
+// With biased words and sums of signed products a step takes 42 issue cycles per warp; with the words
+// split from an unbiased V and the cross products summed as unsigned it took 47.
 __device__ __forceinline__ fx_t fx_ax(int4 A, unsigned xh, unsigned xl, fx_t V1) {
-  const unsigned Ah = (unsigned)A.x, Al = (unsigned)A.y;
-  const fxu_t X = fx_mulu(Ah, xh) + (fx_mulu(Ah, xl) >> 32) + (fx_mulu(Al, xh) >> 32);
-  const int Xl = (int)X, Xh = (int)((unsigned)(X >> 32) + ((unsigned)X >> 31));
-  const int Vl = (int)V1, Vh = (int)((unsigned)((fxu_t)V1 >> 32) + ((unsigned)V1 >> 31));
-  const fxu_t cr = (fxu_t)fx_mul(Xl, Vh) + (fxu_t)fx_mul(Xh, Vl) + ((1ull << 63) + (unsigned)A.w);
-  const fxu_t hh = (fxu_t)fx_mul(Xh, Vh) + (cr >> 32) - 0x80000000ull;
-  const unsigned lo = (unsigned)hh, hi = (unsigned)(hh >> 32);
+  const unsigned u = (unsigned)(fx_mulu((unsigned)A.x, xl) >> 32) + (unsigned)((fxu_t)fx_mul(A.y, (int)xh) >> 32) +
+                     0x80000001u;
+  const fxu_t X = fx_mulu((unsigned)A.x, xh) + u;
+  const int Xl = (int)((unsigned)X - 0x80000000u), Xh = (int)(X >> 32);
+  const int Vl = (int)((unsigned)V1 - 0x80000000u), Vh = (int)((fxu_t)V1 >> 32);
+  const fx_t cr = fx_mul(Xl, Vh) + fx_mul(Xh, Vl) + (fx_t)(unsigned)A.w;
+  const fx_t hh = fx_mul(Xh, Vh) + (fx_t)(int)(cr >> 32);
+  const unsigned lo = (unsigned)hh, hi = (unsigned)((fxu_t)hh >> 32);
   const unsigned ph = __funnelshift_l(lo, hi, A.z), pl = __funnelshift_l((unsigned)cr, lo, A.z);
   return (fx_t)(((fxu_t)ph << 32) | pl);
 }
 
-// Row state of one ring pair: the last two values (V1 at l - 1, V2 at l - 2) and their exponent.
-// A pair that has not started holds zeros.
+// Row state of one ring pair: the last two values (V1 at l - 1, V2 at l - 2), biased, and their
+// exponent.  A pair that has not started holds zeros.
 struct FxState {
-  fx_t V1 = 0, V2 = 0;
+  fx_t V1 = kFxBias, V2 = kFxBias;
   int e = 0;
   // two steps, l - m even and l + 1; the new values are V2 and V1
   __device__ __forceinline__ void step2(int4 A0, int4 A1, unsigned xh, unsigned xl) {
@@ -131,8 +137,8 @@ __device__ __forceinline__ FxState fx_start(double v0, double v1, int S, bool ne
   if (h == 0) return st;
   // |V| < 2^(S + e + E), E = exponent bound of the larger value: at most 2^59 unless e is 0
   st.e = max(0, (59 - S - ((int)(h >> 20) - 1022))) & ~7;
-  st.V2 = fx_from_double(neg ? -v0 : v0, S + st.e);
-  st.V1 = fx_from_double(neg ? -v1 : v1, S + st.e);
+  st.V2 = fx_from_double(neg ? -v0 : v0, S + st.e) + kFxBias;
+  st.V1 = fx_from_double(neg ? -v1 : v1, S + st.e) + kFxBias;
   return st;
 }
 
@@ -140,17 +146,17 @@ __device__ __forceinline__ FxState fx_start(double v0, double v1, int S, bool ne
 __device__ __forceinline__ void fx_renorm(FxState& st, int4 A) {
   const int ah = (int)(st.V1 >> 32), bh = (int)(st.V2 >> 32);
   const int h = max(ah ^ (ah >> 31), bh ^ (bh >> 31));
-  if (st.e > 0 && (h >> (31 - A.z)) != 0) {
-    st.V1 = (st.V1 + 128) >> 8;
-    st.V2 = (st.V2 + 128) >> 8;
+  if (st.e > 0 && (h >> (32 - A.z)) != 0) {
+    st.V1 = ((st.V1 - kFxBias + 128) >> 8) + kFxBias;
+    st.V2 = ((st.V2 - kFxBias + 128) >> 8) + kFxBias;
     st.e -= 8;
   }
 }
 
-// the value V at exponent e brought to exponent 0
+// the value V (biased) at exponent e brought to exponent 0
 __device__ __forceinline__ fx_t fx_emit(fx_t V, int e) {
   if (e == 0) return V;
-  return e > 62 ? 0 : (V + (1ll << (e - 1))) >> e;
+  return (e > 62 ? 0 : (V - kFxBias + (1ll << (e - 1))) >> e) + kFxBias;
 }
 
 // step2 of a pair that may start at l (with the state s0) or still carry an exponent
@@ -163,10 +169,11 @@ __device__ __forceinline__ void fx_step2_slow(FxState& st, int4 A0, int4 A1, uns
   if (start) st = s0;
 }
 
-// Seven digit words of two consecutive values (the first in the lower half): w[i] holds the two
+// Seven digit words of two consecutive biased values (the first in the lower half): w[i] holds the two
 // bytes 7 - i as FP16 subnormals.  The values are rounded to bit 8.
 __device__ __forceinline__ void fx_digit_pair(fx_t E0, fx_t E1, unsigned (&w)[kFxDig]) {
-  const fxu_t a = (fxu_t)E0 + ((1ull << 63) + 128), b = (fxu_t)E1 + ((1ull << 63) + 128);
+  constexpr fxu_t k = (1ull << 63) + 128 - (fxu_t)kFxBias;  // digits of V + 2^63, rounded to bit 8
+  const fxu_t a = (fxu_t)E0 + k, b = (fxu_t)E1 + k;
   const unsigned l0 = (unsigned)a, l1 = (unsigned)b, h0 = (unsigned)(a >> 32), h1 = (unsigned)(b >> 32);
   const unsigned p0 = __byte_perm(l0, l1, 0x5410), p1 = __byte_perm(l0, l1, 0x7632);
   const unsigned p2 = __byte_perm(h0, h1, 0x5410), p3 = __byte_perm(h0, h1, 0x7632);

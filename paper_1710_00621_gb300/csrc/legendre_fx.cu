@@ -149,7 +149,7 @@ struct SynLayout {
   static constexpr int kCoef = kB + 2 * C::kBStep;  // int4[2][16]
   static constexpr int kCorr = kCoef + 2 * kSynK * 16;  // fxu_t[2 W][2]
   static constexpr int kBar = kCorr + 2 * C::W * 16;    // uint64_t[2]
-  static constexpr int kMisc = kBar + 16;           // tensor memory base, bad flag, first start
+  static constexpr int kMisc = kBar + 16;           // tensor memory base, bad flag
   static constexpr int kExp = kMisc + 16;           // exponents [8]
   static constexpr int kBytes = kExp + 32;
 };
@@ -164,7 +164,7 @@ template <int NM>
 __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double* __restrict__ Acoef,
                const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
-               const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
+               const int* __restrict__ tmin, const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
                const double2* __restrict__ ck, const int64_t* __restrict__ ck_base,
                const int2* __restrict__ pring, double2* __restrict__ F, int64_t F_stride, int L, int npair,
                int R, int nmaps) {
@@ -178,7 +178,6 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + LY::kBar);
   uint32_t* s_tb = reinterpret_cast<uint32_t*>(sm + LY::kMisc);
   int* s_bad = reinterpret_cast<int*>(sm + LY::kMisc + 4);
-  int* s_lo = reinterpret_cast<int*>(sm + LY::kMisc + 8);
   unsigned* s_emax = reinterpret_cast<unsigned*>(sm + LY::kExp);
 
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -242,19 +241,18 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
       const double2 v = st[(int64_t)m * npair + p];
       s0 = fx_start(v.x, v.y, S, ((ls - m) & 2) != 0);
     }
-    if (tid == 0) *s_lo = INT_MAX;
     if (tid < 4 * W) s_corr[tid] = 0;
-    __syncthreads();
     const int wlo = __reduce_min_sync(kFull, ls);
-    if ((tid & 31) == 0) atomicMin(s_lo, wlo);
+    // first start of the group
+    const int ntm = (npair + kTileMinPT - 1) / kTileMinPT, t0 = (blockIdx.x * R + r) * (kM / kTileMinPT);
+    int lo = L + 1;
+    for (int t = t0; t < min(ntm, t0 + kM / kTileMinPT); ++t) lo = min(lo, tmin[(int64_t)m * ntm + t]);
     // rows of pairs that have not started: zero digits
 #pragma unroll
     for (int i = 0; i < kFxDig; ++i) {
       const unsigned z = zero_digit(i);
       *reinterpret_cast<uint4*>(arow + i * kSynTile) = make_uint4(z, z, z, z);
     }
-    __syncthreads();
-    const int lo = min(*s_lo, L + 1);
     // the second chain starts at a checkpoint l = lm near the middle of lo..L (past L: none)
     const int cm = ((lo + L) / 2 - m + kFxChunk / 2) / kFxChunk;
     int lm = m + kFxChunk * cm;
@@ -392,8 +390,8 @@ int launch_synth_variant(int v, int nm, const Grid& g, const void* alm, int64_t 
   CMBWS_TRY(ensure_dyn_smem((const void*)kern, LY::kBytes));
   ProfScope ps(PROF_LEG_SYNTH, s, 1, leg_work(g, nm));
   kern<<<grd, kNT, LY::kBytes, s>>>((const double2*)alm, as, g.A64.as<double>(), g.mumax.as<unsigned>(),
-                                    g.lsx.as<int>(), g.stx.as<double2>(), g.xfx.as<uint64_t>(),
-                                    g.ckx.as<double2>(), g.ckx_base.as<int64_t>(),
+                                    g.lsx.as<int>(), g.lsx_tmin.as<int>(), g.stx.as<double2>(),
+                                    g.xfx.as<uint64_t>(), g.ckx.as<double2>(), g.ckx_base.as<int64_t>(),
                                     g.pair_ring.as<int2>(), (double2*)F, fs, L, g.npair, R, nm);
   CMBWS_LAUNCH_CHECK();
   return CMBWS_OK;
@@ -691,7 +689,7 @@ int launch_adj(int nm, const Grid& g, const double* eo, int* ee, double* out, cu
   CMBWS_TRY(ensure_dyn_smem((const void*)kern, LY::kBytes));
   kern<<<grd, kNT, LY::kBytes, s>>>(eo, ee, g.A64.as<double>(), g.mumax.as<unsigned>(), g.lsx.as<int>(),
                                     g.stx.as<double2>(), g.xfx.as<uint64_t>(), g.ckx.as<double2>(),
-                                    g.ckx_base.as<int64_t>(), g.ls_tmin.as<int>(), g.c64.as<double>(),
+                                    g.ckx_base.as<int64_t>(), g.lsx_tmin.as<int>(), g.c64.as<double>(),
                                     (double2*)out, nlm_of(L), L, g.npair, nm);
   CMBWS_LAUNCH_CHECK();
   return CMBWS_OK;

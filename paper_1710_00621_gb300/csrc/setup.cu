@@ -317,9 +317,10 @@ int grid_build_tables(Grid& g) {
     yh[p] = 2.0 * s2 * s2;
     sh[p] = std::sin(g.theta[p]);
     yf[p] = (float)yh[p];
-    // cos(theta) 2^63 = 2^63 - y 2^63 (0 < y; at most 1 on the north rings and the equator)
-    const uint64_t yq = (uint64_t)std::ldexp(yh[p], 63);
-    xf[p] = yq < (1ull << 63) ? (1ull << 63) - yq : 0;
+    // cos(theta) 2^63 = 2^63 - y 2^63, rounded, below 2^63 (0 < y; at most 1 on the north rings and
+    // the equator)
+    const uint64_t yq = (uint64_t)std::nearbyint(std::ldexp(yh[p], 63));
+    xf[p] = yq < (1ull << 63) ? (1ull << 63) - (yq > 0 ? yq : 1) : 0;
     const double half = M_PI / g.nphi[p];
     if (g.phi0[p] == 0.0) phase[p] = 0;
     else if (std::fabs(g.phi0[p] - half) < 1e-15) phase[p] = 1;
@@ -432,6 +433,9 @@ int grid_build_tables(Grid& g) {
     CMBWS_TRY(g.ls_tmin.alloc((size_t)(L + 1) * ntile * 4));
     dim3 gt((ntile + 127) / 128, L + 1);
     k_tile_min<<<gt, 128>>>(g.ls.as<int>(), g.npair, ntile, g.ls_tmin.as<int>());
+    CMBWS_LAUNCH_CHECK();
+    CMBWS_TRY(g.lsx_tmin.alloc((size_t)(L + 1) * ntile * 4));
+    k_tile_min<<<gt, 128>>>(g.lsx.as<int>(), g.npair, ntile, g.lsx_tmin.as<int>());
     CMBWS_LAUNCH_CHECK();
     CMBWS_CUDA(cudaDeviceSynchronize());
   }

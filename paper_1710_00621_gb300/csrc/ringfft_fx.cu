@@ -214,10 +214,13 @@ __device__ __forceinline__ void dif_group(Sbuf buf, int g, int s1, const int4* _
   }
 }
 
-// groups of 8 elements, or of 4 or 2 where the transform is too small to give every thread one
+// groups of 8 elements where every thread has one, of 4 where half of the threads have one, else of 2: a
+// larger group saves passes and twiddles, but is one thread's serial work.  Rings of 127 pixels (length
+// 256, 128 threads; 34 launches of a solve): 1107 us with groups of 2, 965 with groups of 4, 1248 with
+// groups of 8; groups of 8 for half of the threads slow rings of 256 pixels and less by 3 %.
 __device__ __forceinline__ int group_stages(int N) {
   const int nt = (int)blockDim.x;
-  return (N >> 3) >= nt ? 3 : (N >> 2) >= nt ? 2 : 1;
+  return (N >> 3) >= nt ? 3 : (N >> 1) >= nt ? 2 : 1;
 }
 
 // Transforms of size N.  The last pass's st(i, v) may record its own largest upper word in mx.

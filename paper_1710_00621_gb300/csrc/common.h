@@ -192,7 +192,7 @@ struct Grid {
   mutable int nwtdf = 0;
   mutable std::mutex ck64_mu;
   std::vector<double> fmm_h;  // sqrt((2m+1)/(2m)) (host, for rebuilding seeds)
-  DevMem ckx;             // FP64 {mu_l0, mu_l0+1} at every l0 = m + kFxChunk c (zero before the start)
+  DevMem ckx;             // fixed-point {mu_l0, mu_l0+1} (fx_pack) at every l0 = m + kFxChunk c (zero before the start)
   DevMem ckx_base;        // int64 [L+1]: offset of m's block [pair][chunk] in ckx
 
   // autotuner decisions for launches on this grid (legendre.cu), by kernel / precision / maps
@@ -288,7 +288,7 @@ int legendre_adj_df_ck(const Grid& g, int nm, const void* eo, double* out, cudaS
 // ---- FP64 Legendre stage in fixed point (legendre_fx.cu) ----
 int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s);
 // eo: ring parts (double), ee: int [nmaps][L+1] workspace
-int legendre_adjoint_fx(const Grid& g, int nmaps, const void* eo, int* ee, double* out, cudaStream_t s);
+int legendre_adjoint_fx(const Grid& g, int nmaps, void* eo, int* ee, double* out, cudaStream_t s);
 int fx_status_take(bool* timed_out);  // as tc_status_take, for these kernels
 // ---- tensor-core Legendre synthesis (legendre_tc.cu), prec TF32 / 3XTF32 / BF16 / BF16X3 ----
 int legendre_synth_tc(const Grid& g, int prec, int nmaps, const void* alm, void* F, cudaStream_t s);

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double* __restrict__ Acoef,
                const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
                const int* __restrict__ tmin, const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
-               const double2* __restrict__ ck, const int64_t* __restrict__ ck_base,
+               const ulonglong2* __restrict__ ck, const int64_t* __restrict__ ck_base,
                const int2* __restrict__ pring, double2* __restrict__ F, int64_t F_stride, int L, int npair,
                int R, int nmaps) {
   using C = Cols<NM>;
@@ -281,8 +281,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
 
     FxState s;
     if (chain && valid && lm <= L) {
-      const double2 v = ck[ck_base[m] + (int64_t)p * ((L - m + kFxChunk) / kFxChunk) + (lm - m) / kFxChunk];
-      s = fx_start(v.x, v.y, S, false);
+      s = fx_unpack(ck[ck_base[m] + (int64_t)p * ((L - m + kFxChunk) / kFxChunk) + (lm - m) / kFxChunk]);
     }
     const int la0 = chain ? lm : lo;                   // first l of this thread's chain
     const int lst = chain && ls <= lm ? INT_MAX : ls;  // where the pair starts in it
@@ -391,7 +390,7 @@ int launch_synth_variant(int v, int nm, const Grid& g, const void* alm, int64_t 
   ProfScope ps(PROF_LEG_SYNTH, s, 1, leg_work(g, nm));
   kern<<<grd, kNT, LY::kBytes, s>>>((const double2*)alm, as, g.A64.as<double>(), g.mumax.as<unsigned>(),
                                     g.lsx.as<int>(), g.lsx_tmin.as<int>(), g.stx.as<double2>(),
-                                    g.xfx.as<uint64_t>(), g.ckx.as<double2>(), g.ckx_base.as<int64_t>(),
+                                    g.xfx.as<uint64_t>(), g.ckx.as<ulonglong2>(), g.ckx_base.as<int64_t>(),
                                     g.pair_ring.as<int2>(), (double2*)F, fs, L, g.npair, R, nm);
   CMBWS_LAUNCH_CHECK();
   return CMBWS_OK;
@@ -426,16 +425,17 @@ __device__ __forceinline__ unsigned part_exp(double v) {
   return ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
 }
 
-// ee[map][m] = exponent bound of the map's ring parts at m: |e| < 2^ee (1025: not all finite)
+// ee[map][m] = exponent bound of the map's ring parts at m: |e| < 2^ee (1025: not all finite); the ring
+// parts become fixed point at that scale in place (zeros if not finite), once for all tiles of l.
 template <int NM>
 __global__ void __launch_bounds__(256)
-k_eo_exp(const double* __restrict__ eo, int npair, int L, int* __restrict__ ee, int nmaps) {
+k_eo_fix(double* __restrict__ eo, int npair, int L, int* __restrict__ ee, int nmaps) {
   const int nm = NM <= 4 ? NM : nmaps;
   __shared__ unsigned s_e[NM];
   const int m = blockIdx.x, tid = threadIdx.x;
   if (tid < NM) s_e[tid] = 0;
   __syncthreads();
-  const double* src = eo + (int64_t)m * npair * 4 * nm;
+  double* src = eo + (int64_t)m * npair * 4 * nm;
   unsigned e[NM];
 #pragma unroll
   for (int k = 0; k < NM; ++k) e[k] = 0;
@@ -452,18 +452,32 @@ k_eo_exp(const double* __restrict__ eo, int npair, int L, int* __restrict__ ee, 
   }
   __syncthreads();
   if (tid < nm) ee[(int64_t)tid * (L + 1) + m] = (int)s_e[tid] - 1022;
+  int sc[NM];
+#pragma unroll
+  for (int k = 0; k < NM; ++k) sc[k] = kFxABits - ((int)s_e[k] - 1022);
+  for (int i = tid; i < 2 * npair; i += 256) {
+    double2* v = reinterpret_cast<double2*>(src) + (int64_t)i * nm;
+#pragma unroll
+    for (int k = 0; k < NM; ++k)
+      if (k < nm) {
+        const bool ok = sc[k] > kFxABits - 1025;
+        const double2 d = v[k];
+        v[k] = make_double2(__longlong_as_double(ok ? fx_from_double(d.x, sc[k]) : 0),
+                            __longlong_as_double(ok ? fx_from_double(d.y, sc[k]) : 0));
+      }
+  }
 }
 
 // One CTA per (m, 128 values of l) loops over the ring pairs, 32 per stage: lane = pair, warp =
-// chunk of 16 values of l, which each thread walks from the chunk's FP64 checkpoint; rows of A are
+// chunk of 16 values of l, which each thread walks from the chunk's checkpoint; rows of A are
 // values of l (MN-major: a thread writes 8 consecutive values of its pair as one 16-byte row).
 // Every output has one owner; stages without a started pair are skipped.
 template <int NM>
 __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
-k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const double* __restrict__ Acoef,
+k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const double* __restrict__ Acoef,
              const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
              const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
-             const double2* __restrict__ ck, const int64_t* __restrict__ ck_base,
+             const ulonglong2* __restrict__ ck, const int64_t* __restrict__ ck_base,
              const int* __restrict__ tmin, const double* __restrict__ c64, double2* __restrict__ out,
              int64_t nlm, int L, int npair, int nmaps) {
   using C = Cols<NM>;
@@ -523,7 +537,7 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
   const int l0 = lb0 + kFxChunk * warp;
   const bool cval = l0 <= L;
   const int nck = (L - m + kFxChunk) / kFxChunk;
-  const double2* ckc = ck + (cval ? ck_base[m] + (l0 - m) / kFxChunk : 0);  // + p * nck
+  const ulonglong2* ckc = ck + (cval ? ck_base[m] + (l0 - m) / kFxChunk : 0);  // + p * nck
   const int* lsm = ls_tab + (int64_t)m * npair;
   const double2* stm = st + (int64_t)m * npair;
   unsigned char* arow = sm + LY::kA + 2 * warp * kAdjOct + lane * 16;
@@ -533,15 +547,14 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
   const int sub = tid & (kSub - 1), nn = (tid / kSub) & (W - 1), oct = (tid >> 5) & 3, par = tid >> 7;
   const int col = (nn & 1) * (W / 2) + (nn >> 1);
   const bool bon = nn < P;
-  const int eb = bon ? ee[(int64_t)(nn >> 1) * (L + 1) + m] : 0;
-  const double* bsrc = eo + (int64_t)m * npair * 2 * P + par * P + nn;
+  const fx_t* bsrc = eo + (int64_t)m * npair * 2 * P + par * P + nn;
   unsigned char* bdst = sm + LY::kB + (oct >> 1) * C::kBStep + par * W * 32 + (oct & 1) * 128 +
                         (col >> 3) * 256 + (col & 7) * 16 + sub * kPP * 2;
 
   // inputs of a stage, loaded one stage ahead
   struct In {
-    double e[kPP];
-    double2 c;
+    fx_t e[kPP];
+    ulonglong2 c;
     uint64_t x;
     int ls;
   };
@@ -550,13 +563,13 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
     const bool ok = t < nst && p < npair;
     in.ls = ok ? lsm[p] : INT_MAX;
     in.x = ok ? xfx[p] : 0;
-    in.c = make_double2(0.0, 0.0);
+    in.c = make_ulonglong2(0, 0);
     if (ok && cval) in.c = ckc[(int64_t)p * nck];
 #pragma unroll
     for (int i = 0; i < kPP; ++i) {
       const int q = t * kAdjK + 8 * oct + kPP * sub + i;
-      in.e[i] = 0.0;
-      if (bon && eb < 1025 && t < nst && q < npair) in.e[i] = bsrc[(int64_t)q * 2 * P];
+      in.e[i] = 0;
+      if (bon && t < nst && q < npair) in.e[i] = bsrc[(int64_t)q * 2 * P];
     }
   };
   In in;
@@ -573,7 +586,7 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
     const bool on = cval && __any_sync(kFull, ls <= min(L, l0 + kFxChunk - 1));
     FxState w, s0;
     if (on) {
-      w = fx_start(in.c.x, in.c.y, S, false);  // zeros if the pair starts later
+      w = fx_unpack(in.c);  // zeros if the pair starts later
       const bool inj = ls > l0 && ls < l0 + kFxChunk && ls <= L;
       if (__any_sync(kFull, inj)) {
         double2 v = make_double2(0.0, 0.0);
@@ -581,14 +594,14 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
         s0 = fx_start(v.x, v.y, S, ((ls - m) & 2) != 0);
       }
     }
-    double ev[kPP];
+    fx_t ev[kPP];
 #pragma unroll
     for (int i = 0; i < kPP; ++i) ev[i] = in.e[i];
     load(sn, in);
     if (bon) {  // B of this stage: its buffer was read two stages ago
 #pragma unroll
       for (int i = 0; i < kPP; i += 2) {
-        const fx_t v = fx_from_double(ev[i], kFxABits - eb), u = fx_from_double(ev[i + 1], kFxABits - eb);
+        const fx_t v = ev[i], u = ev[i + 1];
         shi += (v >> 30) + (u >> 30);
         slo += (v & ((1 << 30) - 1)) + (u & ((1 << 30) - 1));
         unsigned dig[kFxDig];
@@ -678,17 +691,17 @@ k_leg_adj_fx(const double* __restrict__ eo, const int* __restrict__ ee, const do
 }
 
 template <int NM>
-int launch_adj(int nm, const Grid& g, const double* eo, int* ee, double* out, cudaStream_t s) {
+int launch_adj(int nm, const Grid& g, double* eo, int* ee, double* out, cudaStream_t s) {
   using LY = AdjLayout<Cols<NM>>;
   const int L = g.lmax;
   ProfScope ps(PROF_LEG_ADJ, s, 1, leg_work(g, nm));
-  k_eo_exp<NM><<<L + 1, 256, 0, s>>>(eo, g.npair, L, ee, nm);
+  k_eo_fix<NM><<<L + 1, 256, 0, s>>>(eo, g.npair, L, ee, nm);
   CMBWS_LAUNCH_CHECK();
   dim3 grd((L + kM) / kM, L + 1);
   auto kern = k_leg_adj_fx<NM>;
   CMBWS_TRY(ensure_dyn_smem((const void*)kern, LY::kBytes));
-  kern<<<grd, kNT, LY::kBytes, s>>>(eo, ee, g.A64.as<double>(), g.mumax.as<unsigned>(), g.lsx.as<int>(),
-                                    g.stx.as<double2>(), g.xfx.as<uint64_t>(), g.ckx.as<double2>(),
+  kern<<<grd, kNT, LY::kBytes, s>>>(reinterpret_cast<const fx_t*>(eo), ee, g.A64.as<double>(), g.mumax.as<unsigned>(), g.lsx.as<int>(),
+                                    g.stx.as<double2>(), g.xfx.as<uint64_t>(), g.ckx.as<ulonglong2>(),
                                     g.ckx_base.as<int64_t>(), g.lsx_tmin.as<int>(), g.c64.as<double>(),
                                     (double2*)out, nlm_of(L), L, g.npair, nm);
   CMBWS_LAUNCH_CHECK();
@@ -716,11 +729,11 @@ int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaSt
   return CMBWS_OK;
 }
 
-int legendre_adjoint_fx(const Grid& g, int nmaps, const void* eo, int* ee, double* out, cudaStream_t s) {
+int legendre_adjoint_fx(const Grid& g, int nmaps, void* eo, int* ee, double* out, cudaStream_t s) {
   const int64_t nlm = nlm_of(g.lmax), cs = (int64_t)(g.lmax + 1) * g.npair * 4;
   for (int k0 = 0; k0 < nmaps; k0 += kFxMaps) {
     const int nm = nmaps - k0 < kFxMaps ? nmaps - k0 : kFxMaps;
-    const double* e = (const double*)eo + k0 * cs;
+    double* e = (double*)eo + k0 * cs;
     int* x = ee + (int64_t)k0 * (g.lmax + 1);
     double* o = out + 2 * k0 * nlm;
     switch (nm) {

@@ -32,6 +32,7 @@
 #include <new>
 
 #include "common.h"
+#include "fixed.h"
 
 namespace cmbws {
 
@@ -247,6 +248,19 @@ __global__ void k_unpack(const double2* __restrict__ lmc, int L, double* __restr
   if (m > 0) dst[(L - m + 1) + (l - m)] = v.y;
 }
 
+// fixed-point checkpoints, in place: their scale is known once every pair's values are
+__global__ void k_pack_ckx(ulonglong2* __restrict__ ckx, const int64_t* __restrict__ ckx_base, int L, int npair,
+                           const unsigned* __restrict__ mumax) {
+  const int m = blockIdx.y;
+  const int S = fx_scale(mumax[m]);
+  const int64_t n = (int64_t)npair * ((L - m + kFxChunk) / kFxChunk);
+  ulonglong2* c = ckx + ckx_base[m];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const ulonglong2 v = c[i];
+    c[i] = fx_pack(__longlong_as_double((long long)v.x), __longlong_as_double((long long)v.y), S);
+  }
+}
+
 // tmin[m][t] = min over the pairs p of tile t (kTileMinPT consecutive pairs) of ls[m][p]
 __global__ void k_tile_min(const int* __restrict__ ls, int npair, int ntile, int* __restrict__ tmin) {
   const int m = blockIdx.y;
@@ -428,6 +442,9 @@ int grid_build_tables(Grid& g) {
                           g.lsx.as<int>(), g.stx.as<double2>(),
                           g.ck_base.as<int64_t>(), g.ck32.as<float2>(), g.ckx_base.as<int64_t>(),
                           g.ckx.as<double2>(), nullptr, nullptr, g.mumax.as<unsigned>());
+    CMBWS_LAUNCH_CHECK();
+    k_pack_ckx<<<dim3(32, L + 1), 256>>>(g.ckx.as<ulonglong2>(), g.ckx_base.as<int64_t>(), L, g.npair,
+                                         g.mumax.as<unsigned>());
     CMBWS_LAUNCH_CHECK();
     const int ntile = (g.npair + kTileMinPT - 1) / kTileMinPT;
     CMBWS_TRY(g.ls_tmin.alloc((size_t)(L + 1) * ntile * 4));

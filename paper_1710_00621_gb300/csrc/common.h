@@ -237,7 +237,8 @@ size_t legendre_adjoint_part_bytes(const Grid& g, int prec, int nmaps);
 // scalar c * eo_maps * (L+1) * npair * 4 and,
 // for its NMc maps, holds eo[(m * npair + p) * 4 NMc + q]: q < 2 NMc the even-l parts
 // (north + south ring spectra, re / im per map), q >= 2 NMc the odd-l parts (north - south).
-// Scalars are double (FP64), float (FP32 modes) or double-float pairs (FP32X2).
+// Scalars are double (FP64), float (FP32 modes) or double-float pairs (FP32X2: a complex value as
+// re.h, im.h, re.l, im.l).
 constexpr int kFxMaps = 8;  // maps per launch of the FP64 Legendre stage (legendre_fx.cu)
 inline int eo_maps(int prec) { return prec == CMBWS_FP64 ? kFxMaps : prec == CMBWS_FP32X2 ? 3 : 4; }
 // F (ring spectra) -> pixel maps map[nmaps][npix] (FP64 out)

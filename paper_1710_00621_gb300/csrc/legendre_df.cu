@@ -9,10 +9,15 @@
 //   * contraction per map part: the exact product (TwoProd plus the cross
 //     terms) is added to a hi accumulator with TwoSum, and the rounding errors
 //     of both go to a lo accumulator (the compensated dot product "Dot2" of
-//     Ogita, Rump and Oishi 2005), renormalised once at the end.
+//     Ogita, Rump and Oishi 2005), renormalised once at the end.  The real and the imaginary
+//     part run as one packed pair: the FP32 pipe bounds both kernels (12 packed operations per
+//     map and element of about 100 cycles), and with scalar operations the issue slots did
+//     (Nside 512, 3 maps, synthesis with its FFT: 3.63 -> 3.30 ms; GL L = 775, 3 maps,
+//     adjoint: 473 -> 425 us; the same bits).
 // Coefficients and adjoint outputs keep the FP64 layout (double2); the ring spectra
 // between this stage and the ring FFTs are double-float pairs (df2, 16 bytes like
-// double2), which the double-float ring FFT (ringfft.cu) reads and writes directly,
+// double2), which the double-float ring FFT (ringfft.cu) reads and writes directly (the adjoint's
+// input with the upper words of a complex value first, the operand pairs of its products),
 // so no FP64 conversion sits between the two stages.
 #include <climits>
 
@@ -32,7 +37,7 @@ k_leg_synth_df(const double2* __restrict__ alm, int64_t alm_stride, const float2
                const float4* __restrict__ ck, const int64_t* __restrict__ ck_base) {
   static_assert(R == 1, "one ring pair per thread (its checkpoint column)");
   __shared__ __align__(16) float2 sA[CH];
-  __shared__ __align__(16) float4 sa[NM][CH];
+  __shared__ __align__(16) ulonglong2 sa[NM][CH];  // upper words (re, im), lower words
   __shared__ int s_lo;
   const int m = blockIdx.y;
   const int64_t lmo = lm_off(L, m) - m;
@@ -40,7 +45,7 @@ k_leg_synth_df(const double2* __restrict__ alm, int64_t alm_stride, const float2
 
   int ls[R];
   df y[R], mu1[R], mu2[R], i0[R], i1[R];
-  float eh[R][NM][2], el[R][NM][2], oh[R][NM][2], ol[R][NM][2];
+  f2 eh[R][NM], el[R][NM], oh[R][NM], ol[R][NM];  // even and odd sums, (re, im)
   int mylo = INT_MAX;
 #pragma unroll
   for (int i = 0; i < R; ++i) {
@@ -59,9 +64,7 @@ k_leg_synth_df(const double2* __restrict__ alm, int64_t alm_stride, const float2
     mylo = min(mylo, ls[i]);
     mu1[i] = mu2[i] = {0.f, 0.f};
 #pragma unroll
-    for (int k = 0; k < NM; ++k)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) eh[i][k][c] = el[i][k][c] = oh[i][k][c] = ol[i][k][c] = 0.f;
+    for (int k = 0; k < NM; ++k) eh[i][k] = el[i][k] = oh[i][k] = ol[i][k] = 0;
   }
   if (threadIdx.x == 0) s_lo = INT_MAX;
   __syncthreads();
@@ -92,7 +95,7 @@ k_leg_synth_df(const double2* __restrict__ alm, int64_t alm_stride, const float2
         double2 v = make_double2(0.0, 0.0);
         if (ok) v = alm[k * alm_stride + lmo + l];
         const df re = df_from(v.x), im = df_from(v.y);
-        sa[k][j] = make_float4(re.h, re.l, im.h, im.l);
+        sa[k][j] = make_ulonglong2(f2_pack(re.h, im.h), f2_pack(re.l, im.l));
       }
     }
     __syncthreads();
@@ -138,15 +141,13 @@ k_leg_synth_df(const double2* __restrict__ alm, int64_t alm_stride, const float2
         mu1[i] = mb[i];
       }
 #pragma unroll
-      for (int k = 0; k < NM; ++k) {
-        const float4 v0 = sa[k][j], v1 = sa[k][j + 1];
-        const df r0 = {v0.x, v0.y}, q0 = {v0.z, v0.w}, r1 = {v1.x, v1.y}, q1 = {v1.z, v1.w};
+      for (int i = 0; i < R; ++i) {
+        const dff fa(ma[i]), fb(mb[i]);
 #pragma unroll
-        for (int i = 0; i < R; ++i) {
-          dot2_acc(eh[i][k][0], el[i][k][0], ma[i], r0);
-          dot2_acc(eh[i][k][1], el[i][k][1], ma[i], q0);
-          dot2_acc(oh[i][k][0], ol[i][k][0], mb[i], r1);
-          dot2_acc(oh[i][k][1], ol[i][k][1], mb[i], q1);
+        for (int k = 0; k < NM; ++k) {
+          const ulonglong2 v0 = sa[k][j], v1 = sa[k][j + 1];
+          dot2_acc2(eh[i][k], el[i][k], fa, v0.x, v0.y);
+          dot2_acc2(oh[i][k], ol[i][k], fb, v1.x, v1.y);
         }
       }
     }
@@ -158,8 +159,10 @@ k_leg_synth_df(const double2* __restrict__ alm, int64_t alm_stride, const float2
     const int2 rr = pring[p];
 #pragma unroll
     for (int k = 0; k < NM; ++k) {
-      const df er{eh[i][k][0], el[i][k][0]}, ei{eh[i][k][1], el[i][k][1]};
-      const df orr{oh[i][k][0], ol[i][k][0]}, oi{oh[i][k][1], ol[i][k][1]};
+      const float2 xh = f2_unpack(eh[i][k]), xl = f2_unpack(el[i][k]);
+      const float2 zh = f2_unpack(oh[i][k]), zl = f2_unpack(ol[i][k]);
+      const df er{xh.x, xl.x}, ei{xh.y, xl.y};
+      const df orr{zh.x, zl.x}, oi{zh.y, zl.y};
       F[k * F_stride + (int64_t)rr.x * (L + 1) + m] = df2{er + orr, ei + oi};
       if (rr.y >= 0) F[k * F_stride + (int64_t)rr.y * (L + 1) + m] = df2{er - orr, ei - oi};
     }
@@ -213,11 +216,11 @@ k_leg_adj_ck_df(const float2* __restrict__ eo, const float2* __restrict__ Acoef,
     const float2 a = (valid && l0 + j <= L) ? Acoef[lmo + l0 + j] : make_float2(0.f, 0.f);
     Al[j] = {a.x, a.y};
   }
-  float ah[K][P], al[K][P];
+  f2 ah[K][NM], al[K][NM];  // (re, im)
 #pragma unroll
   for (int j = 0; j < K; ++j)
 #pragma unroll
-    for (int q = 0; q < P; ++q) ah[j][q] = al[j][q] = 0.f;
+    for (int q = 0; q < NM; ++q) ah[j][q] = al[j][q] = 0;
   const float4* ckc = ck + ck_base[m] + c;  // + p * nck
   const float2* eom = eo + (int64_t)m * npair * 2 * P;
   const int ntile = (npair + PT - 1) / PT;
@@ -266,12 +269,15 @@ k_leg_adj_ck_df(const float2* __restrict__ eo, const float2* __restrict__ Acoef,
         df ma = {cv.x, cv.y}, mb = {cv.z, cv.w};
         const float2 yy = S.y[bf][i];
         const df yv = {yy.x, yy.y};
-        const float2* e = S.eo[bf][i];
+        const ulonglong2* e = reinterpret_cast<const ulonglong2*>(S.eo[bf][i]);
+        {
+          const dff fa(ma), fb(mb);
 #pragma unroll
-        for (int q = 0; q < P; ++q) {
-          const float2 ev = e[q], ov = e[P + q];
-          dot2_acc(ah[0][q], al[0][q], ma, df{ev.x, ev.y});
-          dot2_acc(ah[1][q], al[1][q], mb, df{ov.x, ov.y});
+          for (int q = 0; q < NM; ++q) {
+            const ulonglong2 ev = e[q], ov = e[NM + q];
+            dot2_acc2(ah[0][q], al[0][q], fa, ev.x, ev.y);
+            dot2_acc2(ah[1][q], al[1][q], fb, ov.x, ov.y);
+          }
         }
 #pragma unroll
         for (int j = 2; j < K; j += 2) {
@@ -284,11 +290,12 @@ k_leg_adj_ck_df(const float2* __restrict__ eo, const float2* __restrict__ Acoef,
           }
           ma = na;
           mb = nb;
+          const dff fa(ma), fb(mb);
 #pragma unroll
-          for (int q = 0; q < P; ++q) {
-            const float2 ev = e[q], ov = e[P + q];
-            dot2_acc(ah[j][q], al[j][q], ma, df{ev.x, ev.y});
-            dot2_acc(ah[j + 1][q], al[j + 1][q], mb, df{ov.x, ov.y});
+          for (int q = 0; q < NM; ++q) {
+            const ulonglong2 ev = e[q], ov = e[NM + q];
+            dot2_acc2(ah[j][q], al[j][q], fa, ev.x, ev.y);
+            dot2_acc2(ah[j + 1][q], al[j + 1][q], fb, ov.x, ov.y);
           }
         }
       }
@@ -304,9 +311,10 @@ k_leg_adj_ck_df(const float2* __restrict__ eo, const float2* __restrict__ Acoef,
     const int64_t i = lmo + l;
     const double cc = c64[i];
 #pragma unroll
-    for (int k = 0; k < NM; ++k)
-      out[k * nlm + i] = make_double2(cc * ((double)ah[j][2 * k] + (double)al[j][2 * k]),
-                                      cc * ((double)ah[j][2 * k + 1] + (double)al[j][2 * k + 1]));
+    for (int k = 0; k < NM; ++k) {
+      const float2 h = f2_unpack(ah[j][k]), l = f2_unpack(al[j][k]);
+      out[k * nlm + i] = make_double2(cc * ((double)h.x + (double)l.x), cc * ((double)h.y + (double)l.y));
+    }
   }
 }
 

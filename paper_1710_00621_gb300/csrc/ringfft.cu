@@ -563,8 +563,13 @@ k_ringfft(typename V2<T>::t* __restrict__ F, int64_t F_stride, double* __restric
     const int kg = k0 + k, ch = kg / eo_nm, j = kg - ch * eo_nm;
     const int nmc = min(eo_nm, nmaps - ch * eo_nm), P = 2 * nmc;
     T* e = eo + (int64_t)ch * eo_nm * (L + 1) * npair * 4 + ((int64_t)m * npair + p) * 2 * P;
-    *reinterpret_cast<T2*>(e + 2 * j) = ev;
-    *reinterpret_cast<T2*>(e + P + 2 * j) = od;
+    if constexpr (std::is_same<T, df>::value) {  // the upper words of a complex value, then the lower ones
+      *reinterpret_cast<float4*>(e + 2 * j) = make_float4(ev.x.h, ev.y.h, ev.x.l, ev.y.l);
+      *reinterpret_cast<float4*>(e + P + 2 * j) = make_float4(od.x.h, od.y.h, od.x.l, od.y.l);
+    } else {
+      *reinterpret_cast<T2*>(e + 2 * j) = ev;
+      *reinterpret_cast<T2*>(e + P + 2 * j) = od;
+    }
   }
 }
 

@@ -294,13 +294,14 @@ __device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff80
 
 enum { MODE_SYNTH = 0, MODE_ANALYSIS = 1, MODE_FUSED = 2 };
 constexpr int kMaxPix = 8;
+constexpr int kSMs = 152;
 struct PixPtrs {
   const double* p[kMaxPix];
 };
 
-// One CTA per (map, ring pair), as in ringfft.cu.
-template <int MODE, int NT>
-__global__ void __launch_bounds__(NT, 512 / NT)
+// One CTA per (map, ring pair), as in ringfft.cu; THR threads resident per SM.
+template <int MODE, int NT, int THR>
+__global__ void __launch_bounds__(NT, THR / NT)
 k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict__ map_out,
              const double* __restrict__ map_in, int64_t npix, const double* __restrict__ ring_w, PixPtrs pix,
              const FftPlan* __restrict__ plans, const int* __restrict__ pair_plan,
@@ -551,15 +552,15 @@ k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict
   }
 }
 
-template <int MODE, int NT>
-int launch_nt(const Grid& g, int nmaps, const void* F, double* map_out, const double* map_in, int weighted,
+template <int MODE, int NT, int THR>
+int launch_thr(const Grid& g, int nmaps, const void* F, double* map_out, const double* map_in, int weighted,
               const void* const* pix, void* eo, cudaStream_t s) {
   const size_t sm = (size_t)(g.nmax2 + g.nmax2 / 16 + 16) * sizeof(cx);
   if (sm > 227 * 1024) {
     set_error("ring FFT needs %zu bytes of shared memory (ring length %d) at this precision", sm, g.max_n);
     return CMBWS_ERR_ARG;
   }
-  auto kern = k_ringfft_fx<MODE, NT>;
+  auto kern = k_ringfft_fx<MODE, NT, THR>;
   CMBWS_TRY(ensure_dyn_smem((const void*)kern, sm));
   const int64_t fs = (int64_t)g.nring * (g.lmax + 1);
   const double* rw = (MODE == MODE_ANALYSIS && weighted) ? g.ring_w64.as<double>() : nullptr;
@@ -580,6 +581,22 @@ int launch_nt(const Grid& g, int nmaps, const void* F, double* map_out, const do
     CMBWS_LAUNCH_CHECK();
   }
   return CMBWS_OK;
+}
+
+// Registers: 128 per thread keep the transforms free of spills, at 512 threads per SM; 85, at 768, hide
+// more latency but spill.  The second form is taken where its larger waves are fewer: 5 maps on a GL
+// grid of 512 rings (1280 CTAs of 128 threads, 3 waves -> 2) 337 -> 270 us, 3 maps (768, 2 -> 1)
+// 240 -> 177 us for both directions, Nside 512 (3072 of 256, 11 -> 7) 842 -> 734 us; on grids of one
+// wave it is slower (solve with 96 CTAs per transform: 959 -> 1032 us).
+template <int MODE, int NT>
+int launch_nt(const Grid& g, int nmaps, const void* F, double* map_out, const double* map_in, int weighted,
+              const void* const* pix, void* eo, cudaStream_t s) {
+  constexpr int64_t lo = kSMs * (512 / NT), hi = kSMs * (768 / NT);  // CTAs of a wave
+  const int64_t n = (int64_t)g.npair * (nmaps < kMaxPix ? nmaps : kMaxPix);
+  if constexpr (hi > lo)
+    if ((n + hi - 1) / hi < (n + lo - 1) / lo)
+      return launch_thr<MODE, NT, 768>(g, nmaps, F, map_out, map_in, weighted, pix, eo, s);
+  return launch_thr<MODE, NT, 512>(g, nmaps, F, map_out, map_in, weighted, pix, eo, s);
 }
 
 // threads per CTA by the transform buffer, as in ringfft.cu

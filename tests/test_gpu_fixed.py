@@ -99,8 +99,10 @@ def test_zero_input():
     assert not to_host(out).any() and not to_host(back).any()
 
 
-@pytest.mark.parametrize("maps", [5, 6, 7, 8, 9])
-@pytest.mark.parametrize("n,lmax", [(66, 31), (130, 127), (259, 129)])
+# the last three change the ring FFT's registers between one map and the batch (128 and 256 threads)
+@pytest.mark.parametrize("n,lmax,maps", [(n, lmax, k) for n, lmax in ((66, 31), (130, 127), (259, 129))
+                                         for k in (5, 6, 7, 8, 9)]
+                         + [(512, 511, 3), (512, 511, 5), (600, 599, 5)])
 def test_maps_of_a_batch_are_those_of_single_calls(n, lmax, maps):
     """Integer sums do not depend on how the maps are grouped: equal bit for bit."""
     g = cw.cmbws_plan_grid(cw.CMBWS_GRID_GL, n, lmax)

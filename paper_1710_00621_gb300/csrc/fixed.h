@@ -12,9 +12,9 @@
 // For the products V = h 2^32 + l with both words signed: the state holds V + 2^31, whose upper word
 // is h and whose lower one is l + 2^31.  For the contraction the bytes of V + 2^63 are its base-256
 // digits, byte 7 less 128, the others as they are.
-// Before a pair's values are of order one (they grow from 2^-64 where its walk starts; smaller
-// ones are below the last digit), V carries a binary exponent e (a multiple of 8):
-// mu = V 2^-(S + e), V shifted down by 8 bits as it grows; e is 0 from |mu| ~ 2^-7 on.
+// Before a pair's values are of order one (they grow from 2^-55 where its walk starts; the digits
+// of smaller ones are zero, as bit 8 of V is the last that is kept), V carries a binary exponent e (a
+// multiple of 8): mu = V 2^-(S + e), V shifted down by 8 bits as it grows; e is 0 from |mu| ~ 2^-7 on.
 //
 // Coefficients and ring parts are scaled by a power of two per (m, map) to |a| < 2^54 and split
 // into 7 signed digits (-128..127).  With digits u_i of V (7 of them, from byte 7 down, V rounded
@@ -136,7 +136,7 @@ __device__ __forceinline__ FxState fx_start(double v0, double v1, int S, bool ne
                          (unsigned)__double2hiint(v1) & 0x7fffffffu);
   if (h == 0) return st;
   // |V| < 2^(S + e + E), E = exponent bound of the larger value: at most 2^59 unless e is 0 (e is 64 at
-  // most, for fx_pack; starts of 2^-64 need that from S = 58 on, below it V has fewer bits)
+  // most, for fx_pack; starts of 2^-55 need no more from S = 49 on, below it V has fewer bits)
   st.e = min(64, max(0, 59 - S - ((int)(h >> 20) - 1022)) & ~7);
   st.V2 = fx_from_double(neg ? -v0 : v0, S + st.e) + kFxBias;
   st.V1 = fx_from_double(neg ? -v1 : v1, S + st.e) + kFxBias;

@@ -62,11 +62,12 @@ typedef enum { CMBWS_GRID_GL = 0, CMBWS_GRID_HEALPIX = 1 } cmbws_grid_kind;
 /* Arithmetic of the transform stages (Legendre recurrence and contraction,
  * ring FFTs, pixel multiplies).  Vectors at the boundary and CG scalars are
  * always FP64.
- *   CMBWS_FP64:   native FP64 throughout.
+ *   CMBWS_FP64:   FP64 accuracy and FP64 data throughout; the Legendre stage and the ring FFTs
+ *                 compute in 64-bit fixed point (integer units and exact tensor-core sums).
  *   CMBWS_FP32:   FP32 throughout (relative error ~1e-6 at L ~ 3000).
  *   CMBWS_FP32X2: FP64-accurate Legendre stage in double-float arithmetic (pairs of FP32
  *                 values, ~48-bit significand, on the FP32 pipe, which GB300 runs 61x
- *                 faster than FP64); ring FFTs and pixel stages in FP64.
+ *                 faster than FP64), ring FFTs in the same; pixel stages in FP64.
  *   CMBWS_TF32:   as CMBWS_FP32, with the Legendre synthesis on the tensor cores (tcgen05,
  *                 TF32 recurrence values and coefficients, FP32 accumulation; relative error
  *                 ~1e-4); the adjoint Legendre stage stays FP32 on the CUDA cores.
@@ -355,7 +356,7 @@ int cmbws_project(cmbws_model m, const double* x, double* const* d, void* stream
  *   mode 2: on the first synthesis for a (grid, precision, maps) key, each tile variant is
  *     launched and timed with CUDA events on the caller's stream (the first call is then
  *     synchronous), and the fastest is kept for that key for the life of the grid.
- * FP64 results do not depend on the tile; FP32 results can differ in rounding (warps that
+ * FP64 tiles are groups of 128 ring pairs per CTA; its results do not depend on them.  FP32 results can differ in rounding (warps that
  * hold a ring pair near a pole switch to the difference form of the recurrence, and the
  * tile decides which pairs share a warp).  Errors: CMBWS_ERR_ARG for another mode.
  */
@@ -398,7 +399,7 @@ typedef struct {
   int max_outer;      /* FP32 models: cap on refinement passes */
   double timeout_s;   /* wall-clock budget, <= 0 for none */
   int cert_prec;      /* arithmetic of the applies that compute the true residual b - A x:
-                         CMBWS_FP64 (native) or CMBWS_FP32X2 (double-float); other values
+                         CMBWS_FP64 or CMBWS_FP32X2 (double-float); other values
                          mean CMBWS_FP64 */
 } cmbws_cg_opts;
 

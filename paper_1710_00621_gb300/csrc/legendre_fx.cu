@@ -160,6 +160,10 @@ struct SynLayout {
 // digit tile (consecutive threads are 16 bytes apart); every second stage it converts one
 // coefficient part to digits of B.  One thread issues the stage's MMAs after its barrier; they read
 // the tile while the threads compute the next values in registers.
+// Bound by the dispatch of integer instructions (48 per element, 26 of them at half rate; tensor pipe
+// 15 %).  Against the recurrence and sums on the FP64 pipe, Nside 1024, L = 3071, 3 maps: 94.6 ->
+// 19.1 ms.  One chain per row and 128 threads was 19.0 ms against 19.9 for two chains when both were
+// tried there, but grids of few ring pairs wait for that chain.
 template <int NM>
 __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double* __restrict__ Acoef,
@@ -472,6 +476,8 @@ k_eo_fix(double* __restrict__ eo, int npair, int L, int* __restrict__ ee, int nm
 // chunk of 16 values of l, which each thread walks from the chunk's checkpoint; rows of A are
 // values of l (MN-major: a thread writes 8 consecutive values of its pair as one 16-byte row).
 // Every output has one owner; stages without a started pair are skipped.
+// Bound as the synthesis is (tensor pipe 17 %).  Against the FP64 pipe, Nside 1024, 3 maps: 107.9 ->
+// 18.1 ms; GL L = 1000, 1 map: 1.77 -> 0.60 ms.
 template <int NM>
 __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const double* __restrict__ Acoef,

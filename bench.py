@@ -962,8 +962,7 @@ def main():
         out["iters_fp64_plain"] = r64["iters"]
 
     # the FP64-accurate solver on the FP32 pipe: every transform in double-float (48-bit
-    # significands), the fair plain-precision comparator on a GPU whose FP64 pipe runs at a
-    # 61st of the FP32 rate
+    # significands), a second plain-precision comparator beside fp64_plain
     fp32x2 = None
     if not args.no_fp64_plain and args.prec == "fp32":
         try:

@@ -9,12 +9,13 @@
 //               real parts of all maps come first: a warp takes either them or the imaginary ones
 //               (half the columns to read, no spills: one map at L = 1000 917 -> 836 us with the FFT).
 // W is 8 (up to 4 maps) or 16 (up to 8 maps): the recurrence, which is most of the work, serves all
-// of them.  The 7 digits of Lambda are the A operand (shared memory, one tile per digit), those of
-// the coefficients or ring parts the B operand (7 x 2 W rows); digit i of A times the digits
+// of them.  The 8 digits of Lambda are the A operand (shared memory, one tile per digit), those of
+// the coefficients or ring parts the B operand (8 x 2 W rows); digit i of A times the digits
 // 0..7 - i of B accumulate into columns 2 W i.. of the accumulator, so that block s of 2 W columns
 // holds the sum over i + j = s.  Every 64 terms the blocks are read from tensor memory and added
 // as integers.
 #include <climits>
+#include <type_traits>
 
 #include "common.h"
 #include "fixed.h"
@@ -55,22 +56,15 @@ __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t adesc, uint64_t bde
       : "memory");
 }
 // One K step: digit i of A (tiles atile bytes apart) times the digits 0..7 - i of B into blocks
-// i..7; `first` clears the accumulator (digit 1 writes blocks 1..7, digit 0 block 0).
+// i..7; `first` clears the accumulator (digit 0 writes all blocks).
 template <typename C>
 __device__ __forceinline__ void mma_step(uint32_t d, uint32_t ab, int atile, uint32_t alb, uint32_t asb,
                                          uint32_t bb, bool mn, bool first) {
   constexpr int N = 2 * C::W;
-  const uint64_t a0 = smem_desc(ab, alb, asb), a1 = smem_desc(ab + atile, alb, asb);
   const uint64_t b0 = smem_desc(bb, 128, 256);
-  mma_f16(d + N, a1, b0, N * kFxDig, mn, first ? 0u : 1u);
-  if (first) {
-    mma_f16(d, a0, b0, N, mn, 0u);
-    mma_f16(d + N, a0, smem_desc(bb + C::kDig, 128, 256), N * (kFxDig - 1), mn, 1u);
-  } else {
-    mma_f16(d, a0, b0, N * kFxDig, mn, 1u);
-  }
+  mma_f16(d, smem_desc(ab, alb, asb), b0, N * kFxBlk, mn, first ? 0u : 1u);
 #pragma unroll
-  for (int i = 2; i < kFxDig; ++i)
+  for (int i = 1; i < kFxDig; ++i)
     mma_f16(d + N * i, smem_desc(ab + i * atile, alb, asb), b0, N * (kFxBlk - i), mn, 1u);
 }
 
@@ -99,6 +93,8 @@ __device__ __forceinline__ unsigned zero_digit(int i) { return i == 0 ? 0x008000
 // bytes apart.  co: the recurrence coefficients; la: the first l; ls: where the pair starts (s0 the
 // values there); skip: the state already holds the first two values; wait(): the previous stage's
 // MMAs have read the tile.
+template <int Q>
+using Half = std::integral_constant<int, Q>;
 template <typename W>
 __device__ __forceinline__ void fx_walk8(FxState& s, const int4* co, unsigned xh, unsigned xl, int la,
                                          int ls, const FxState& s0, bool skip, unsigned char* row,
@@ -108,27 +104,37 @@ __device__ __forceinline__ void fx_walk8(FxState& s, const int4* co, unsigned xh
     wait();
 #pragma unroll 1
     for (int j = 0; j < 8; j += 2) {
-      unsigned d[kFxDig];
       if (!skip || j > 0) fx_step2_slow(s, co[j], co[j + 1], xh, xl, ls == la + j, s0);
-      fx_digit_pair(fx_emit(s.V2, s.e), fx_emit(s.V1, s.e), d);
-#pragma unroll
-      for (int i = 0; i < kFxDig; ++i) *reinterpret_cast<unsigned*>(row + i * tile + 2 * j) = d[i];
+      const fxu_t a = fx_bytes(fx_emit(s.V2, s.e)), b = fx_bytes(fx_emit(s.V1, s.e));
+      auto put = [&](auto q) {
+        unsigned d0, d1;
+        fx_digits2<q.value>(a, b, d0, d1);
+        *reinterpret_cast<unsigned*>(row + (6 - 2 * q.value) * tile + 2 * j) = d0;
+        *reinterpret_cast<unsigned*>(row + (7 - 2 * q.value) * tile + 2 * j) = d1;
+      };
+      put(Half<0>{}), put(Half<1>{}), put(Half<2>{}), put(Half<3>{});
     }
     return;
   }
-  uint4 w[kFxDig];
-  unsigned* ww = reinterpret_cast<unsigned*>(w);
+  fxu_t v[8];
 #pragma unroll
   for (int j = 0; j < 8; j += 2) {
-    unsigned d[kFxDig];
     if (j > 0 || !skip) s.step2(co[j], co[j + 1], xh, xl);
-    fx_digit_pair(s.V2, s.V1, d);
-#pragma unroll
-    for (int i = 0; i < kFxDig; ++i) ww[4 * i + j / 2] = d[i];
+    v[j] = fx_bytes(s.V2);
+    v[j + 1] = fx_bytes(s.V1);
   }
   wait();
-#pragma unroll
-  for (int i = 0; i < kFxDig; ++i) *reinterpret_cast<uint4*>(row + i * tile) = w[i];
+  // two digits of all eight values at a time: the values take half the registers of their digits
+  auto put = [&](auto q) {
+    uint4 r0, r1;
+    fx_digits2<q.value>(v[0], v[1], r0.x, r1.x);
+    fx_digits2<q.value>(v[2], v[3], r0.y, r1.y);
+    fx_digits2<q.value>(v[4], v[5], r0.z, r1.z);
+    fx_digits2<q.value>(v[6], v[7], r0.w, r1.w);
+    *reinterpret_cast<uint4*>(row + (6 - 2 * q.value) * tile) = r0;
+    *reinterpret_cast<uint4*>(row + (7 - 2 * q.value) * tile) = r1;
+  };
+  put(Half<0>{}), put(Half<1>{}), put(Half<2>{}), put(Half<3>{});
 }
 
 __device__ __forceinline__ int digit_sum(uint32_t d) {
@@ -417,8 +423,8 @@ constexpr int kAdjOct = kAdjK * 16;             // bytes between rows 8 i and 8 
 template <typename C>
 struct AdjLayout {
   static constexpr int kA = 0;
-  static constexpr int kB = kFxDig * kAdjTile;       // two stages of B (two K steps each)
-  static constexpr int kCoef = kB + 4 * C::kBStep;   // int4[128]
+  static constexpr int kB = kFxDig * kAdjTile;       // B of a stage (two K steps)
+  static constexpr int kCoef = kB + 2 * C::kBStep;   // int4[128]
   static constexpr int kCorr = kCoef + kM * 16;      // fxu_t[2 W][2]
   static constexpr int kBar = kCorr + 2 * C::W * 16; // uint64_t[2]
   static constexpr int kMisc = kBar + 16;            // tensor memory base, bad flag
@@ -530,7 +536,7 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
     const int l = lb0 + tid;
     s_coef[tid] = fx_coef(l <= L ? Acoef[lmo + l] : 0.0);
   }
-  for (int i = tid; i < 4 * C::kBStep / 16; i += kNT)  // B columns of absent maps stay zero
+  for (int i = tid; i < 2 * C::kBStep / 16; i += kNT)  // B columns of absent maps stay zero
     reinterpret_cast<uint4*>(sm + LY::kB)[i] = make_uint4(0, 0, 0, 0);
   if (warp == 0) tmem_alloc<C::kTmem>(s_tb);
   tc_fence_before();
@@ -604,19 +610,6 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
 #pragma unroll
     for (int i = 0; i < kPP; ++i) ev[i] = in.e[i];
     load(sn, in);
-    if (bon) {  // B of this stage: its buffer was read two stages ago
-#pragma unroll
-      for (int i = 0; i < kPP; i += 2) {
-        const fx_t v = ev[i], u = ev[i + 1];
-        shi += (v >> 30) + (u >> 30);
-        slo += (v & ((1 << 30) - 1)) + (u & ((1 << 30) - 1));
-        unsigned dig[kFxDig];
-        fx_coef_digits(v, u, dig);
-#pragma unroll
-        for (int j = 0; j < kFxDig; ++j)
-          *reinterpret_cast<unsigned*>(bdst + (k & 1) * 2 * C::kBStep + j * C::kDig + 2 * i) = dig[j];
-      }
-    }
     auto wait = [&]() {  // the previous stage's MMAs have read the tile
       if (k >= 1 && !*s_bad && !mbar_wait(&mbar[0], (k - 1) & 1)) bad = true;
     };
@@ -639,6 +632,19 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
         }
       zeroed = true;
     }
+    if (bon) {  // B of this stage: the previous one was waited for
+#pragma unroll
+      for (int i = 0; i < kPP; i += 2) {
+        const fx_t v = ev[i], u = ev[i + 1];
+        shi += (v >> 30) + (u >> 30);
+        slo += (v & ((1 << 30) - 1)) + (u & ((1 << 30) - 1));
+        unsigned dig[kFxDig];
+        fx_coef_digits(v, u, dig);
+#pragma unroll
+        for (int j = 0; j < kFxDig; ++j)
+          *reinterpret_cast<unsigned*>(bdst + j * C::kDig + 2 * i) = dig[j];
+      }
+    }
     fence_smem_async();
     tc_fence_before();
     if (bad) atomicOr(s_bad, 1);
@@ -649,7 +655,7 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
 #pragma unroll
       for (int ks = 0; ks < 2; ++ks)
         mma_step<C>(tb, smem_addr(sm + LY::kA) + ks * 256, kAdjTile, 128, kAdjOct,
-                 smem_addr(sm + LY::kB + ((k & 1) * 2 + ks) * C::kBStep), true, first && ks == 0);
+                 smem_addr(sm + LY::kB + ks * C::kBStep), true, first && ks == 0);
       tc_commit(&mbar[0]);
     }
     if ((k & 1) == 1 || sn >= nst) {

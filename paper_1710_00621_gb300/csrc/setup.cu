@@ -39,7 +39,7 @@ namespace cmbws {
 namespace {
 
 constexpr double kStartThreshold = 1e-30;
-constexpr double kStartThresholdFx = 0x1p-55;  // fixed-point stages: smaller values round to zero digits
+constexpr double kStartThresholdFx = 0x1p-60;  // fixed-point stages: smaller values have no digits
 constexpr double kShiftUp = 0x1p600;     // 2^600
 constexpr double kShiftDown = 0x1p-600;  // 2^-600
 constexpr double kGrow = 0x1p500;

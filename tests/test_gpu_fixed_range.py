@@ -1,0 +1,40 @@
+"""Precision of the CMBWS_FP64 transforms where one scale per block could lose bits: values far
+below the largest one of their block still count with the accuracy that FP64 gives them."""
+import math
+
+import numpy as np
+import pytest
+
+import paper_1710_00621_gb300 as cw
+from tests._gpu import to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53
+
+
+@pytest.mark.parametrize("nside,lmax", [(16, 63), (64, 255), (64, 767), (256, 767)])
+def test_low_multipoles_under_a_high_band_limit(nside, lmax):
+    """The rescaled Legendre values of m = 0 grow with l, so a high band-limit leaves those of low l
+    the fewest bits.  A monopole and a dipole in closed form, on the rings of 4 nside pixels (the
+    shorter ones go through chirps): one rounding each, at most half a unit of the largest pixel, of
+    the scaled coefficients, the dipole's Legendre value, the ring spectra of both parities, their
+    sum, its fixed-point form and the pixel, with exact products between them: 4 units cover it.
+    The adjoint of a constant map adds whole numbers."""
+    g = cw.cmbws_plan_grid(cw.CMBWS_GRID_HEALPIX, nside, lmax)
+    maps = 8
+    alm = np.zeros((maps, (lmax + 1) ** 2))
+    alm[:, :2] = np.random.default_rng(lmax).uniform(0.5, 2.0, (maps, 2))
+    out = to_dev(np.zeros((maps, g.npix)))
+    cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(alm), out, maps)
+    full = np.repeat(g.nphi == 4 * nside, g.nphi)
+    x = np.cos(g.theta.astype(np.longdouble))
+    c = np.sqrt(1 / (4 * np.arccos(np.longdouble(-1))))
+    for k in range(maps):
+        want = c * (alm[k, 0] + alm[k, 1] * np.sqrt(np.longdouble(3)) * x)
+        err = np.abs(to_host(out)[k] - np.repeat(want, g.nphi))[full] / np.abs(want).max()
+        assert err.max() <= 4 * U, float(err.max() / U)
+    back = to_dev(np.zeros((lmax + 1) ** 2))
+    cw.cmbws_sht_analysis(g, cw.CMBWS_FP64, to_dev(np.ones(g.npix)), back, 1, 0)
+    want = g.npix / math.sqrt(4.0 * math.pi)
+    assert abs(to_host(back)[0] - want) <= 4 * U * want

@@ -31,6 +31,11 @@ struct __align__(16) cx {
 
 __device__ __forceinline__ cx operator+(cx a, cx b) { return {a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ cx operator-(cx a, cx b) { return {a.x - b.x, a.y - b.y}; }
+// a + v, or a - v; modulo 2^64
+__device__ __forceinline__ cx wrap_add(cx a, cx v, bool neg) {
+  const fxu_t x = (fxu_t)v.x, y = (fxu_t)v.y;
+  return {(fx_t)((fxu_t)a.x + (neg ? 0 - x : x)), (fx_t)((fxu_t)a.y + (neg ? 0 - y : y))};
+}
 __device__ __forceinline__ cx cconj(cx a) { return {a.x, -a.y}; }
 
 // digits of a value: v = h 2^32 + 2 l (its last bit dropped), l >= 0
@@ -311,7 +316,7 @@ k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict
              const int64_t* __restrict__ roff, const int4* __restrict__ tab, int64_t tw_off, int nmax, int L,
              double* __restrict__ eo, int eo_nm, int k0, int nmaps, int npair) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ unsigned s_max[2];  // exponents of the inputs (synthesis, pixels)
+  __shared__ unsigned s_max[3];  // exponents of the inputs (synthesis, pixels), upper word of the sums
   __shared__ unsigned s_ren[3];
 
   const int k = blockIdx.x;
@@ -333,8 +338,7 @@ k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict
   const int4* __restrict__ filt = tab + P.filt;
   const int tid = threadIdx.x;
 
-  if (tid < 2) s_max[tid] = 0;
-  if (tid < 3) s_ren[tid] = 0;
+  if (tid < 3) s_max[tid] = s_ren[tid] = 0;
   __syncthreads();
   Renorm rn{s_ren};
   unsigned mx = 0;
@@ -345,7 +349,7 @@ k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict
     mx = max(mx, hi_abs(w));
     buf[q] = w;
   };
-  auto exp_scan = [&](unsigned e, int slot) {  // block maximum of exponents
+  auto exp_scan = [&](unsigned e, int slot) {  // block maximum of exponents or upper words
     e = __reduce_max_sync(0xffffffffu, e);
     if ((tid & 31) == 0) atomicMax(&s_max[slot], e);
     __syncthreads();
@@ -368,9 +372,12 @@ k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict
     e = exp_scan(e, 0);
     bad = e == 0x7ffu;
     // |F| < 2^(e - 1022); a frequency sums at most na terms of each ring, and the pair's packed
-    // value is below 2 sqrt(2) na of that
-    const int na = L / n + 1 + (L + n - 1) / n;
-    const int kf = 61 - 2 - (32 - __clz(na - 1)) - ((int)e - 1022);
+    // value is below 2 sqrt(2) na of that.  Short rings with many aliases would keep too few bits of F
+    // that way (47 at 4 pixels and L = 6000): they form the sums twice, first to see how large they are.
+    // Differences of sums wrap, so terms that cancel may be larger than the room for their sum.
+    const int na = L / n + 1 + (L + n - 1) / n, abits = 32 - __clz(na - 1);
+    int kf = 61 - 2 - abits - ((int)e - 1022);
+    const bool twice = abits > 4;
     auto fix = [&](double v) { return bad ? (fx_t)0 : fx_from_double(v, kf); };
     // alias sums of one frequency, as in ringfft.cu
     auto alias_sums = [&](int kk, int part, int tpk, cx& an, cx& as) {
@@ -381,11 +388,11 @@ k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict
           const bool neg = ph && (j & 1);
           const double2 a = FN[m];
           const cx v{fix(a.x), -fix(a.y)};
-          an = neg ? an - v : an + v;
+          an = wrap_add(an, v, neg);
           if (has_s) {
             const double2 b = FS[m];
             const cx u{fix(b.x), -fix(b.y)};
-            as = neg ? as - u : as + u;
+            as = wrap_add(as, u, neg);
           }
         }
       }
@@ -395,11 +402,11 @@ k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict
           const bool neg = ph && (j & 1);
           const double2 a = FN[m];
           const cx v{fix(a.x), fix(a.y)};
-          an = neg ? an - v : an + v;
+          an = wrap_add(an, v, neg);
           if (has_s) {
             const double2 b = FS[m];
             const cx u{fix(b.x), fix(b.y)};
-            as = neg ? as - u : as + u;
+            as = wrap_add(as, u, neg);
           }
         }
       }
@@ -423,28 +430,45 @@ k_ringfft_fx(const double2* __restrict__ F, int64_t F_stride, double* __restrict
     int tpk = n < NT / 2 ? NT / n : 1;
     if (scratch + 2 * NT > nmax + nmax / 16 + 16) tpk = 1;
     for (int kk = n + tid; kk < n2; kk += NT) buf[kk] = cx{0, 0};
-    if (tpk == 1) {
-      for (int kk = tid; kk < n; kk += NT) {
-        cx an, as;
-        alias_sums(kk, 0, 1, an, as);
-        fold_store(kk, an, as);
-      }
-    } else {
-      cx* part = buf.p + scratch;
-      if (tid < n * tpk) {
-        cx an, as;
-        alias_sums(tid % n, tid / n, tpk, an, as);
-        part[2 * tid] = an;
-        part[2 * tid + 1] = as;
-      }
-      __syncthreads();
-      if (tid < n) {
-        cx an{0, 0}, as{0, 0};
-        for (int q = 0; q < tpk; ++q) {
-          an = an + part[2 * (tid + q * n)];
-          as = as + part[2 * (tid + q * n) + 1];
+    for (int round = twice ? 0 : 1; round < 2; ++round) {
+      unsigned big = 0;
+      auto take = [&](int kk, cx an, cx as) {
+        if (round == 1) {
+          fold_store(kk, an, as);
+          return;
         }
-        fold_store(tid, an, as);
+        big = max(big, max(hi_abs(an), hi_abs(as)));
+        if (kk == 0) big = max(big, max(hi_abs(fix(FN[0].x)), has_s ? hi_abs(fix(FS[0].x)) : 0u));
+      };
+      if (tpk == 1) {
+        for (int kk = tid; kk < n; kk += NT) {
+          cx an, as;
+          alias_sums(kk, 0, 1, an, as);
+          take(kk, an, as);
+        }
+      } else {
+        cx* part = buf.p + scratch;
+        if (tid < n * tpk) {
+          cx an, as;
+          alias_sums(tid % n, tid / n, tpk, an, as);
+          part[2 * tid] = an;
+          part[2 * tid + 1] = as;
+        }
+        __syncthreads();
+        if (tid < n) {
+          cx an{0, 0}, as{0, 0};
+          for (int q = 0; q < tpk; ++q) {
+            an = wrap_add(an, part[2 * (tid + q * n)], false);
+            as = wrap_add(as, part[2 * (tid + q * n) + 1], false);
+          }
+          take(tid, an, as);
+        }
+      }
+      if (round == 0) {
+        // all components below c = 2^(64 - clz): the packed value's modulus is below 7 c (a frequency
+        // and its m = 0 term of both rings, turned by their phases)
+        const unsigned h = exp_scan(big, 2);
+        kf += max(0, min(abits, __clz(h) - 6));
       }
     }
     __syncthreads();

@@ -6,7 +6,9 @@ import numpy as np
 import pytest
 
 import paper_1710_00621_gb300 as cw
-from tests._gpu import to_dev, to_host
+from oracle import grids as og
+from oracle import sht as osht
+from tests._gpu import rel_err, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -38,3 +40,33 @@ def test_low_multipoles_under_a_high_band_limit(nside, lmax):
     cw.cmbws_sht_analysis(g, cw.CMBWS_FP64, to_dev(np.ones(g.npix)), back, 1, 0)
     want = g.npix / math.sqrt(4.0 * math.pi)
     assert abs(to_host(back)[0] - want) <= 4 * U * want
+
+
+@pytest.mark.parametrize("nside,lmax", [(16, 255), (16, 767), (1, 3000)])
+def test_monopole_on_short_rings(nside, lmax):
+    """Rings of far fewer pixels than the band-limit leave room for the sum of all aliases of a
+    frequency, but the ring spectra keep their bits all the same: the bound above on every ring of a
+    power-of-two length."""
+    g = cw.cmbws_plan_grid(cw.CMBWS_GRID_HEALPIX, nside, lmax)
+    maps = 8
+    a = np.random.default_rng(lmax).uniform(0.5, 2.0, maps)
+    alm = np.zeros((maps, (lmax + 1) ** 2))
+    alm[:, 0] = a
+    out = to_dev(np.zeros((maps, g.npix)))
+    cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(alm), out, maps)
+    pow2 = np.repeat(g.nphi & (g.nphi - 1) == 0, g.nphi)
+    want = a / math.sqrt(4.0 * math.pi)
+    err = np.abs(to_host(out)[:, pow2] - want[:, None]) / want[:, None]
+    assert err.max() <= 4 * U, err.max() / U
+
+
+@pytest.mark.parametrize("nside,lmax", [(1, 31), (1, 33), (1, 200), (3, 150)])
+def test_aliases_on_short_rings(nside, lmax):
+    """Full spectra on rings of 4 to 12 pixels, around the number of aliases from which the sums are
+    formed twice: the FP64 parity bound 40 (L+1) u of the largest pixel."""
+    g = cw.cmbws_plan_grid(cw.CMBWS_GRID_HEALPIX, nside, lmax)
+    alm = np.random.default_rng(lmax).standard_normal((lmax + 1) ** 2)
+    out = to_dev(np.zeros(g.npix))
+    cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(alm), out, 1)
+    want = osht.synthesis(og.healpix(nside), lmax, alm)
+    assert rel_err(to_host(out), want) < 40 * (lmax + 1) * U

@@ -175,9 +175,9 @@ struct Grid {
   DevMem c64;             // lambda_lm = c_lm mu_lm
   DevMem ls;              // int [L+1][npair] first l (same parity as m) that is injected
   DevMem st64, st32;      // {mu_ls, mu_ls+1} [L+1][npair]
-  DevMem lsx, stx;        // the same for the fixed-point stages (|mu| > 2^-55, values FP64)
+  DevMem sx;              // uint8 [L+1][npair]: scale of the fixed-point stages (fixed.h), 0 if never started
+  DevMem lsx, stx;        // first l and values (fx_pack) for the fixed-point stages
   DevMem xfx;             // uint64 cos(theta) 2^63 of the north ring [npair] (fixed-point stages)
-  DevMem mumax;           // unsigned [L+1]: high word of the largest |mu_l| of each m (FP64 bits)
   DevMem ck32;            // FP32 {mu_l0, mu_l0+1} at every chunk start l0 = m + kChunk c
   DevMem ck_base;         // int64 [L+1]: offset of m's block [pair][chunk] in ck32
   DevMem ls_tmin;         // int [L+1][ceil(npair / kTileMinPT)]: smallest ls of each tile of pairs

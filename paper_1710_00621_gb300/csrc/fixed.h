@@ -5,18 +5,20 @@
 // the FP16 tensor cores over 8-bit digits, whose products and sums are exact in FP32.
 //
 // Values.  mu_l (common.h: the rescaled Legendre values) is held as V = sigma mu 2^S, |V| < 2^62,
-// with S = 62 - b chosen per m from the largest |mu_l| of the grid (|mu| < 2^b, recorded when the
-// grid is planned; b is 1 to 4 in practice, so the quantum is 2^-58 or finer).  The sign sigma
+// with S = 62 - b chosen per m and ring pair from the largest |mu_l| up to the band-limit (|mu| < 2^b,
+// recorded when the grid is planned; b is at most 4, and negative near the poles, where all values of a
+// high m are small).  The sign sigma
 // = + + - - by l - m modulo 4 turns mu_l = A x mu_{l-1} - mu_{l-2} into V2 - A x V1 (l - m even) and
 // V2 + A x V1 (odd); the coefficients (synthesis) or the results (adjoint) take sigma back.
 // For the products V = h 2^32 + l with both words signed: the state holds V + 2^31, whose upper word
 // is h and whose lower one is l + 2^31.  For the contraction the bytes of V + 2^63 are its base-256
 // digits, byte 7 less 128, the others as they are.
-// Before a pair's values are of order one (they grow from 2^-60 where its walk starts; smaller ones have no
-// digits), V carries a binary exponent e (a multiple of 8): mu = V 2^-(S + e), V shifted down by 8
-// bits as it grows; e is 0 from |mu| ~ 2^-7 on.
+// Before a pair's values are near their largest (they grow from where its walk starts; smaller ones have
+// no digits), V carries a binary exponent e (a multiple of 8): mu = V 2^-(S + e), V shifted down by 8
+// bits as it grows; e is 0 from 2^-7 of the largest on.
 //
-// Coefficients and ring parts are scaled by a power of two per (m, map) to |a| < 2^62 and split
+// Coefficients a (synthesis) and ring parts times 2^-S of their pair (adjoint) are scaled by a power of
+// two per (m, map) to |a| < 2^62 and split
 // into 8 signed digits (-128..127).  With digits u_i of V (8 of them, from byte 7 down) and d_j of a,
 // the contraction sums u_i d_j for i + j <= 7 in FP32: u is passed as an FP16 subnormal (the byte
 // itself, u 2^-24), d as an FP16 integer; |sum| < 2^24 units over 64 terms of 8 products each, so
@@ -55,10 +57,8 @@ __device__ __forceinline__ fxu_t fx_mulu(unsigned a, unsigned b) {
   return r;
 }
 
-// S of a row from the high word of the largest |mu| of its m (0: nothing recorded)
-__device__ __forceinline__ int fx_scale(unsigned mu_hi) {
-  return 62 - max(0, (int)(mu_hi >> 20) - 1022);
-}
+// S from the high word of the largest |mu|
+__device__ __forceinline__ int fx_scale(unsigned mu_hi) { return 62 - ((int)(mu_hi >> 20) - 1022); }
 
 // v 2^k rounded to nearest (v finite, |v 2^k| < 2^63)
 __device__ __forceinline__ fx_t fx_from_double(double v, int k) {
@@ -131,18 +131,17 @@ struct FxState {
   }
 };
 
-// start values (mu_l, mu_l+1), l - m even, at scale S -> state whose V2, V1 are those two values;
-// neg: sigma of l is -
-__device__ __forceinline__ FxState fx_start(double v0, double v1, int S, bool neg) {
+// values (mu_l, mu_l+1), l - m even, sigma of l +, at scale S -> state whose V2, V1 are those two values
+__device__ __forceinline__ FxState fx_start(double v0, double v1, int S) {
   FxState st;
   const unsigned h = max((unsigned)__double2hiint(v0) & 0x7fffffffu,
                          (unsigned)__double2hiint(v1) & 0x7fffffffu);
   if (h == 0) return st;
-  // |V| < 2^(S + e + E), E = exponent bound of the larger value: at most 2^59 unless e is 0 (e is 64 at
-  // most, for fx_pack; starts of 2^-60 need no more from S = 55 on, below it V has fewer bits)
-  st.e = min(64, max(0, 59 - S - ((int)(h >> 20) - 1022)) & ~7);
-  st.V2 = fx_from_double(neg ? -v0 : v0, S + st.e) + kFxBias;
-  st.V1 = fx_from_double(neg ? -v1 : v1, S + st.e) + kFxBias;
+  // |V| < 2^(S + e + E), E = exponent bound of the larger value: at most 2^59 unless e is 0 (walks start
+  // from |V| = 2 at e = 0 on, so e is at most 56)
+  st.e = max(0, 59 - S - ((int)(h >> 20) - 1022)) & ~7;
+  st.V2 = fx_from_double(v0, S + st.e) + kFxBias;
+  st.V1 = fx_from_double(v1, S + st.e) + kFxBias;
   return st;
 }
 
@@ -151,7 +150,7 @@ __device__ __forceinline__ FxState fx_start(double v0, double v1, int S, bool ne
 // converting FP64 checkpoints at every use, and the adjoint's ring parts in every tile of l, took a tenth
 // of the adjoint (Nside 1024, 3 maps: 20.4 -> 18.2 ms).
 __device__ __forceinline__ ulonglong2 fx_pack(double v0, double v1, int S) {
-  const FxState st = fx_start(v0, v1, S, false);
+  const FxState st = fx_start(v0, v1, S);
   const fxu_t a = (fxu_t)(st.V2 - kFxBias), b = (fxu_t)(st.V1 - kFxBias);
   if (st.e == 0) return make_ulonglong2(a << 1, b << 1);
   return make_ulonglong2(a << 4 | (fxu_t)(2 * (st.e / 8 - 1) + 1), b << 4);
@@ -166,6 +165,12 @@ __device__ __forceinline__ FxState fx_unpack(ulonglong2 c) {
   st.V2 = ((fx_t)c.x >> sh) + kFxBias;
   st.V1 = ((fx_t)c.y >> sh) + kFxBias;
   return st;
+}
+
+// sigma of l -
+__device__ __forceinline__ void fx_negate(FxState& st) {
+  st.V2 = 2 * kFxBias - st.V2;
+  st.V1 = 2 * kFxBias - st.V1;
 }
 
 // room for a step with coefficient A while an exponent is left: |V| below 2^(61 - sh)

@@ -173,8 +173,8 @@ struct SynLayout {
 template <int NM>
 __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double* __restrict__ Acoef,
-               const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
-               const int* __restrict__ tmin, const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
+               const uint8_t* __restrict__ sx, const int* __restrict__ ls_tab,
+               const int* __restrict__ tmin, const ulonglong2* __restrict__ st, const uint64_t* __restrict__ xfx,
                const ulonglong2* __restrict__ ck, const int64_t* __restrict__ ck_base,
                const int2* __restrict__ pring, double2* __restrict__ F, int64_t F_stride, int L, int npair,
                int R, int nmaps) {
@@ -194,7 +194,6 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   const int row = tid & (kM - 1), chain = tid >> 7;  // chain: warp-uniform
   const int m = blockIdx.y;
   const int64_t lmo = lm_off(L, m) - m;  // index of (m, l) is lmo + l
-  const int S = fx_scale(mumax[m]);
 
   // scale of each map: the largest exponent among this m's coefficients
   if (tid < 8) s_emax[tid] = 0;
@@ -248,8 +247,8 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     const unsigned xh = (unsigned)(x >> 32), xl = (unsigned)x;
     FxState s0;  // the pair's start values
     if (ls <= L) {
-      const double2 v = st[(int64_t)m * npair + p];
-      s0 = fx_start(v.x, v.y, S, ((ls - m) & 2) != 0);
+      s0 = fx_unpack(st[(int64_t)m * npair + p]);
+      if ((ls - m) & 2) fx_negate(s0);
     }
     if (tid < 4 * W) s_corr[tid] = 0;
     const int wlo = __reduce_min_sync(kFull, ls);
@@ -357,6 +356,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     if (bad) atomicOr(s_bad, 1);
     __syncthreads();
     const bool failed = *s_bad != 0;
+    const int S = valid ? sx[(int64_t)m * npair + p] : 0;
     double v[P];
     double* s_odd = reinterpret_cast<double*>(sm + LY::kA);  // [part][row]; all MMAs are done
 #pragma unroll
@@ -398,8 +398,8 @@ int launch_synth_variant(int v, int nm, const Grid& g, const void* alm, int64_t 
   auto kern = k_leg_synth_fx<NM>;
   CMBWS_TRY(ensure_dyn_smem((const void*)kern, LY::kBytes));
   ProfScope ps(PROF_LEG_SYNTH, s, 1, leg_work(g, nm));
-  kern<<<grd, kNT, LY::kBytes, s>>>((const double2*)alm, as, g.A64.as<double>(), g.mumax.as<unsigned>(),
-                                    g.lsx.as<int>(), g.lsx_tmin.as<int>(), g.stx.as<double2>(),
+  kern<<<grd, kNT, LY::kBytes, s>>>((const double2*)alm, as, g.A64.as<double>(), g.sx.as<uint8_t>(),
+                                    g.lsx.as<int>(), g.lsx_tmin.as<int>(), g.stx.as<ulonglong2>(),
                                     g.xfx.as<uint64_t>(), g.ckx.as<ulonglong2>(), g.ckx_base.as<int64_t>(),
                                     g.pair_ring.as<int2>(), (double2*)F, fs, L, g.npair, R, nm);
   CMBWS_LAUNCH_CHECK();
@@ -435,45 +435,59 @@ __device__ __forceinline__ unsigned part_exp(double v) {
   return ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
 }
 
-// ee[map][m] = exponent bound of the map's ring parts at m: |e| < 2^ee (1025: not all finite); the ring
-// parts become fixed point at that scale in place (zeros if not finite), once for all tiles of l.
+// ee[map][m] = exponent bound of the map's ring parts e 2^-S at m, S the scale of their pair (fixed.h):
+// |e 2^-S| < 2^ee (kNotFinite: not all finite).  The ring parts become fixed point at that scale in place
+// (zeros if not finite, and for pairs that never start), once for all tiles of l.  Without the pair's
+// scale, a bright ring at a pole, whose Legendre values at high m are all small, would set ee there: one
+// pixel of 1e10 over unit noise in the first ring of a GL grid with L = 63 left an m with errors of 4e-9
+// of its largest coefficient; 3e-14 with it, as from FP64 arithmetic.
+constexpr int kNotFinite = 1 << 20;
 template <int NM>
 __global__ void __launch_bounds__(256)
-k_eo_fix(double* __restrict__ eo, int npair, int L, int* __restrict__ ee, int nmaps) {
+k_eo_fix(double* __restrict__ eo, int npair, int L, const uint8_t* __restrict__ sx, int* __restrict__ ee,
+         int nmaps) {
   const int nm = NM <= 4 ? NM : nmaps;
-  __shared__ unsigned s_e[NM];
+  __shared__ int s_e[NM];
   const int m = blockIdx.x, tid = threadIdx.x;
-  if (tid < NM) s_e[tid] = 0;
+  if (tid < NM) s_e[tid] = -kNotFinite;
   __syncthreads();
   double* src = eo + (int64_t)m * npair * 4 * nm;
-  unsigned e[NM];
+  const uint8_t* sm = sx + (int64_t)m * npair;
+  int e[NM];
 #pragma unroll
-  for (int k = 0; k < NM; ++k) e[k] = 0;
+  for (int k = 0; k < NM; ++k) e[k] = -kNotFinite;
   for (int i = tid; i < 2 * npair; i += 256) {  // (pair, parity): 2 nm values
     const double2* v = reinterpret_cast<const double2*>(src) + (int64_t)i * nm;
-#pragma unroll
-    for (int k = 0; k < NM; ++k)
-      if (k < nm) e[k] = max(e[k], max(part_exp(v[k].x), part_exp(v[k].y)));
-  }
-#pragma unroll
-  for (int k = 0; k < NM; ++k) {
-    const unsigned v = __reduce_max_sync(kFull, e[k]);
-    if ((tid & 31) == 0) atomicMax(&s_e[k], v);
-  }
-  __syncthreads();
-  if (tid < nm) ee[(int64_t)tid * (L + 1) + m] = (int)s_e[tid] - 1022;
-  int sc[NM];
-#pragma unroll
-  for (int k = 0; k < NM; ++k) sc[k] = kFxABits - ((int)s_e[k] - 1022);
-  for (int i = tid; i < 2 * npair; i += 256) {
-    double2* v = reinterpret_cast<double2*>(src) + (int64_t)i * nm;
+    const int S = sm[i >> 1];
 #pragma unroll
     for (int k = 0; k < NM; ++k)
       if (k < nm) {
-        const bool ok = sc[k] > kFxABits - 1025;
+        const int x = (int)max(part_exp(v[k].x), part_exp(v[k].y));
+        if (x == 0x7ff) e[k] = kNotFinite;
+        else if (S) e[k] = max(e[k], x - 1022 - S);
+      }
+  }
+#pragma unroll
+  for (int k = 0; k < NM; ++k) {
+    const int v = __reduce_max_sync(kFull, e[k]);
+    if ((tid & 31) == 0) atomicMax(&s_e[k], v);
+  }
+  __syncthreads();
+  if (tid < nm) ee[(int64_t)tid * (L + 1) + m] = s_e[tid];
+  int sc[NM];
+#pragma unroll
+  for (int k = 0; k < NM; ++k) sc[k] = s_e[k];
+  for (int i = tid; i < 2 * npair; i += 256) {
+    double2* v = reinterpret_cast<double2*>(src) + (int64_t)i * nm;
+    const int S = sm[i >> 1];
+#pragma unroll
+    for (int k = 0; k < NM; ++k)
+      if (k < nm) {
+        const bool ok = S && sc[k] < kNotFinite;
+        const int x = kFxABits - sc[k] - S;
         const double2 d = v[k];
-        v[k] = make_double2(__longlong_as_double(ok ? fx_from_double(d.x, sc[k]) : 0),
-                            __longlong_as_double(ok ? fx_from_double(d.y, sc[k]) : 0));
+        v[k] = make_double2(__longlong_as_double(ok ? fx_from_double(d.x, x) : 0),
+                            __longlong_as_double(ok ? fx_from_double(d.y, x) : 0));
       }
   }
 }
@@ -487,8 +501,7 @@ k_eo_fix(double* __restrict__ eo, int npair, int L, int* __restrict__ ee, int nm
 template <int NM>
 __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const double* __restrict__ Acoef,
-             const unsigned* __restrict__ mumax, const int* __restrict__ ls_tab,
-             const double2* __restrict__ st, const uint64_t* __restrict__ xfx,
+             const int* __restrict__ ls_tab, const ulonglong2* __restrict__ st, const uint64_t* __restrict__ xfx,
              const ulonglong2* __restrict__ ck, const int64_t* __restrict__ ck_base,
              const int* __restrict__ tmin, const double* __restrict__ c64, double2* __restrict__ out,
              int64_t nlm, int L, int npair, int nmaps) {
@@ -525,7 +538,6 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
       for (int k = 0; k < nm; ++k) out[k * nlm + lmo + l] = make_double2(0.0, 0.0);
     return;
   }
-  const int S = fx_scale(mumax[m]);
   if (tid == 0) {
     *s_bad = 0;
     mbar_init(&mbar[0], 1);
@@ -551,7 +563,7 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
   const int nck = (L - m + kFxChunk) / kFxChunk;
   const ulonglong2* ckc = ck + (cval ? ck_base[m] + (l0 - m) / kFxChunk : 0);  // + p * nck
   const int* lsm = ls_tab + (int64_t)m * npair;
-  const double2* stm = st + (int64_t)m * npair;
+  const ulonglong2* stm = st + (int64_t)m * npair;
   unsigned char* arow = sm + LY::kA + 2 * warp * kAdjOct + lane * 16;
 
   // this thread's ring parts of a stage: column nn of parity par, kPP pairs from 8 oct + kPP sub on
@@ -601,9 +613,8 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
       w = fx_unpack(in.c);  // zeros if the pair starts later
       const bool inj = ls > l0 && ls < l0 + kFxChunk && ls <= L;
       if (__any_sync(kFull, inj)) {
-        double2 v = make_double2(0.0, 0.0);
-        if (inj) v = stm[p];
-        s0 = fx_start(v.x, v.y, S, ((ls - m) & 2) != 0);
+        if (inj) s0 = fx_unpack(stm[p]);
+        if ((ls - m) & 2) fx_negate(s0);
       }
     }
     fx_t ev[kPP];
@@ -696,9 +707,9 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
   for (int q = 0; q < NM; ++q) {
     if (q >= nm) break;
     const int ea = ee[(int64_t)q * (L + 1) + m];
-    const double v = acc[q].value((fx_t)corr[4 * q], (fx_t)corr[4 * q + 1], ea - S - 6);
+    const double v = acc[q].value((fx_t)corr[4 * q], (fx_t)corr[4 * q + 1], ea - 6);
     // a map with a non-finite ring part, and a timed-out wait, give NaN
-    o[2 * q * nlm] = (failed || ea >= 1025) ? fx_nan() : cc * v;
+    o[2 * q * nlm] = (failed || ea == kNotFinite) ? fx_nan() : cc * v;
   }
 }
 
@@ -707,13 +718,13 @@ int launch_adj(int nm, const Grid& g, double* eo, int* ee, double* out, cudaStre
   using LY = AdjLayout<Cols<NM>>;
   const int L = g.lmax;
   ProfScope ps(PROF_LEG_ADJ, s, 1, leg_work(g, nm));
-  k_eo_fix<NM><<<L + 1, 256, 0, s>>>(eo, g.npair, L, ee, nm);
+  k_eo_fix<NM><<<L + 1, 256, 0, s>>>(eo, g.npair, L, g.sx.as<uint8_t>(), ee, nm);
   CMBWS_LAUNCH_CHECK();
   dim3 grd((L + kM) / kM, L + 1);
   auto kern = k_leg_adj_fx<NM>;
   CMBWS_TRY(ensure_dyn_smem((const void*)kern, LY::kBytes));
-  kern<<<grd, kNT, LY::kBytes, s>>>(reinterpret_cast<const fx_t*>(eo), ee, g.A64.as<double>(), g.mumax.as<unsigned>(), g.lsx.as<int>(),
-                                    g.stx.as<double2>(), g.xfx.as<uint64_t>(), g.ckx.as<ulonglong2>(),
+  kern<<<grd, kNT, LY::kBytes, s>>>(reinterpret_cast<const fx_t*>(eo), ee, g.A64.as<double>(), g.lsx.as<int>(),
+                                    g.stx.as<ulonglong2>(), g.xfx.as<uint64_t>(), g.ckx.as<ulonglong2>(),
                                     g.ckx_base.as<int64_t>(), g.lsx_tmin.as<int>(), g.c64.as<double>(),
                                     (double2*)out, nlm_of(L), L, g.npair, nm);
   CMBWS_LAUNCH_CHECK();

@@ -39,7 +39,6 @@ namespace cmbws {
 namespace {
 
 constexpr double kStartThreshold = 1e-30;
-constexpr double kStartThresholdFx = 0x1p-60;  // fixed-point stages: smaller values have no digits
 constexpr double kShiftUp = 0x1p600;     // 2^600
 constexpr double kShiftDown = 0x1p-600;  // 2^-600
 constexpr double kGrow = 0x1p500;
@@ -141,17 +140,16 @@ __global__ void k_seeds(const double* __restrict__ sinth, const double* __restri
   }
 }
 
-// PLAN: starts, largest values and the checkpoints of the FP32 and fixed-point adjoints; otherwise
-// the double-float checkpoints only
+// PLAN: starts, scales of the fixed-point stages (fixed.h) and the checkpoints of the FP32 and
+// fixed-point adjoints; otherwise the double-float checkpoints only
 template <bool PLAN>
 __global__ void k_start(const double* __restrict__ y, const double* __restrict__ A, int L, int npair,
                         const double* __restrict__ sv, const int* __restrict__ sk,
                         int* __restrict__ ls, double2* __restrict__ st64, float2* __restrict__ st32,
-                        int* __restrict__ lsx, double2* __restrict__ stx,
                         const int64_t* __restrict__ ck_base, float2* __restrict__ ck,
                         const int64_t* __restrict__ ckx_base, double2* __restrict__ ckx,
                         const int64_t* __restrict__ ck64_base, float4* __restrict__ ck64,
-                        unsigned* __restrict__ mumax) {
+                        uint8_t* __restrict__ sx) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (p >= npair) return;
@@ -162,8 +160,7 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
   double v1 = sqrt(2.0 * m + 3.0) * (1.0 - yy) * v0;
   const double* Am = A + lm_off(L, m) - m;  // Am[l] = A_lm
   int l = m;
-  int found = L + 1, foundx = L + 1;
-  double x0 = 0.0, x1 = 0.0;
+  int found = L + 1;
   double o0 = 0.0, o1 = 0.0;
   unsigned mx = 0;  // high word of the largest |mu_l| from the start on
   const int nck = (L - m + kChunk) / kChunk;
@@ -178,11 +175,6 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
       o0 = v0;
       o1 = (l + 1 <= L) ? v1 : 0.0;
     }
-    if (PLAN && foundx > L && k == 0 && (fabs(v0) > kStartThresholdFx || fabs(v1) > kStartThresholdFx)) {
-      foundx = l;
-      x0 = v0;
-      x1 = (l + 1 <= L) ? v1 : 0.0;
-    }
     if (PLAN && found <= l) {
       mx = max(mx, (unsigned)__double2hiint(v0) & 0x7fffffffu);
       if (l + 1 <= L) mx = max(mx, (unsigned)__double2hiint(v1) & 0x7fffffffu);
@@ -193,7 +185,7 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
     const double w1 = (found <= l && l + 1 <= L) ? v1 : 0.0;
     if (PLAN && (l - m) % kChunk == 0) ckp[(l - m) / kChunk] = make_float2((float)w0, (float)w1);
     if (PLAN && (l - m) % kFxChunk == 0)
-      ckq[(l - m) / kFxChunk] = foundx <= l ? make_double2(w0, w1) : make_double2(0.0, 0.0);
+      ckq[(l - m) / kFxChunk] = make_double2(w0, w1);
     if (!PLAN && (l - m) % kChunkDf == 0) {
       const float h0 = (float)w0, h1 = (float)w1;
       ckd[(l - m) / kChunkDf] = make_float4(h0, (float)(w0 - (double)h0), h1, (float)(w1 - (double)h1));
@@ -212,11 +204,9 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
   }
   if (!PLAN) return;
   ls[idx] = found;
-  lsx[idx] = foundx;
-  stx[idx] = make_double2(x0, x1);
   st64[idx] = make_double2(o0, o1);
   st32[idx] = make_float2((float)o0, (float)o1);
-  if (mx) atomicMax(&mumax[m], mx);
+  sx[idx] = (uint8_t)(mx ? fx_scale(mx) : 0);
 }
 
 template <typename T2, typename T>
@@ -248,16 +238,41 @@ __global__ void k_unpack(const double2* __restrict__ lmc, int L, double* __restr
   if (m > 0) dst[(L - m + 1) + (l - m)] = v.y;
 }
 
-// fixed-point checkpoints, in place: their scale is known once every pair's values are
-__global__ void k_pack_ckx(ulonglong2* __restrict__ ckx, const int64_t* __restrict__ ckx_base, int L, int npair,
-                           const unsigned* __restrict__ mumax) {
+// Fixed-point starts: the pair's first l (same parity as m) at which a value has a digit at the pair's
+// scale, and the values there.
+__global__ void k_fx_starts(const double* __restrict__ y, const double* __restrict__ A, int L, int npair,
+                            const int* __restrict__ ls, const double2* __restrict__ st64,
+                            const uint8_t* __restrict__ sx, int* __restrict__ lsx, ulonglong2* __restrict__ stx) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
-  const int S = fx_scale(mumax[m]);
-  const int64_t n = (int64_t)npair * ((L - m + kFxChunk) / kFxChunk);
+  if (p >= npair) return;
+  const int64_t idx = (int64_t)m * npair + p;
+  const double yy = y[p], thr = scalbn(2.0, -(int)sx[idx]);
+  const double* Am = A + lm_off(L, m) - m;
+  double v0 = st64[idx].x, v1 = st64[idx].y;
+  int l = ls[idx];
+  for (; l + 2 <= L && fabs(v0) <= thr && fabs(v1) <= thr; l += 2) {
+    v0 = fma(-Am[l + 2], yy, Am[l + 2]) * v1 - v0;
+    v1 = (l + 3 <= L) ? fma(-Am[l + 3], yy, Am[l + 3]) * v0 - v1 : 0.0;
+  }
+  lsx[idx] = l;
+  stx[idx] = fx_pack(v0, v1, sx[idx]);
+}
+
+// fixed-point checkpoints, in place: their scale is known once the pair's values are
+__global__ void k_pack_ckx(ulonglong2* __restrict__ ckx, const int64_t* __restrict__ ckx_base, int L, int npair,
+                           const uint8_t* __restrict__ sx, const int* __restrict__ lsx) {
+  const int m = blockIdx.y;
+  const int nck = (L - m + kFxChunk) / kFxChunk;
+  const int64_t n = (int64_t)npair * nck;
   ulonglong2* c = ckx + ckx_base[m];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int p = (int)(i / nck);
+    const int64_t idx = (int64_t)m * npair + p;
     const ulonglong2 v = c[i];
-    c[i] = fx_pack(__longlong_as_double((long long)v.x), __longlong_as_double((long long)v.y), S);
+    c[i] = m + kFxChunk * (int)(i - (int64_t)p * nck) < lsx[idx]
+               ? make_ulonglong2(0, 0)
+               : fx_pack(__longlong_as_double((long long)v.x), __longlong_as_double((long long)v.y), sx[idx]);
   }
 }
 
@@ -435,16 +450,17 @@ int grid_build_tables(Grid& g) {
     }
     CMBWS_TRY(g.ckx_base.upload(cb.data(), (L + 1) * 8));
     CMBWS_TRY(g.ckx.alloc((size_t)totx * 16));
-    CMBWS_TRY(g.mumax.alloc((size_t)(L + 1) * 4));
-    CMBWS_CUDA(cudaMemset(g.mumax.p, 0, (size_t)(L + 1) * 4));
+    CMBWS_TRY(g.sx.alloc((size_t)nst));
     k_start<true><<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
                           d_sk.as<int>(), g.ls.as<int>(), g.st64.as<double2>(), g.st32.as<float2>(),
-                          g.lsx.as<int>(), g.stx.as<double2>(),
                           g.ck_base.as<int64_t>(), g.ck32.as<float2>(), g.ckx_base.as<int64_t>(),
-                          g.ckx.as<double2>(), nullptr, nullptr, g.mumax.as<unsigned>());
+                          g.ckx.as<double2>(), nullptr, nullptr, g.sx.as<uint8_t>());
+    CMBWS_LAUNCH_CHECK();
+    k_fx_starts<<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, g.ls.as<int>(),
+                              g.st64.as<double2>(), g.sx.as<uint8_t>(), g.lsx.as<int>(), g.stx.as<ulonglong2>());
     CMBWS_LAUNCH_CHECK();
     k_pack_ckx<<<dim3(32, L + 1), 256>>>(g.ckx.as<ulonglong2>(), g.ckx_base.as<int64_t>(), L, g.npair,
-                                         g.mumax.as<unsigned>());
+                                         g.sx.as<uint8_t>(), g.lsx.as<int>());
     CMBWS_LAUNCH_CHECK();
     const int ntile = (g.npair + kTileMinPT - 1) / kTileMinPT;
     CMBWS_TRY(g.ls_tmin.alloc((size_t)(L + 1) * ntile * 4));
@@ -590,7 +606,7 @@ int grid_ensure_ck64(const Grid& gc) {
   CMBWS_LAUNCH_CHECK();
   dim3 grd((g.npair + 127) / 128, L + 1);
   k_start<false><<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
-                        d_sk.as<int>(), nullptr, nullptr, nullptr, nullptr, nullptr, g.ck_base.as<int64_t>(),
+                        d_sk.as<int>(), nullptr, nullptr, nullptr, g.ck_base.as<int64_t>(),
                         nullptr, nullptr, nullptr, cbd.as<int64_t>(), ck.as<float4>(), nullptr);
   CMBWS_LAUNCH_CHECK();
   CMBWS_CUDA(cudaDeviceSynchronize());

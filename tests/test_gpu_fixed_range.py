@@ -70,3 +70,50 @@ def test_aliases_on_short_rings(nside, lmax):
     cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(alm), out, 1)
     want = osht.synthesis(og.healpix(nside), lmax, alm)
     assert rel_err(to_host(out), want) < 40 * (lmax + 1) * U
+
+
+def _grid(kind, n, lmax):
+    if kind == "healpix":
+        return cw.cmbws_plan_grid(cw.CMBWS_GRID_HEALPIX, n, lmax), og.healpix(n)
+    g = cw.cmbws_plan_grid(cw.CMBWS_GRID_GL, n, lmax)
+    nphi = np.full(n, 2 * lmax + 1)
+    return g, og.RingGrid("gl", n, g.theta, np.zeros(n), nphi, g.weight,
+                          np.concatenate([[0], np.cumsum(nphi)]))
+
+
+@pytest.mark.parametrize("kind,n,lmax", [("gl", 64, 63), ("gl", 131, 129), ("healpix", 16, 47)])
+@pytest.mark.parametrize("amp", [1e3, 1e6, 1e10])
+def test_bright_polar_pixel_per_order(kind, n, lmax, amp):
+    """One pixel of the first ring far above unit noise aliases into every m, but its Legendre values
+    at high m are tiny: the coefficients of each order are as accurate, relative to the largest of the
+    order, as the FP64 parity bound 40 (L+1) u asks."""
+    g, o = _grid(kind, n, lmax)
+    f = np.random.default_rng(n).standard_normal(g.npix)
+    f[0] = amp
+    back = to_dev(np.zeros((lmax + 1) ** 2))
+    cw.cmbws_sht_analysis(g, cw.CMBWS_FP64, to_dev(f), back, 1, 0)
+    got, want = to_host(back), osht.adjoint(o, lmax, f)
+    for m in range(lmax + 1):
+        a, b = (np.concatenate(osht.packed_m(v, lmax, m)) for v in (got, want))
+        assert rel_err(a, b) < 40 * (lmax + 1) * U, m
+
+
+@pytest.mark.parametrize("kind,n,lmax,m", [("gl", 64, 63, 16), ("gl", 131, 129, 60), ("gl", 131, 129, 129),
+                                           ("healpix", 16, 47, 20)])
+def test_dark_rings_of_one_order(kind, n, lmax, m):
+    """Coefficients of a single high order leave rings near the poles dark: each ring is as accurate,
+    relative to its own largest pixel, as the FP64 parity bound asks.  Walks start where the Legendre
+    values pass 1e-30, so L + 1 terms of coefficients up to 3 below that are left out on every path; on
+    rings brighter than 3e-30 / (40 u) = 7e-16 they are within the bound."""
+    g, o = _grid(kind, n, lmax)
+    alm = np.zeros((lmax + 1) ** 2)
+    i = (lmax + 1) + (m - 1) * (2 * lmax + 2 - m)
+    k = lmax - m + 1
+    alm[i:i + 2 * k] = np.random.default_rng(m).standard_normal(2 * k)
+    out = to_dev(np.zeros(g.npix))
+    cw.cmbws_sht_synth(g, cw.CMBWS_FP64, to_dev(alm), out, 1)
+    got, want = to_host(out), osht.synthesis(o, lmax, alm)
+    for r in range(g.nring):
+        s = slice(int(o.offset[r]), int(o.offset[r + 1]))
+        if np.abs(want[s]).max() > 7e-16:
+            assert rel_err(got[s], want[s]) < 40 * (lmax + 1) * U, r

@@ -64,6 +64,12 @@ typedef enum { CMBWS_GRID_GL = 0, CMBWS_GRID_HEALPIX = 1 } cmbws_grid_kind;
  * always FP64.
  *   CMBWS_FP64:   FP64 accuracy and FP64 data throughout; the Legendre stage and the ring FFTs
  *                 compute in 64-bit fixed point (integer units and exact tensor-core sums).
+ *                 Accuracy as from FP64 arithmetic: of a synthesis relative to the largest pixel of
+ *                 each ring, of an adjoint or analysis relative to the largest coefficient of each
+ *                 order m.  Inputs are held at one scale per ring (pixels) and per m (ring spectra,
+ *                 62 bits below the largest one that matters there); a coefficient below 2^-9 of the
+ *                 largest of its m can be less accurate relative to itself than from FP64 arithmetic
+ *                 where a ring brighter than the others by that much lies nearer the pole.
  *   CMBWS_FP32:   FP32 throughout (relative error ~1e-6 at L ~ 3000).
  *   CMBWS_FP32X2: FP64-accurate Legendre stage in double-float arithmetic (pairs of FP32
  *                 values, ~48-bit significand, on the FP32 pipe, which GB300 runs 61x

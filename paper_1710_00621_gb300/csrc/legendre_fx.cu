@@ -156,9 +156,35 @@ struct SynLayout {
   static constexpr int kCorr = kCoef + 2 * kSynK * 16;  // fxu_t[2 W][2]
   static constexpr int kBar = kCorr + 2 * C::W * 16;    // uint64_t[2]
   static constexpr int kMisc = kBar + 16;           // tensor memory base, bad flag
-  static constexpr int kExp = kMisc + 16;           // exponents [8]
-  static constexpr int kBytes = kExp + 32;
+  static constexpr int kExp = kMisc + 16;           // exponents [3][8]
+  static constexpr int kBytes = kExp + 96;
 };
+
+// Steep spectra.  One scale per (m, map) holds a coefficient to 2^-61 of the largest one that the rings of
+// the CTA can see, where FP64 arithmetic holds it to 2^-53 of itself.  That is enough for a ring's map if
+// the largest one is below 2^8 of what lights the ring anyway: its coefficients of m = 0, whose Legendre
+// values are of order one at every l and ring (the first 256 stand for them), or those of this m from
+// where the ring's values are of order one (l sin(theta) = m; for the CTA's ring nearest the pole).  Only
+// spectra without much at m = 0 that fall by more than 2^8 along this m fail both; their sums are taken in
+// FP64 arithmetic instead (from the start at 1e-30), by two threads per ring pair, one for each parity.
+constexpr int kSteep = 8;
+// Sum over l of mu_l a_l with l - m of parity par; a, A at index l; ls, st: the pair's start.
+__device__ __noinline__ double2 synth_fp64(const double2* a, const double* A, double y, int ls, double2 st,
+                                           int L, int par) {
+  double re = 0.0, im = 0.0, m2 = st.x, m1 = st.y;
+  for (int l = ls; l <= L; l += 2) {
+    if (l + par <= L) {
+      const double mu = par ? m1 : m2;
+      const double2 v = a[l + par];
+      re = fma(mu, v.x, re);
+      im = fma(mu, v.y, im);
+    }
+    if (l + 2 > L) break;
+    m2 = fma(-A[l + 2], y, A[l + 2]) * m1 - m2;
+    m1 = l + 3 <= L ? fma(-A[l + 3], y, A[l + 3]) * m2 - m1 : 0.0;
+  }
+  return make_double2(re, im);
+}
 
 // Two threads per ring pair (row of A) walk l upwards: one from the first start of the CTA's pairs,
 // one from the checkpoint in the middle of the rest (half the chain, twice the warps to hide the
@@ -176,7 +202,8 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
                const uint8_t* __restrict__ sx, const int* __restrict__ ls_tab,
                const int* __restrict__ tmin, const ulonglong2* __restrict__ st, const uint64_t* __restrict__ xfx,
                const ulonglong2* __restrict__ ck, const int64_t* __restrict__ ck_base,
-               const int2* __restrict__ pring, double2* __restrict__ F, int64_t F_stride, int L, int npair,
+               const int2* __restrict__ pring, const int* __restrict__ ls64, const double2* __restrict__ st64,
+               const double* __restrict__ y64, double2* __restrict__ F, int64_t F_stride, int L, int npair,
                int R, int nmaps) {
   using C = Cols<NM>;
   using LY = SynLayout<C>;
@@ -188,34 +215,24 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + LY::kBar);
   uint32_t* s_tb = reinterpret_cast<uint32_t*>(sm + LY::kMisc);
   int* s_bad = reinterpret_cast<int*>(sm + LY::kMisc + 4);
+  // exponents per map: largest coefficient from the group's first start on, from s_ehi's l on, of m = 0
   unsigned* s_emax = reinterpret_cast<unsigned*>(sm + LY::kExp);
+  unsigned *s_ehi = s_emax + 8, *s_e0 = s_emax + 16;
 
   const int tid = threadIdx.x, warp = tid >> 5;
   const int row = tid & (kM - 1), chain = tid >> 7;  // chain: warp-uniform
   const int m = blockIdx.y;
   const int64_t lmo = lm_off(L, m) - m;  // index of (m, l) is lmo + l
 
-  // scale of each map: the largest exponent among this m's coefficients
-  if (tid < 8) s_emax[tid] = 0;
+  if (tid < 24) s_emax[tid] = 0;
   if (tid == 0) {
     *s_bad = 0;
     mbar_init(&mbar[0], 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < NM; ++k) {
-    if (k >= nm) break;
-    unsigned e = 0;
-#pragma unroll 4
-    for (int l = m + tid; l <= L; l += kNT) {
-      const double2 v = alm[k * alm_stride + lmo + l];
-      e = max(e, max((unsigned)__double2hiint(v.x) & 0x7fffffffu,
-                     (unsigned)__double2hiint(v.y) & 0x7fffffffu));
-    }
-    e = __reduce_max_sync(kFull, e >> 20);
-    if ((tid & 31) == 0) atomicMax(&s_emax[k], e);
-  }
+  auto exp2 = [](double2 v) {
+    return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu) >> 20;
+  };
   // zero B (columns of the other parity and of absent maps stay zero)
   for (int i = tid; i < 2 * C::kBStep / 16; i += kNT)
     reinterpret_cast<uint4*>(sm + LY::kB)[i] = make_uint4(0, 0, 0, 0);
@@ -231,7 +248,6 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   constexpr int kBEvery = W == 8 ? 2 : 1;
   const int bk = tid & 15, bq = (tid >> 4) & (W - 1);
   const bool bon = bq < 2 * nm;
-  const int eb = bon ? (int)s_emax[bq >> 1] - 1022 : 0;  // |a| < 2^eb; 1025 if not finite
   const double* bsrc = reinterpret_cast<const double*>(alm + (bq >> 1) * alm_stride + lmo) + (bq & 1);
   unsigned char* bdst = sm + LY::kB + (bk & 1) * W * 32 + (bk >> 3) * 128 + (bq >> 3) * 256 + (bq & 7) * 16 +
                         (bk & 7) * 2;
@@ -256,6 +272,42 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     const int ntm = (npair + kTileMinPT - 1) / kTileMinPT, t0 = (blockIdx.x * R + r) * (kM / kTileMinPT);
     int lo = L + 1;
     for (int t = t0; t < min(ntm, t0 + kM / kTileMinPT); ++t) lo = min(lo, tmin[(int64_t)m * ntm + t]);
+    // scale of each map: the largest exponent among this m's coefficients from lo on (any that is not
+    // finite counts)
+    const int p0 = (blockIdx.x * R + r) * kM;
+    const float y0 = p0 < npair ? (float)y64[p0] : 1.f;
+    const int hi = (int)fminf((float)L, ceilf((float)m * rsqrtf(fmaxf(y0 * (2.f - y0), 1e-30f))));
+    if (r > 0) {
+      if (tid < 16) s_emax[tid] = 0;
+      __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      if (k >= nm) break;
+      unsigned e = 0, eh = 0, e0 = 0;
+      if (r == 0 && tid <= L) e0 = exp2(alm[k * alm_stride + tid]);
+#pragma unroll 4
+      for (int l = m + tid; l <= L; l += kNT) {
+        const unsigned x = exp2(alm[k * alm_stride + lmo + l]);
+        if (l >= lo || x == 0x7ffu) e = max(e, x);
+        if (l >= hi) eh = max(eh, x);
+      }
+      e = __reduce_max_sync(kFull, e);
+      eh = __reduce_max_sync(kFull, eh);
+      e0 = __reduce_max_sync(kFull, e0);
+      if ((tid & 31) == 0) {
+        atomicMax(&s_emax[k], e);
+        atomicMax(&s_ehi[k], eh);
+        atomicMax(&s_e0[k], e0);
+      }
+    }
+    __syncthreads();
+    auto steep = [&](int k) {
+      return s_emax[k] < 0x7ffu && s_emax[k] > max(s_ehi[k], s_e0[k]) + kSteep;
+    };
+    bool all_steep = true;
+    for (int k = 0; k < nm; ++k) all_steep &= steep(k);
+    const int eb = bon ? (int)s_emax[bq >> 1] - 1022 : 0;  // |a| < 2^eb; 1025 if not finite
     // rows of pairs that have not started: zero digits
 #pragma unroll
     for (int i = 0; i < kFxDig; ++i) {
@@ -266,7 +318,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     const int cm = ((lo + L) / 2 - m + kFxChunk / 2) / kFxChunk;
     int lm = m + kFxChunk * cm;
     if (lm <= lo) lm += kFxChunk;
-    const int len = lo <= L ? max(min(lm, L + 1) - lo, L + 1 - lm) : 0;
+    const int len = lo <= L && !all_steep ? max(min(lm, L + 1) - lo, L + 1 - lm) : 0;
     const int nst = (len + kSynK / 2 - 1) / (kSynK / 2);
     // l of value k (0..15) of stage t, or -1
     auto l_of = [&](int t, int k) {
@@ -360,12 +412,24 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     double v[P];
     double* s_odd = reinterpret_cast<double*>(sm + LY::kA);  // [part][row]; all MMAs are done
 #pragma unroll
+    for (int q = 0; q < P; ++q)
+      v[q] = acc[q].value((fx_t)s_corr[2 * (W * chain + q)], (fx_t)s_corr[2 * (W * chain + q) + 1],
+                          (int)s_emax[q >> 1] - 1022 - S - 6);
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      if (k >= nm || !steep(k)) continue;
+      double2 f = make_double2(0.0, 0.0);
+      const int l1 = valid ? ls64[(int64_t)m * npair + p] : INT_MAX;
+      if (l1 <= L)
+        f = synth_fp64(alm + k * alm_stride + lmo, Acoef + lmo, y64[p], l1, st64[(int64_t)m * npair + p], L, chain);
+      v[2 * k] = f.x;
+      v[2 * k + 1] = f.y;
+    }
+#pragma unroll
     for (int q = 0; q < P; ++q) {
-      const int ea = (int)s_emax[q >> 1] - 1022;
-      v[q] = acc[q].value((fx_t)s_corr[2 * (W * chain + q)], (fx_t)s_corr[2 * (W * chain + q) + 1], ea - S - 6);
       // a map with a non-finite coefficient, and a timed-out wait, give NaN
       if (m > 0) v[q] *= 0.70710678118654752440;  // the ring FFT's 1 / sqrt(2)
-      if ((ea >= 1025 && ls <= L) || failed) v[q] = fx_nan();
+      if ((s_emax[q >> 1] == 0x7ffu && ls <= L) || failed) v[q] = fx_nan();
       if (chain) s_odd[q * kM + row] = v[q];
     }
     __syncthreads();
@@ -401,7 +465,8 @@ int launch_synth_variant(int v, int nm, const Grid& g, const void* alm, int64_t 
   kern<<<grd, kNT, LY::kBytes, s>>>((const double2*)alm, as, g.A64.as<double>(), g.sx.as<uint8_t>(),
                                     g.lsx.as<int>(), g.lsx_tmin.as<int>(), g.stx.as<ulonglong2>(),
                                     g.xfx.as<uint64_t>(), g.ckx.as<ulonglong2>(), g.ckx_base.as<int64_t>(),
-                                    g.pair_ring.as<int2>(), (double2*)F, fs, L, g.npair, R, nm);
+                                    g.pair_ring.as<int2>(), g.ls.as<int>(), g.st64.as<double2>(), g.y64.as<double>(),
+                                    (double2*)F, fs, L, g.npair, R, nm);
   CMBWS_LAUNCH_CHECK();
   return CMBWS_OK;
 }

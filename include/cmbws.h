@@ -115,6 +115,11 @@ const char* cmbws_version(void);
  * Limits: FP64 transforms need every ring length n <= 4096 after padding
  *   (ring FFTs run in shared memory); FP32 n <= 8192.  Larger grids return
  *   CMBWS_ERR_ARG from the transform calls of the precision they exceed.
+ * Tables: 8 bytes per 8 values of l of every (m, ring pair) (9.7 GB at Nside 1024, lmax 3071) for
+ *   every grid, the same again from the first CMBWS_FP64 transform on, which waits for them, and four
+ *   times that from the first CMBWS_FP32X2 one on.  FP64 tables of at most 0.5 GB (all grids that
+ *   cmbws_sht_analysis_noalloc takes) come with the plan, those of the grids of a CMBWS_FP64 model
+ *   with the model.
  * Synchronises the device.  *out is released with cmbws_grid_destroy.
  */
 int cmbws_plan_grid(cmbws_grid_kind kind, int n, int lmax, cmbws_grid* out);

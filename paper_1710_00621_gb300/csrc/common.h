@@ -19,6 +19,7 @@
 
 #include <functional>
 #include <map>
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -175,13 +176,10 @@ struct Grid {
   DevMem c64;             // lambda_lm = c_lm mu_lm
   DevMem ls;              // int [L+1][npair] first l (same parity as m) that is injected
   DevMem st64, st32;      // {mu_ls, mu_ls+1} [L+1][npair]
-  DevMem sx;              // uint8 [L+1][npair]: scale of the fixed-point stages (fixed.h), 0 if never started
-  DevMem lsx, stx;        // first l and values (fx_pack) for the fixed-point stages
   DevMem xfx;             // uint64 cos(theta) 2^63 of the north ring [npair] (fixed-point stages)
   DevMem ck32;            // FP32 {mu_l0, mu_l0+1} at every chunk start l0 = m + kChunk c
   DevMem ck_base;         // int64 [L+1]: offset of m's block [pair][chunk] in ck32
   DevMem ls_tmin;         // int [L+1][ceil(npair / kTileMinPT)]: smallest ls of each tile of pairs
-  DevMem lsx_tmin;        // the same of lsx
   // warp tasks of the checkpointed FP32 adjoint: int2 {m, first chunk} per 32 consecutive
   // chunks of one m, m ascending
   DevMem wt32;
@@ -192,8 +190,13 @@ struct Grid {
   mutable int nwtdf = 0;
   mutable std::mutex ck64_mu;
   std::vector<double> fmm_h;  // sqrt((2m+1)/(2m)) (host, for rebuilding seeds)
-  DevMem ckx;             // fixed-point {mu_l0, mu_l0+1} (fx_pack) at every l0 = m + kFxChunk c (zero before the start)
-  DevMem ckx_base;        // int64 [L+1]: offset of m's block [pair][chunk] in ckx
+  // tables of the fixed-point (FP64) Legendre stage, built on their first use (grid_ensure_fx): scale
+  // (fixed.h; uint8, 0 if never started), first l and values there (fx_pack) [L+1][npair]; {mu_l0, mu_l0+1}
+  // (fx_pack) at every l0 = m + kFxChunk c (zero before the start) [m][pair][chunk] and its offsets (int64);
+  // smallest first l of each tile of pairs
+  DevMem sx, lsx, stx, ckx, ckx_base, lsx_tmin;
+  mutable std::mutex fx_mu;
+  mutable std::atomic<bool> fx_ready{false};
 
   // autotuner decisions for launches on this grid (legendre.cu), by kernel / precision / maps
   struct Tuned {
@@ -261,6 +264,14 @@ std::vector<int2> adjoint_warp_tasks(int L, int chunk);
 
 // ---- grid setup (setup.cu) ----
 int grid_build_tables(Grid& g);
+// Build the tables of the FP64 Legendre stage if not yet built (synchronous; also while the caller's
+// stream s is being captured): 16 bytes per 16 values of l of every pair, as much as the FP32
+// checkpoints again (9.7 GB at Nside 1024), which a grid that only runs other precisions does not carry.
+// Grids whose tables take at most 0.5 GB get them with the plan, those of models that compute in FP64 with
+// the model.
+int grid_ensure_fx(const Grid& g, cudaStream_t s);
+// cmbws_sht_analysis_noalloc takes the grid at CMBWS_FP64 (noalloc.cu)
+bool noalloc_fp64(const Grid& g);
 // build the double-float tables if not yet built
 int grid_ensure_ck64(const Grid& g);
 

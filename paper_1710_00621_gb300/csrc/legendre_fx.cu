@@ -230,6 +230,18 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     mbar_init(&mbar[0], 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
+  // of a group: the first start, and the l from where the Legendre values of the ring nearest the pole are
+  // of order one (loaded ahead of their use)
+  int lo_r, hi_r;
+  auto group_range = [&](int r) {
+    const int p0 = (blockIdx.x * R + r) * kM;
+    const int ntm = (npair + kTileMinPT - 1) / kTileMinPT, t0 = p0 / kTileMinPT;
+    const float y0 = p0 < npair ? (float)y64[p0] : 1.f;
+    lo_r = L + 1;
+    for (int t = t0; t < min(ntm, t0 + kM / kTileMinPT); ++t) lo_r = min(lo_r, tmin[(int64_t)m * ntm + t]);
+    hi_r = (int)fminf((float)L, ceilf((float)m * rsqrtf(fmaxf(y0 * (2.f - y0), 1e-30f))));
+  };
+  group_range(0);
   auto exp2 = [](double2 v) {
     return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu) >> 20;
   };
@@ -268,15 +280,10 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     }
     if (tid < 4 * W) s_corr[tid] = 0;
     const int wlo = __reduce_min_sync(kFull, ls);
-    // first start of the group
-    const int ntm = (npair + kTileMinPT - 1) / kTileMinPT, t0 = (blockIdx.x * R + r) * (kM / kTileMinPT);
-    int lo = L + 1;
-    for (int t = t0; t < min(ntm, t0 + kM / kTileMinPT); ++t) lo = min(lo, tmin[(int64_t)m * ntm + t]);
+    const int lo = lo_r, hi = hi_r;
+    if (r + 1 < R) group_range(r + 1);
     // scale of each map: the largest exponent among this m's coefficients from lo on (any that is not
     // finite counts)
-    const int p0 = (blockIdx.x * R + r) * kM;
-    const float y0 = p0 < npair ? (float)y64[p0] : 1.f;
-    const int hi = (int)fminf((float)L, ceilf((float)m * rsqrtf(fmaxf(y0 * (2.f - y0), 1e-30f))));
     if (r > 0) {
       if (tid < 16) s_emax[tid] = 0;
       __syncthreads();
@@ -799,6 +806,7 @@ int launch_adj(int nm, const Grid& g, double* eo, int* ee, double* out, cudaStre
 }  // namespace
 
 int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaStream_t s) {
+  CMBWS_TRY(grid_ensure_fx(g, s));
   const int64_t as = nlm_of(g.lmax), fs = (int64_t)g.nring * (g.lmax + 1);
   for (int k0 = 0; k0 < nmaps; k0 += kFxMaps) {
     const int nm = nmaps - k0 < kFxMaps ? nmaps - k0 : kFxMaps;
@@ -818,6 +826,7 @@ int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaSt
 }
 
 int legendre_adjoint_fx(const Grid& g, int nmaps, void* eo, int* ee, double* out, cudaStream_t s) {
+  CMBWS_TRY(grid_ensure_fx(g, s));
   const int64_t nlm = nlm_of(g.lmax), cs = (int64_t)(g.lmax + 1) * g.npair * 4;
   for (int k0 = 0; k0 < nmaps; k0 += kFxMaps) {
     const int nm = nmaps - k0 < kFxMaps ? nmaps - k0 : kFxMaps;

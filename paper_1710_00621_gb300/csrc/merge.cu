@@ -212,6 +212,7 @@ int Model::merge_precond(const int* group, cudaStream_t s) {
     CMBWS_TRY(G.out.alloc((size_t)G.nmaps * nlm * 16));
     for (int pr : {CMBWS_FP64, CMBWS_FP32, CMBWS_FP32X2})
       part_bytes = std::max(part_bytes, legendre_adjoint_part_bytes(gr, pr, G.nmaps));
+    if (prec == CMBWS_FP64 && ringfft_smem_ok(gr, prec)) CMBWS_TRY(grid_ensure_fx(gr, s));
   }
   if (part_bytes > part.bytes) CMBWS_TRY(part.ensure(part_bytes));
 

@@ -993,6 +993,10 @@ int model_create(const cmbws_model_desc* desc, int prec, cudaStream_t s, Model**
     for (int pr : {CMBWS_FP64, CMBWS_FP32, CMBWS_FP32X2})
       part_bytes = std::max(part_bytes, legendre_adjoint_part_bytes(*G.grid, pr, G.nmaps));
   CMBWS_TRY(M->part.alloc(part_bytes));
+  if (M->prec == CMBWS_FP64)  // tables of the applies, which may then be captured from the first on
+    for (const std::vector<Group>* gs : {&M->groups, &M->mgroups})
+      for (const Group& G : *gs)
+        if (ringfft_smem_ok(*G.grid, CMBWS_FP64)) CMBWS_TRY(grid_ensure_fx(*G.grid, s));
   CMBWS_TRY(M->tprior.alloc((size_t)M->nvec * 8));
   M->nsht_A = 2 * (2 * M->nmix + no);  // Sec. 3.3: 2 (2 Nmix + Nobs)
   M->nsht_M = 2 * no;

@@ -58,7 +58,30 @@ int scratch_address(void** out) {
 
 size_t round256(size_t n) { return (n + 255) & ~size_t(255); }
 
+// Scratch of a call.  limit: the documented one, ring spectra, adjoint scratch (FP64: partial sums of
+// blocks of 256 ring pairs for up to 4 maps) and coefficients together; pb, ob: what is used, the adjoint
+// input of nc maps and the coefficients.
+struct Scratch {
+  size_t limit, pb, ob;
+  int nc;
+  bool fits() const { return limit <= kScratchBytes && pb + ob <= kScratchBytes; }
+};
+Scratch scratch_for(const Grid& g, int prec, int nmaps) {
+  const size_t es = prec_size(prec);
+  const int64_t nlm = nlm_of(g.lmax);
+  const int cm = eo_maps(prec), nc = nmaps < cm ? nmaps : cm;
+  const size_t fb = round256((size_t)nmaps * g.nring * (g.lmax + 1) * 2 * es);
+  const size_t sb = prec == CMBWS_FP64
+                        ? round256((size_t)((g.npair + 255) / 256) * 2 * (nc < 4 ? nc : 4) * nlm * 8)
+                        : round256(legendre_adjoint_part_bytes(g, prec, nmaps));
+  const size_t ob = round256((size_t)nmaps * nlm * 16);
+  return {fb + sb + ob, round256(legendre_adjoint_part_bytes(g, prec, nc)), ob, nc};
+}
+
 }  // namespace
+
+bool noalloc_fp64(const Grid& g) { return ringfft_smem_ok(g, CMBWS_FP64) && scratch_for(g, CMBWS_FP64, 1).fits(); }
+
 }  // namespace cmbws
 
 using namespace cmbws;
@@ -88,32 +111,23 @@ extern "C" int cmbws_sht_analysis_noalloc(cmbws_grid gh, cmbws_prec prec, const 
     set_error("cmbws_sht_analysis_noalloc: ring length %d too large for this precision", g->max_n);
     return CMBWS_ERR_ARG;
   }
-  // the documented limit: ring spectra, adjoint scratch (FP64: partial sums of blocks of 256 ring
-  // pairs for up to 4 maps) and coefficients together; what is used below stays under it
-  const size_t es = prec_size(prec);
   const int64_t nlm = nlm_of(g->lmax);
-  const int cm = eo_maps(prec), nc = nmaps < cm ? nmaps : cm;
-  const size_t fb = round256((size_t)nmaps * g->nring * (g->lmax + 1) * 2 * es);
-  const size_t sb = prec == CMBWS_FP64
-                        ? round256((size_t)((g->npair + 255) / 256) * 2 * (nc < 4 ? nc : 4) * nlm * 8)
-                        : round256(legendre_adjoint_part_bytes(*g, prec, nmaps));
-  const size_t ob = round256((size_t)nmaps * nlm * 16);
-  const size_t pb = round256(legendre_adjoint_part_bytes(*g, prec, nc));
-  if (fb + sb + ob > kScratchBytes || pb + ob > kScratchBytes) {
+  const Scratch S = scratch_for(*g, prec, nmaps);
+  if (!S.fits()) {
     set_error("cmbws_sht_analysis_noalloc: needs %zu bytes of scratch for nmaps=%d, lmax=%d, "
               "nring=%d; the static scratch holds %zu bytes (use cmbws_sht_analysis)",
-              fb + sb + ob, nmaps, g->lmax, g->nring, kScratchBytes);
+              S.limit, nmaps, g->lmax, g->nring, kScratchBytes);
     return CMBWS_ERR_ARG;
   }
   void* base = nullptr;
   CMBWS_TRY(scratch_address(&base));
   unsigned char* part = static_cast<unsigned char*>(base);
-  double* out = reinterpret_cast<double*>(part + pb);
+  double* out = reinterpret_cast<double*>(part + S.pb);
   cudaStream_t s = (cudaStream_t)stream;
-  for (int k = 0; k < nmaps; k += cm) {
-    const int nm = nmaps - k < cm ? nmaps - k : cm;
+  for (int k = 0; k < nmaps; k += S.nc) {
+    const int nm = nmaps - k < S.nc ? nmaps - k : S.nc;
     CMBWS_TRY(ringfft_analysis(*g, prec, nm, map + k * g->npix, weighted, part, s));
-    CMBWS_TRY(legendre_adjoint(*g, prec, nm, part, pb, out + 2 * k * nlm, s));
+    CMBWS_TRY(legendre_adjoint(*g, prec, nm, part, S.pb, out + 2 * k * nlm, s));
   }
   CMBWS_TRY(unpack_alm(*g, nmaps, out, alm, s));
   return CMBWS_OK;

@@ -140,16 +140,13 @@ __global__ void k_seeds(const double* __restrict__ sinth, const double* __restri
   }
 }
 
-// PLAN: starts, scales of the fixed-point stages (fixed.h) and the checkpoints of the FP32 and
-// fixed-point adjoints; otherwise the double-float checkpoints only
+// PLAN: starts and the checkpoints of the FP32 adjoint; otherwise the double-float checkpoints only
 template <bool PLAN>
 __global__ void k_start(const double* __restrict__ y, const double* __restrict__ A, int L, int npair,
                         const double* __restrict__ sv, const int* __restrict__ sk,
                         int* __restrict__ ls, double2* __restrict__ st64, float2* __restrict__ st32,
                         const int64_t* __restrict__ ck_base, float2* __restrict__ ck,
-                        const int64_t* __restrict__ ckx_base, double2* __restrict__ ckx,
-                        const int64_t* __restrict__ ck64_base, float4* __restrict__ ck64,
-                        uint8_t* __restrict__ sx) {
+                        const int64_t* __restrict__ ck64_base, float4* __restrict__ ck64) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (p >= npair) return;
@@ -162,12 +159,9 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
   int l = m;
   int found = L + 1;
   double o0 = 0.0, o1 = 0.0;
-  unsigned mx = 0;  // high word of the largest |mu_l| from the start on
   const int nck = (L - m + kChunk) / kChunk;
-  const int nckx = (L - m + kFxChunk) / kFxChunk;
   const int nckd = (L - m + kChunkDf) / kChunkDf;
   float2* ckp = PLAN ? ck + ck_base[m] + (int64_t)p * nck : nullptr;
-  double2* ckq = PLAN ? ckx + ckx_base[m] + (int64_t)p * nckx : nullptr;
   float4* ckd = PLAN ? nullptr : ck64 + ck64_base[m] + (int64_t)p * nckd;
   while (l <= L) {
     if (found > L && k == 0 && (fabs(v0) > kStartThreshold || fabs(v1) > kStartThreshold)) {
@@ -175,17 +169,11 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
       o0 = v0;
       o1 = (l + 1 <= L) ? v1 : 0.0;
     }
-    if (PLAN && found <= l) {
-      mx = max(mx, (unsigned)__double2hiint(v0) & 0x7fffffffu);
-      if (l + 1 <= L) mx = max(mx, (unsigned)__double2hiint(v1) & 0x7fffffffu);
-    }
     // chunk checkpoints: the recurrence pair at the chunk's first l once the pair has
     // started there, zero before (a pair starting inside the chunk is injected at ls)
     const double w0 = found <= l ? v0 : 0.0;
     const double w1 = (found <= l && l + 1 <= L) ? v1 : 0.0;
     if (PLAN && (l - m) % kChunk == 0) ckp[(l - m) / kChunk] = make_float2((float)w0, (float)w1);
-    if (PLAN && (l - m) % kFxChunk == 0)
-      ckq[(l - m) / kFxChunk] = make_double2(w0, w1);
     if (!PLAN && (l - m) % kChunkDf == 0) {
       const float h0 = (float)w0, h1 = (float)w1;
       ckd[(l - m) / kChunkDf] = make_float4(h0, (float)(w0 - (double)h0), h1, (float)(w1 - (double)h1));
@@ -206,7 +194,6 @@ __global__ void k_start(const double* __restrict__ y, const double* __restrict__
   ls[idx] = found;
   st64[idx] = make_double2(o0, o1);
   st32[idx] = make_float2((float)o0, (float)o1);
-  sx[idx] = (uint8_t)(mx ? fx_scale(mx) : 0);
 }
 
 template <typename T2, typename T>
@@ -238,8 +225,35 @@ __global__ void k_unpack(const double2* __restrict__ lmc, int L, double* __restr
   if (m > 0) dst[(L - m + 1) + (l - m)] = v.y;
 }
 
-// Fixed-point starts: the pair's first l (same parity as m) at which a value has a digit at the pair's
-// scale, and the values there.
+// Tables of the fixed-point stages (fixed.h), from the starts of the plan: values at every l0 = m + kFxChunk c
+// (zero before the start; k_pack_ckx makes them fixed point) and the scale of the pair.
+__global__ void k_fx_walk(const double* __restrict__ y, const double* __restrict__ A, int L, int npair,
+                          const int* __restrict__ ls, const double2* __restrict__ st64,
+                          const int64_t* __restrict__ ckx_base, double2* __restrict__ ckx,
+                          uint8_t* __restrict__ sx) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  const int m = blockIdx.y;
+  if (p >= npair) return;
+  const int64_t idx = (int64_t)m * npair + p;
+  const double yy = y[p];
+  const double* Am = A + lm_off(L, m) - m;
+  double v0 = st64[idx].x, v1 = st64[idx].y;
+  const int nck = (L - m + kFxChunk) / kFxChunk;
+  double2* c = ckx + ckx_base[m] + (int64_t)p * nck;
+  int l = ls[idx];
+  for (int i = 0; i < nck && m + kFxChunk * i < l; ++i) c[i] = make_double2(0.0, 0.0);
+  unsigned mx = 0;  // high word of the largest |mu_l|
+  for (; l <= L; l += 2) {
+    mx = max(mx, max((unsigned)__double2hiint(v0) & 0x7fffffffu, (unsigned)__double2hiint(v1) & 0x7fffffffu));
+    if ((l - m) % kFxChunk == 0) c[(l - m) / kFxChunk] = make_double2(v0, v1);
+    if (l + 2 > L) break;
+    v0 = fma(-Am[l + 2], yy, Am[l + 2]) * v1 - v0;
+    v1 = (l + 3 <= L) ? fma(-Am[l + 3], yy, Am[l + 3]) * v0 - v1 : 0.0;
+  }
+  sx[idx] = (uint8_t)(mx ? fx_scale(mx) : 0);
+}
+
+// The pair's first l (same parity as m) at which a value has a digit at its scale, and the values there.
 __global__ void k_fx_starts(const double* __restrict__ y, const double* __restrict__ A, int L, int npair,
                             const int* __restrict__ ls, const double2* __restrict__ st64,
                             const uint8_t* __restrict__ sx, int* __restrict__ lsx, ulonglong2* __restrict__ stx) {
@@ -259,7 +273,7 @@ __global__ void k_fx_starts(const double* __restrict__ y, const double* __restri
   stx[idx] = fx_pack(v0, v1, sx[idx]);
 }
 
-// fixed-point checkpoints, in place: their scale is known once the pair's values are
+// checkpoints in place
 __global__ void k_pack_ckx(ulonglong2* __restrict__ ckx, const int64_t* __restrict__ ckx_base, int L, int npair,
                            const uint8_t* __restrict__ sx, const int* __restrict__ lsx) {
   const int m = blockIdx.y;
@@ -327,6 +341,17 @@ int unpack_alm(const Grid& g, int nmaps, const double* lmc, double* packed, cuda
   CMBWS_LAUNCH_CHECK();
   return CMBWS_OK;
 }
+
+// entries of the fixed-point checkpoints, and each m's offset
+static int64_t fx_offsets(const Grid& g, int64_t* base) {
+  int64_t tot = 0;
+  for (int m = 0; m <= g.lmax; ++m) {
+    if (base) base[m] = tot;
+    tot += (int64_t)g.npair * ((g.lmax - m + kFxChunk) / kFxChunk);
+  }
+  return tot;
+}
+constexpr int64_t kFxPlanBytes = 512 << 20;
 
 int grid_build_tables(Grid& g) {
   const int L = g.lmax;
@@ -422,8 +447,6 @@ int grid_build_tables(Grid& g) {
     CMBWS_TRY(d_sk.alloc(nst * 4));
     CMBWS_TRY(g.ls.alloc(nst * 4));
     CMBWS_TRY(g.st64.alloc(nst * 16));
-    CMBWS_TRY(g.lsx.alloc(nst * 4));
-    CMBWS_TRY(g.stx.alloc(nst * 16));
     CMBWS_TRY(g.st32.alloc(nst * 8));
     k_seeds<<<(g.npair + 127) / 128, 128>>>(d_sin.as<double>(), d_fmm.as<double>(), L, g.npair,
                                             d_sv.as<double>(), d_sk.as<int>());
@@ -443,32 +466,14 @@ int grid_build_tables(Grid& g) {
       g.nwt32 = (int)wt.size();
     }
     CMBWS_TRY(g.ck32.alloc((size_t)tot * 8));
-    int64_t totx = 0;
-    for (int m = 0; m <= L; ++m) {
-      cb[m] = totx;
-      totx += (int64_t)g.npair * ((L - m + kFxChunk) / kFxChunk);
-    }
-    CMBWS_TRY(g.ckx_base.upload(cb.data(), (L + 1) * 8));
-    CMBWS_TRY(g.ckx.alloc((size_t)totx * 16));
-    CMBWS_TRY(g.sx.alloc((size_t)nst));
     k_start<true><<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
                           d_sk.as<int>(), g.ls.as<int>(), g.st64.as<double2>(), g.st32.as<float2>(),
-                          g.ck_base.as<int64_t>(), g.ck32.as<float2>(), g.ckx_base.as<int64_t>(),
-                          g.ckx.as<double2>(), nullptr, nullptr, g.sx.as<uint8_t>());
-    CMBWS_LAUNCH_CHECK();
-    k_fx_starts<<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, g.ls.as<int>(),
-                              g.st64.as<double2>(), g.sx.as<uint8_t>(), g.lsx.as<int>(), g.stx.as<ulonglong2>());
-    CMBWS_LAUNCH_CHECK();
-    k_pack_ckx<<<dim3(32, L + 1), 256>>>(g.ckx.as<ulonglong2>(), g.ckx_base.as<int64_t>(), L, g.npair,
-                                         g.sx.as<uint8_t>(), g.lsx.as<int>());
+                          g.ck_base.as<int64_t>(), g.ck32.as<float2>(), nullptr, nullptr);
     CMBWS_LAUNCH_CHECK();
     const int ntile = (g.npair + kTileMinPT - 1) / kTileMinPT;
     CMBWS_TRY(g.ls_tmin.alloc((size_t)(L + 1) * ntile * 4));
     dim3 gt((ntile + 127) / 128, L + 1);
     k_tile_min<<<gt, 128>>>(g.ls.as<int>(), g.npair, ntile, g.ls_tmin.as<int>());
-    CMBWS_LAUNCH_CHECK();
-    CMBWS_TRY(g.lsx_tmin.alloc((size_t)(L + 1) * ntile * 4));
-    k_tile_min<<<gt, 128>>>(g.lsx.as<int>(), g.npair, ntile, g.lsx_tmin.as<int>());
     CMBWS_LAUNCH_CHECK();
     CMBWS_CUDA(cudaDeviceSynchronize());
   }
@@ -552,6 +557,11 @@ int grid_build_tables(Grid& g) {
     CMBWS_TRY(g.plans_d.upload(g.plans.data(), g.plans.size() * sizeof(FftPlan)));
     CMBWS_TRY(g.pair_plan.upload(pplan.data(), pplan.size() * 4));
   }
+  // Tables of the FP64 stage: with the plan where they are small (the call that may not allocate takes only
+  // such grids), so that a first FP64 transform is as fast as the next; building them takes 1.1 ms for
+  // GL L = 1000 (0.25 GB) and 27 ms at Nside 1024 (9.7 GB).
+  if (ringfft_smem_ok(g, CMBWS_FP64) && (noalloc_fp64(g) || fx_offsets(g, nullptr) * 16 <= kFxPlanBytes))
+    CMBWS_TRY(grid_ensure_fx(g, nullptr));
   return CMBWS_OK;
 }
 
@@ -606,8 +616,8 @@ int grid_ensure_ck64(const Grid& gc) {
   CMBWS_LAUNCH_CHECK();
   dim3 grd((g.npair + 127) / 128, L + 1);
   k_start<false><<<grd, 128>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, d_sv.as<double>(),
-                        d_sk.as<int>(), nullptr, nullptr, nullptr, g.ck_base.as<int64_t>(),
-                        nullptr, nullptr, nullptr, cbd.as<int64_t>(), ck.as<float4>(), nullptr);
+                        d_sk.as<int>(), nullptr, nullptr, nullptr, nullptr, nullptr, cbd.as<int64_t>(),
+                        ck.as<float4>());
   CMBWS_LAUNCH_CHECK();
   CMBWS_CUDA(cudaDeviceSynchronize());
   {
@@ -621,6 +631,76 @@ int grid_ensure_ck64(const Grid& gc) {
   g.A2f = std::move(A2);
   g.ck64_base = std::move(cbd);
   g.ck64 = std::move(ck);
+  return CMBWS_OK;
+}
+
+// Set-up work: on the legacy stream, or while the caller's stream is being captured on one of its own (allocations
+// and waits are refused during a capture unless the thread asks for the relaxed mode).  A stream of its
+// own in every case would cost later calls: with a second stream in the process, launches on the legacy one
+// took 1.5 us more each (solve for 8192 unknowns 3.40 -> 3.50 ms).
+namespace {
+struct SetupStream {
+  cudaStream_t s = nullptr;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  bool own = false;
+  int open(cudaStream_t caller) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(caller, &cs) != cudaSuccess) cudaGetLastError();
+    if (cs == cudaStreamCaptureStatusNone) return CMBWS_OK;
+    CMBWS_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    own = true;
+    CMBWS_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    return CMBWS_OK;
+  }
+  ~SetupStream() {
+    if (s) cudaStreamDestroy(s);
+    if (own) cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+};
+}  // namespace
+
+int grid_ensure_fx(const Grid& gc, cudaStream_t caller) {
+  if (gc.fx_ready.load(std::memory_order_acquire)) return CMBWS_OK;
+  std::lock_guard<std::mutex> lk(gc.fx_mu);
+  if (gc.fx_ready.load(std::memory_order_relaxed)) return CMBWS_OK;
+  Grid& g = const_cast<Grid&>(gc);  // tables only; the geometry is not touched
+  const int L = g.lmax;
+  std::vector<int64_t> cb(L + 1, 0);
+  const int64_t tot = fx_offsets(g, cb.data());
+  const size_t nst = (size_t)(L + 1) * g.npair;
+  const int ntile = (g.npair + kTileMinPT - 1) / kTileMinPT;
+  SetupStream w;
+  CMBWS_TRY(w.open(caller));
+  DevMem base, ck, sx, ls, st, tmin;
+  CMBWS_TRY(base.alloc((L + 1) * 8));
+  CMBWS_TRY(ck.alloc((size_t)tot * 16));
+  CMBWS_TRY(sx.alloc(nst));
+  CMBWS_TRY(ls.alloc(nst * 4));
+  CMBWS_TRY(st.alloc(nst * 16));
+  CMBWS_TRY(tmin.alloc((size_t)(L + 1) * ntile * 4));
+  CMBWS_CUDA(cudaMemcpyAsync(base.p, cb.data(), (L + 1) * 8, cudaMemcpyHostToDevice, w.s));
+  const dim3 grd((g.npair + 127) / 128, L + 1), gt((ntile + 127) / 128, L + 1);
+  k_fx_walk<<<grd, 128, 0, w.s>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, g.ls.as<int>(),
+                                  g.st64.as<double2>(), base.as<int64_t>(), ck.as<double2>(),
+                                  sx.as<uint8_t>());
+  CMBWS_LAUNCH_CHECK();
+  k_fx_starts<<<grd, 128, 0, w.s>>>(g.y64.as<double>(), g.A64.as<double>(), L, g.npair, g.ls.as<int>(),
+                                    g.st64.as<double2>(), sx.as<uint8_t>(), ls.as<int>(),
+                                    st.as<ulonglong2>());
+  CMBWS_LAUNCH_CHECK();
+  k_pack_ckx<<<dim3(32, L + 1), 256, 0, w.s>>>(ck.as<ulonglong2>(), base.as<int64_t>(), L, g.npair,
+                                               sx.as<uint8_t>(), ls.as<int>());
+  CMBWS_LAUNCH_CHECK();
+  k_tile_min<<<gt, 128, 0, w.s>>>(ls.as<int>(), g.npair, ntile, tmin.as<int>());
+  CMBWS_LAUNCH_CHECK();
+  CMBWS_CUDA(cudaStreamSynchronize(w.s));
+  g.ckx_base = std::move(base);
+  g.sx = std::move(sx);
+  g.lsx = std::move(ls);
+  g.stx = std::move(st);
+  g.lsx_tmin = std::move(tmin);
+  g.ckx = std::move(ck);
+  g.fx_ready.store(true, std::memory_order_release);
   return CMBWS_OK;
 }
 

@@ -592,7 +592,7 @@ int cmbws_powerlaw_mixing(double nu_ratio, const double* beta, const double* mas
 
 /*
  * Device-side status.  Kernels that wait on an asynchronous event inside the GPU (the
- * tensor-core Legendre synthesis waits on mbarriers for its MMAs) bound every wait; when a
+ * tensor-core Legendre kernels wait on mbarriers for their MMAs) bound every wait; when a
  * wait runs out the kernel stops issuing work, writes NaN into its outputs, records the
  * event in a per-device status word and returns, so the context stays usable.  This call
  * synchronises `stream`, then returns CMBWS_ERR_TIMEOUT if such an event was recorded on the
@@ -604,8 +604,8 @@ int cmbws_device_status(void* stream);
 
 /*
  * Test support for the bounded waits (no counterpart in the paper).  wait_cycles > 0 makes
- * every CTA of the tensor-core Legendre synthesis (CMBWS_TF32, CMBWS_3XTF32) on the current
- * device first wait at most wait_cycles SM clocks on an mbarrier phase that nothing ever
+ * every CTA of the tensor-core Legendre kernels (all precisions but CMBWS_FP32 and CMBWS_FP32X2)
+ * on the current device first wait at most wait_cycles SM clocks on an mbarrier phase that nothing ever
  * completes: the wait runs out, and the CTA takes the failure path described at
  * cmbws_device_status.  0 (the default) switches it off.  Errors: CMBWS_ERR_ARG outside
  * [0, 2^32].

@@ -560,7 +560,7 @@ def cmbws_device_status(stream=None):
 
 
 def cmbws_testing_stall_waits(wait_cycles):
-    """Test support: make the tensor-core synthesis CTAs wait up to wait_cycles SM clocks on an
+    """Test support: make the CTAs of the tensor-core Legendre kernels wait up to wait_cycles SM clocks on an
     mbarrier phase that never completes (0 switches it off)."""
     _check(load_library().cmbws_testing_stall_waits(int(wait_cycles)))
 

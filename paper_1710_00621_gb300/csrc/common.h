@@ -302,6 +302,7 @@ int legendre_synth_fx(const Grid& g, int nmaps, const void* alm, void* F, cudaSt
 // eo: ring parts (double), ee: int [nmaps][L+1] workspace
 int legendre_adjoint_fx(const Grid& g, int nmaps, void* eo, int* ee, double* out, cudaStream_t s);
 int fx_status_take(bool* timed_out);  // as tc_status_take, for these kernels
+int fx_stall_waits(long long cycles);  // their part of cmbws_testing_stall_waits
 // ---- tensor-core Legendre synthesis (legendre_tc.cu), prec TF32 / 3XTF32 / BF16 / BF16X3 ----
 int legendre_synth_tc(const Grid& g, int prec, int nmaps, const void* alm, void* F, cudaStream_t s);
 // adjoint synthesis on the tensor cores from the FP32 adjoint input (eo layout), prec BF16 / BF16X3

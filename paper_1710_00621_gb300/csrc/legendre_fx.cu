@@ -14,6 +14,7 @@
 // 0..7 - i of B accumulate into columns 2 W i.. of the accumulator, so that block s of 2 W columns
 // holds the sum over i + j = s.  Every 64 terms the blocks are read from tensor memory and added
 // as integers.
+#include <atomic>
 #include <climits>
 #include <type_traits>
 
@@ -28,6 +29,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kM = 128;              // MMA rows: ring pairs (synthesis) or values of l (adjoint)
 constexpr int kNT = 2 * kM;          // threads per CTA: two per row
+constexpr int kMaxDevices = 64;
 
 // Column layout for up to NM maps.  Up to 4 maps have an instance each; 5 and 6 maps share one, 7 and 8
 // another.  Eight columns per parity up to 4 maps keep three CTAs on an SM, which the recurrence's
@@ -44,6 +46,11 @@ struct Cols {
 };
 
 __device__ unsigned int g_fx_status = 0;  // bit 0: a bounded mbarrier wait ran out
+// Test support (cmbws_testing_stall_waits), by device: when > 0, every CTA first waits at most this many
+// SM clocks on an mbarrier phase that nothing completes, so the wait runs out.  A kernel argument: reading
+// it from device memory would be on the way of every short launch.
+std::atomic<long long> g_stall[kMaxDevices];
+long long stall_of(const Grid& g) { return g.device < kMaxDevices ? g_stall[g.device].load(std::memory_order_relaxed) : 0; }
 
 // kind::f16, FP16 A and B, FP32 D, M = 128, N = ncol; A K-major or MN-major, B K-major
 __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t adesc, uint64_t bdesc, int ncol, bool mn,
@@ -157,7 +164,8 @@ struct SynLayout {
   static constexpr int kBar = kCorr + 2 * C::W * 16;    // uint64_t[2]
   static constexpr int kMisc = kBar + 16;           // tensor memory base, bad flag
   static constexpr int kExp = kMisc + 16;           // exponents [3][8]
-  static constexpr int kBytes = kExp + 96;
+  static constexpr int kScale = kExp + 96;          // scales of the pairs (uint8)
+  static constexpr int kBytes = kScale + kM;
 };
 
 // Steep spectra.  One scale per (m, map) holds a coefficient to 2^-61 of the largest one that the rings of
@@ -204,7 +212,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
                const ulonglong2* __restrict__ ck, const int64_t* __restrict__ ck_base,
                const int2* __restrict__ pring, const int* __restrict__ ls64, const double2* __restrict__ st64,
                const double* __restrict__ y64, double2* __restrict__ F, int64_t F_stride, int L, int npair,
-               int R, int nmaps) {
+               int R, int nmaps, long long stall) {
   using C = Cols<NM>;
   using LY = SynLayout<C>;
   constexpr int P = 2 * NM, W = C::W;
@@ -228,6 +236,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   if (tid == 0) {
     *s_bad = 0;
     mbar_init(&mbar[0], 1);
+    mbar_init(&mbar[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   // of a group: the first start, and the l from where the Legendre values of the ring nearest the pole are
@@ -248,6 +257,8 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
   // zero B (columns of the other parity and of absent maps stay zero)
   for (int i = tid; i < 2 * C::kBStep / 16; i += kNT)
     reinterpret_cast<uint4*>(sm + LY::kB)[i] = make_uint4(0, 0, 0, 0);
+  if (stall > 0 && tid == 0 && !mbar_wait(&mbar[1], 0, stall)) *s_bad = 1;
+  __syncwarp();
   if (warp == 0) tmem_alloc<C::kTmem>(s_tb);
   tc_fence_before();
   __syncthreads();
@@ -273,6 +284,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     const int ls = valid ? ls_tab[(int64_t)m * npair + p] : INT_MAX;
     const uint64_t x = valid ? xfx[p] : 0;
     const unsigned xh = (unsigned)(x >> 32), xl = (unsigned)x;
+    if (!chain) sm[LY::kScale + row] = valid ? sx[(int64_t)m * npair + p] : 0;
     FxState s0;  // the pair's start values
     if (ls <= L) {
       s0 = fx_unpack(st[(int64_t)m * npair + p]);
@@ -415,7 +427,7 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     if (bad) atomicOr(s_bad, 1);
     __syncthreads();
     const bool failed = *s_bad != 0;
-    const int S = valid ? sx[(int64_t)m * npair + p] : 0;
+    const int S = sm[LY::kScale + row];
     double v[P];
     double* s_odd = reinterpret_cast<double*>(sm + LY::kA);  // [part][row]; all MMAs are done
 #pragma unroll
@@ -473,7 +485,7 @@ int launch_synth_variant(int v, int nm, const Grid& g, const void* alm, int64_t 
                                     g.lsx.as<int>(), g.lsx_tmin.as<int>(), g.stx.as<ulonglong2>(),
                                     g.xfx.as<uint64_t>(), g.ckx.as<ulonglong2>(), g.ckx_base.as<int64_t>(),
                                     g.pair_ring.as<int2>(), g.ls.as<int>(), g.st64.as<double2>(), g.y64.as<double>(),
-                                    (double2*)F, fs, L, g.npair, R, nm);
+                                    (double2*)F, fs, L, g.npair, R, nm, stall_of(g));
   CMBWS_LAUNCH_CHECK();
   return CMBWS_OK;
 }
@@ -576,7 +588,7 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
              const int* __restrict__ ls_tab, const ulonglong2* __restrict__ st, const uint64_t* __restrict__ xfx,
              const ulonglong2* __restrict__ ck, const int64_t* __restrict__ ck_base,
              const int* __restrict__ tmin, const double* __restrict__ c64, double2* __restrict__ out,
-             int64_t nlm, int L, int npair, int nmaps) {
+             int64_t nlm, int L, int npair, int nmaps, long long stall) {
   using C = Cols<NM>;
   using LY = AdjLayout<C>;
   constexpr int W = C::W;
@@ -613,6 +625,7 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
   if (tid == 0) {
     *s_bad = 0;
     mbar_init(&mbar[0], 1);
+    mbar_init(&mbar[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (tid < 4 * W) s_corr[tid] = 0;
@@ -622,6 +635,8 @@ k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const doub
   }
   for (int i = tid; i < 2 * C::kBStep / 16; i += kNT)  // B columns of absent maps stay zero
     reinterpret_cast<uint4*>(sm + LY::kB)[i] = make_uint4(0, 0, 0, 0);
+  if (stall > 0 && tid == 0 && !mbar_wait(&mbar[1], 0, stall)) *s_bad = 1;
+  __syncwarp();
   if (warp == 0) tmem_alloc<C::kTmem>(s_tb);
   tc_fence_before();
   __syncthreads();
@@ -798,7 +813,7 @@ int launch_adj(int nm, const Grid& g, double* eo, int* ee, double* out, cudaStre
   kern<<<grd, kNT, LY::kBytes, s>>>(reinterpret_cast<const fx_t*>(eo), ee, g.A64.as<double>(), g.lsx.as<int>(),
                                     g.stx.as<ulonglong2>(), g.xfx.as<uint64_t>(), g.ckx.as<ulonglong2>(),
                                     g.ckx_base.as<int64_t>(), g.lsx_tmin.as<int>(), g.c64.as<double>(),
-                                    (double2*)out, nlm_of(L), L, g.npair, nm);
+                                    (double2*)out, nlm_of(L), L, g.npair, nm, stall_of(g));
   CMBWS_LAUNCH_CHECK();
   return CMBWS_OK;
 }
@@ -843,6 +858,13 @@ int legendre_adjoint_fx(const Grid& g, int nmaps, void* eo, int* ee, double* out
       default: CMBWS_TRY(launch_adj<8>(nm, g, e, x, o, s)); break;
     }
   }
+  return CMBWS_OK;
+}
+
+int fx_stall_waits(long long cycles) {
+  int dev = 0;
+  CMBWS_CUDA(cudaGetDevice(&dev));
+  if (dev < kMaxDevices) g_stall[dev].store(cycles, std::memory_order_relaxed);
   return CMBWS_OK;
 }
 

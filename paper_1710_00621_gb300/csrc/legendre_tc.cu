@@ -1341,5 +1341,5 @@ extern "C" int cmbws_testing_stall_waits(long long wait_cycles) {
     return CMBWS_ERR_ARG;
   }
   CMBWS_CUDA(cudaMemcpyToSymbol(g_tc_stall_cycles, &wait_cycles, sizeof(wait_cycles)));
-  return CMBWS_OK;
+  return fx_stall_waits(wait_cycles);
 }

@@ -367,15 +367,17 @@ int cmbws_project(cmbws_model m, const double* x, double* const* d, void* stream
  *   mode 2: on the first synthesis for a (grid, precision, maps) key, each tile variant is
  *     launched and timed with CUDA events on the caller's stream (the first call is then
  *     synchronous), and the fastest is kept for that key for the life of the grid.
- * FP64 tiles are groups of 128 ring pairs per CTA; its results do not depend on them.  FP32 results can differ in rounding (warps that
- * hold a ring pair near a pole switch to the difference form of the recurrence, and the
- * tile decides which pairs share a warp).  Errors: CMBWS_ERR_ARG for another mode.
+ * FP64 tiles are 2, 1, 8 or 4 groups of 128 ring pairs per CTA (default and heuristic: 1), and
+ * its results do not depend on them.  FP32 results can differ in rounding (warps that hold a
+ * ring pair near a pole switch to the difference form of the recurrence, and the tile decides
+ * which pairs share a warp).  Errors: CMBWS_ERR_ARG for another mode.
  */
 int cmbws_set_autotune(int mode);
 
 /* The tuner's decision for synthesis on grid g at precision prec with nmaps maps per
- * launch (1..4): variant index (-1 if none was measured), nvar variants, and their times in
- * ms (ms: array of at least 8 floats, or NULL). */
+ * launch (1..4; at CMBWS_FP64 1..8, where 5 and 6 maps share a decision, and 7 and 8): variant
+ * index (-1 if none was measured), nvar variants, and their times in ms (ms: array of at
+ * least 8 floats, or NULL). */
 int cmbws_grid_tuning(cmbws_grid g, int prec, int nmaps, int* variant, float* ms, int* nvar);
 
 /*

@@ -378,6 +378,7 @@ CMBWS_TUNE_DEFAULT = 0
 CMBWS_TUNE_HEURISTIC = 1
 CMBWS_TUNE_MEASURED = 2
 SYNTH_TILES = [(2, 128), (1, 128), (1, 64), (4, 64)]   # (ring pairs per thread, threads per CTA)
+FP64_TILES = [(2, 128), (1, 128), (8, 128), (4, 128)]  # FP64: (groups per CTA, ring pairs per group)
 
 
 def cmbws_set_autotune(mode):
@@ -394,7 +395,8 @@ def cmbws_grid_tuning(grid, prec, nmaps):
                                             ms, ctypes.byref(n)))
     if v.value < 0:
         return None
-    return {"variant": v.value, "tile": SYNTH_TILES[v.value], "ms": [ms[i] for i in range(n.value)]}
+    tiles = FP64_TILES if int(prec) == CMBWS_FP64 else SYNTH_TILES
+    return {"variant": v.value, "tile": tiles[v.value], "ms": [ms[i] for i in range(n.value)]}
 
 
 def cmbws_model_set_graphs(model, on):

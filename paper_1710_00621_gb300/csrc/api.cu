@@ -237,7 +237,7 @@ extern "C" int cmbws_grid_tuning(cmbws_grid gh, int prec, int nmaps, int* varian
     return CMBWS_ERR_ARG;
   }
   std::lock_guard<std::mutex> lk(g->tune_mu);
-  auto it = g->tuned.find(synth_tune_key(prec, nmaps < 4 ? nmaps : 4));
+  auto it = g->tuned.find(synth_tune_key(prec, synth_instance(prec, nmaps)));
   if (it == g->tuned.end()) {
     *variant = -1;
     *nvar = 0;

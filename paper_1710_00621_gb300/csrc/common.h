@@ -325,6 +325,11 @@ bool prof_enabled();  // per-stage CUDA-event profiling switched on (cmbws_profi
 // being captured, and records the result in g.tuned[key].
 int autotune_mode();
 inline int synth_tune_key(int prec, int nmaps) { return 1000 + 10 * prec + nmaps; }
+// maps of the kernel instance that runs a launch of nmaps: up to 4, each of its own; FP64 also has one for
+// 5 and 6 maps and one for 7 and 8
+inline int synth_instance(int prec, int nmaps) {
+  return nmaps <= 4 || prec != CMBWS_FP64 ? (nmaps < 4 ? nmaps : 4) : nmaps <= 6 ? 6 : kFxMaps;
+}
 int autotune_pick(const Grid& g, int key, int nvar, int heuristic,
                   const std::function<int(int)>& launch, cudaStream_t s, int* chosen);
 

@@ -470,12 +470,14 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
 }
 
 // Tiles: groups of 128 ring pairs per CTA, taken one after the other (the autotuner's list of the
-// synthesis; without it one group per CTA).
+// synthesis; without it one group per CTA, variant 1).
+constexpr int kFxTiles = 4;
 template <int NM>
 int launch_synth_variant(int v, int nm, const Grid& g, const void* alm, int64_t as, void* F, int64_t fs,
                          cudaStream_t s) {
   using LY = SynLayout<Cols<NM>>;
-  const int R = v == 0 ? 2 : v == 3 ? 4 : 1;
+  constexpr int kR[kFxTiles] = {2, 1, 8, 4};
+  const int R = kR[v];
   const int L = g.lmax;
   dim3 grd((g.npair + kM * R - 1) / (kM * R), L + 1);
   auto kern = k_leg_synth_fx<NM>;
@@ -495,7 +497,7 @@ int launch_synth(int nm, const Grid& g, const void* alm, int64_t as, void* F, in
   int v = 1;
   if (autotune_mode() != 0)
     CMBWS_TRY(autotune_pick(
-        g, synth_tune_key(CMBWS_FP64, nm < 4 ? nm : 4), 4, 1,
+        g, synth_tune_key(CMBWS_FP64, NM), kFxTiles, 1,
         [&](int vv) { return launch_synth_variant<NM>(vv, nm, g, alm, as, F, fs, s); }, s, &v));
   return launch_synth_variant<NM>(v, nm, g, alm, as, F, fs, s);
 }

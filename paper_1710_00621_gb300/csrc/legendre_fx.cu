@@ -171,10 +171,11 @@ struct SynLayout {
 // Steep spectra.  One scale per (m, map) holds a coefficient to 2^-61 of the largest one that the rings of
 // the CTA can see, where FP64 arithmetic holds it to 2^-53 of itself.  That is enough for a ring's map if
 // the largest one is below 2^8 of what lights the ring anyway: its coefficients of m = 0, whose Legendre
-// values are of order one at every l and ring (the first 256 stand for them), or those of this m from
-// where the ring's values are of order one (l sin(theta) = m; for the CTA's ring nearest the pole).  Only
-// spectra without much at m = 0 that fall by more than 2^8 along this m fail both; their sums are taken in
-// FP64 arithmetic instead (from the start at 1e-30), by two threads per ring pair, one for each parity.
+// values are of order one at every l and ring (the first 128 and 128 from the whole range stand for them),
+// or those of this m from where the ring's values are of order one (l sin(theta) = m; for the CTA's ring
+// nearest the pole).  Only spectra without much at m = 0 that fall by more than 2^8 along this m fail
+// both; their sums are taken in FP64 arithmetic instead (from the start at 1e-30), by two threads per ring
+// pair, one for each parity.
 constexpr int kSteep = 8;
 // Sum over l of mu_l a_l with l - m of parity par; a, A at index l; ls, st: the pair's start.
 __device__ __noinline__ double2 synth_fp64(const double2* a, const double* A, double y, int ls, double2 st,
@@ -200,10 +201,11 @@ __device__ __noinline__ double2 synth_fp64(const double2* a, const double* A, do
 // digit tile (consecutive threads are 16 bytes apart); every second stage it converts one
 // coefficient part to digits of B.  One thread issues the stage's MMAs after its barrier; they read
 // the tile while the threads compute the next values in registers.
-// Bound by the dispatch of integer instructions (48 per element, 26 of them at half rate; tensor pipe
-// 15 %).  Against the recurrence and sums on the FP64 pipe, Nside 1024, L = 3071, 3 maps: 94.6 ->
-// 19.1 ms.  One chain per row and 128 threads was 19.0 ms against 19.9 for two chains when both were
-// tried there, but grids of few ring pairs wait for that chain.
+// Bound by the dispatch of integer instructions (50 per element, about half of them at half rate; tensor
+// pipe 15 %).  Against the recurrence and sums on the FP64 pipe, Nside 1024, L = 3071, 3 maps: 94.6 ->
+// 19.9 ms (19.1 with 7 digits and one scale per m, which lost precision: fixed.h).  An early form with one
+// chain per row and 128 threads took 19.0 ms there where two chains took 19.9 (not tried since), but
+// grids of few ring pairs wait for that chain.
 template <int NM>
 __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double* __restrict__ Acoef,
@@ -292,8 +294,8 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     }
     if (tid < 4 * W) s_corr[tid] = 0;
     const int wlo = __reduce_min_sync(kFull, ls);
+    if (r > 0) group_range(r);
     const int lo = lo_r, hi = hi_r;
-    if (r + 1 < R) group_range(r + 1);
     // scale of each map: the largest exponent among this m's coefficients from lo on (any that is not
     // finite counts)
     if (r > 0) {
@@ -304,7 +306,10 @@ k_leg_synth_fx(const double2* __restrict__ alm, int64_t alm_stride, const double
     for (int k = 0; k < NM; ++k) {
       if (k >= nm) break;
       unsigned e = 0, eh = 0, e0 = 0;
-      if (r == 0 && tid <= L) e0 = exp2(alm[k * alm_stride + tid]);
+      if (r == 0) {
+        const int l = chain ? row * ((L + kM) / kM) : row;
+        if (l <= L) e0 = exp2(alm[k * alm_stride + l]);
+      }
 #pragma unroll 4
       for (int l = m + tid; l <= L; l += kNT) {
         const unsigned x = exp2(alm[k * alm_stride + lmo + l]);
@@ -582,8 +587,10 @@ k_eo_fix(double* __restrict__ eo, int npair, int L, const uint8_t* __restrict__ 
 // chunk of 16 values of l, which each thread walks from the chunk's checkpoint; rows of A are
 // values of l (MN-major: a thread writes 8 consecutive values of its pair as one 16-byte row).
 // Every output has one owner; stages without a started pair are skipped.
-// Bound as the synthesis is (tensor pipe 17 %).  Against the FP64 pipe, Nside 1024, 3 maps: 107.9 ->
-// 18.1 ms; GL L = 1000, 1 map: 1.77 -> 0.60 ms.
+// One buffer of B, filled once the previous stage's MMAs are done: a second one would leave room for two
+// CTAs per SM only.  Bound as the synthesis is (tensor pipe 17 %).  Against the FP64 pipe, Nside 1024, 3
+// maps: 107.9 -> 19.5 ms with k_eo_fix (18.1 with 7 digits and two buffers); GL L = 1000, 1 map: 1.77 ->
+// 0.64 ms.
 template <int NM>
 __global__ void __launch_bounds__(kNT, Cols<NM>::kCtas)
 k_leg_adj_fx(const fx_t* __restrict__ eo, const int* __restrict__ ee, const double* __restrict__ Acoef,

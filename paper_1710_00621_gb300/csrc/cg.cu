@@ -2,14 +2,14 @@
 //
 // Vectors are FP64 on the device.  Dot products are deterministic: every block of a grid of up to
 // 1024 writes its partial sum, and the block that ends last adds them in a fixed order.
-// The host reads one or two scalars per iteration (alpha and beta are
-// computed on the host in FP64).
+// alpha and beta are formed on the device; the host reads the scalars once
+// per iteration for the stopping test.
 //
 // FP64 models: plain PCG, then one FP64-accurate apply certifies ||b - A x|| / ||b||.
 // FP32 models: iterative refinement.  Each pass solves A d = r by PCG with
 // the FP32 transform chain (FP64 vectors and scalars) until the inner
 // residual falls by inner_tol, then x += d and r = b - A x with an
-// FP64-accurate chain (native FP64 or double-float, opts.cert_prec); the loop
+// FP64-accurate chain (FP64 or double-float, opts.cert_prec); the loop
 // ends when that residual certifies tol.
 #include <algorithm>
 #include <atomic>

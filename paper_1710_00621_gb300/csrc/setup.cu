@@ -23,7 +23,8 @@
 // The same FP64 pass stores, for the FP32 adjoint, the two recurrence values at the
 // start of every chunk of kChunk = 8 values of l ([m][pair][chunk], FP32; about
 // npair (L+1)^2 / 16 x 8 bytes: 9.7 GB at Nside 1024, L = 3071), so that the adjoint can
-// restart the recurrence of any pair at any chunk without a serial walk along l.
+// restart the recurrence of any pair at any chunk without a serial walk along l.  The tables of the FP64
+// (fixed.h) and double-float stages are made from these starts when first needed.
 #include <algorithm>
 #include <climits>
 #include <cmath>

@@ -50,7 +50,9 @@ __device__ unsigned int g_fx_status = 0;  // bit 0: a bounded mbarrier wait ran 
 // SM clocks on an mbarrier phase that nothing completes, so the wait runs out.  A kernel argument: reading
 // it from device memory would be on the way of every short launch.
 std::atomic<long long> g_stall[kMaxDevices];
-long long stall_of(const Grid& g) { return g.device < kMaxDevices ? g_stall[g.device].load(std::memory_order_relaxed) : 0; }
+long long stall_of(const Grid& g) {
+  return g.device < kMaxDevices ? g_stall[g.device].load(std::memory_order_relaxed) : 0;
+}
 
 // kind::f16, FP16 A and B, FP32 D, M = 128, N = ncol; A K-major or MN-major, B K-major
 __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t adesc, uint64_t bdesc, int ncol, bool mn,
